@@ -10,7 +10,7 @@ template <int Q>
 cudaError_t launch(const Params& P, const void* w_in, const void* w_out, int sms, cudaStream_t stream) {
   const void* k = reinterpret_cast<const void*>(k_block_fast<Q>);
   int occ = 0;
-  cudaError_t e = fast::occupancy_cached(k, SMEM_BYTES, &occ);
+  cudaError_t e = fast::occupancy_cached(k, THREADS, SMEM_BYTES, &occ);
   if (e != cudaSuccess) return e;
   if (occ != 1) return cudaErrorInvalidConfiguration;  // all 512 TMEM columns per CTA: one CTA per SM
   Params p = P;

@@ -10,13 +10,14 @@
 
 #include "whtmix_fast.cuh"
 #include "whtmix_fast_bwd.cuh"
+#include "whtmix_tri.cuh"
 
 namespace whtmix {
 namespace fast {
 
 // Resident CTAs per SM for one kernel and smem size, per device (first query also raises the
 // kernel's dynamic shared memory limit).
-inline cudaError_t occupancy_cached(const void* kernel, size_t smem, int* occ) {
+inline cudaError_t occupancy_cached(const void* kernel, int threads, size_t smem, int* occ) {
   static std::mutex mu;
   static std::map<std::pair<int, const void*>, int> cache;
   int dev = 0;
@@ -30,7 +31,7 @@ inline cudaError_t occupancy_cached(const void* kernel, size_t smem, int* occ) {
   }
   e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kernel, THREADS, smem);
+  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(occ, kernel, threads, smem);
   if (e != cudaSuccess) return e;
   if (*occ < 1) return cudaErrorInvalidConfiguration;
   cache[{dev, kernel}] = *occ;
@@ -42,15 +43,15 @@ inline cudaError_t occupancy_cached(const void* kernel, size_t smem, int* occ) {
 // tcgen05.alloc while the first waits for it at the device-wide barrier.  The grid is one CTA per
 // SM, all resident at once; it is launched with programmatic stream serialisation (launch_pdl),
 // which lets its launch and tensor-memory allocation overlap the previous kernel's tail.
-inline cudaError_t launch_persistent(const void* k, const Params& P, int sms, cudaStream_t stream) {
-  const size_t smem = SMEM_BYTES;
+inline cudaError_t launch_persistent(const void* k, const Params& P, int sms, cudaStream_t stream, int threads = THREADS,
+                                     size_t smem = SMEM_BYTES) {
   int occ = 0;
-  cudaError_t e = occupancy_cached(k, smem, &occ);
+  cudaError_t e = occupancy_cached(k, threads, smem, &occ);
   if (e != cudaSuccess) return e;
   if (occ != 1) return cudaErrorInvalidConfiguration;
   Params p = P;
   void* args[] = {&p};
-  return launch_pdl(k, static_cast<unsigned>(sms), THREADS, smem, stream, args);
+  return launch_pdl(k, static_cast<unsigned>(sms), threads, smem, stream, args);
 }
 template <int D, int R, int Q, bool SEP, class WS = WsF32>
 cudaError_t launch_one(const Params& P, int sms, cudaStream_t stream) {
@@ -61,6 +62,8 @@ cudaError_t launch_bwd_one(const Params& P, int sms, cudaStream_t stream) {
   return launch_persistent(reinterpret_cast<const void*>(k_backward_fast<D, R, Q>), P, sms, stream);
 }
 
+// The older three-phase kernel, for the 2^21-element planes and the bf16 exchange (WS = WsB16,
+// whtmix_forward_x16).
 // Rows of 2^13 elements at every size but 2^21; 2^23-element planes take 1024-row columns (two
 // lanes per column).  With 152 SMs, 1024 rows of 2^13 spread as 7 or 6 per CTA, where 512 rows of
 // 2^14 give 56 CTAs four rows against three; measured on the 2^22 planes, 2^13 rows with 512-row
@@ -69,6 +72,30 @@ cudaError_t launch_bwd_one(const Params& P, int sms, cudaStream_t stream) {
 // planes (bf16), 138 us against 146 us per call.
 // SEP: separable log gains (P.gt, P.gc) instead of G; needs 1 <= P.cbits <= row bits.
 // WS: the workspace element (WsB16: whtmix_forward_x16).
+// The three-phase forward: rows of 2^13 at every size but 2^21, whose rows of 2^14 and 128-row columns stay with
+// the older kernel: next to the backward of a training step it measured no faster ([16, 8192, 256] bf16, forward
+// and backward: 465 us against 470).
+template <int D, int Q, bool SEP>
+cudaError_t launch_tri(const Params& P, int sms, cudaStream_t stream) {
+  return launch_persistent(reinterpret_cast<const void*>(tri::k_forward_fast<D, Q, SEP>), P, sms, stream, tri::THREADS,
+                           tri::smem_bytes<D>());
+}
+template <int D, bool SEP>
+cudaError_t launch_forward_tri(const Params& P, int sms, cudaStream_t stream) {
+  switch (P.m) {
+    case 14: return launch_tri<D, 1, SEP>(P, sms, stream);
+    case 15: return launch_tri<D, 2, SEP>(P, sms, stream);
+    case 16: return launch_tri<D, 3, SEP>(P, sms, stream);
+    case 17: return launch_tri<D, 4, SEP>(P, sms, stream);
+    case 18: return launch_tri<D, 5, SEP>(P, sms, stream);
+    case 19: return launch_tri<D, 6, SEP>(P, sms, stream);
+    case 20: return launch_tri<D, 7, SEP>(P, sms, stream);
+    case 21: return launch_one<D, 14, 7, SEP>(P, sms, stream);
+    case 22: return launch_tri<D, 9, SEP>(P, sms, stream);
+    case 23: return launch_tri<D, 10, SEP>(P, sms, stream);
+    default: return cudaErrorInvalidValue;
+  }
+}
 template <int D, bool SEP, class WS = WsF32>
 cudaError_t launch_forward(const Params& P, int sms, cudaStream_t stream) {
   switch (P.m) {

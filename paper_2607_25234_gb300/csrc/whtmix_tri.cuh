@@ -1,0 +1,875 @@
+// whtmix_tri.cuh -- three-phase forward for fp32 / bf16 planes, every workspace and input access staged
+// asynchronously through shared memory (Section III-B map; see whtmix_kernels.cuh for the flattening).
+//
+// A plane of 2^m elements is 2^Q rows of 2^13 contiguous elements (m = 13 + Q), transformed as
+//   phase 1  every row: its 13 bits                                     X  -> workspace (fp32)
+//   phase 2  every column: its Q bits, gain G/L, the Q bits again       workspace -> workspace
+//   phase 3  every row: its 13 bits again                               workspace -> Y
+// with the bounded device-wide barrier between phases.  The workspace is in natural order.
+//
+// One CTA of 16 warps per SM, 64 elements a thread (128 registers).  A worker of 128 threads holds a row,
+// a team of two workers 2^(14-Q) adjacent columns; a ring of shared-memory slots keeps the next tiles in
+// flight, so that loads, butterflies and stores of different tiles overlap.
+//   rows of bf16 X  the 7 low bits on the tensor cores: D[i, n] = sum_k H_128[i, k] x[128 n + k] (M = 128,
+//            N = 64, K = 128; bf16 times +-1 is exact, fp32 accumulation), then lane i of the worker reads its
+//            64 values n from tensor memory and runs the other 6 bits in registers: no exchange at all;
+//   other rows  two register rounds with one exchange inside the slot: A on bits {0, 1, 9..12} (16-byte
+//            vectors), B on bits {3..8} and, by one shuffle stage, bit 2;
+//   columns  rounds of five bits each, in place in the slot.
+// Slots are XOR-swizzled so that every access is conflict-free.
+//
+// What bounds it: the fp32 workspace crosses between SMs through L2 twice (32 MiB each way at 2^23 elements;
+// measured without arithmetic: 4.4 us to write it, 5.9 to read and write it by columns, 1.8 to read it back,
+// 1.4 per barrier), and within an SM the shared-memory data path (one 128-byte wavefront a cycle) more than the
+// additions.  Measured against the previous kernel (8 warps, 128 elements a thread, columns read straight from
+// L2): [32, 4096, 64] f32 40.6 -> 32.9 us, [1, 4096, 64] bf16 11.6 -> 9.7, [1, 65536, 128] bf16 41.9 -> 39.7, with
+// log gains 39.2 -> 37.9, [1, 32768, 128] bf16 28.4 -> 27.1, [8, 4096, 256] f32 42.6 -> 36.3; of that the tensor-core
+// rows took phase 1 of the 2^23-element plane from 13.5 to 8.7 us.
+#pragma once
+
+#include "whtmix_fast.cuh"
+#include "whtmix_tc.cuh"
+
+namespace whtmix {
+namespace tri {
+
+using fast::add2;
+using fast::bf2;
+using fast::bf_in;
+using fast::mul2;
+
+constexpr int THREADS = 512;
+constexpr int WORKERS = 4;
+constexpr int WT = 128;              // threads per worker
+constexpr int R = 13;                // row bits
+constexpr int TILE = 1 << R;         // elements per row
+constexpr int SLOTS = 6;             // ring of rows; the column ring is three pairs of slots
+constexpr int PAIRS = SLOTS / 2;
+constexpr int XSLOTS = 3;            // bf16 X rows (16 KiB) staged per worker
+constexpr int H_BYTES = 128 * 128 * 2;  // H_128 in bf16, the tensor cores' A operand
+constexpr int SLOT_BYTES = SLOTS * TILE * 4;
+static_assert(WORKERS * XSLOTS * TILE * 2 <= SLOT_BYTES, "the X staging areas share the slots");
+// more than half an SM: one CTA per SM (both for the barriers and for tensor memory)
+template <int D>
+constexpr size_t smem_bytes() { return SLOT_BYTES + (D == DT_BF16 ? H_BYTES : 0); }
+
+// Mbarriers of the rings: two per slot, taken in turn, so that all uses of one barrier belong to one
+// worker or team (12 is a multiple of four workers, 6 of two teams) and no wait can start two phases ahead.
+constexpr int ROW_BARS = 2 * SLOTS;
+constexpr int PAIR_BARS = 2 * PAIRS;
+
+__device__ __forceinline__ void worker_sync(int worker) {
+  asm volatile("bar.sync %0, %1;" ::"r"(worker + 1), "r"(WT) : "memory");
+}
+__device__ __forceinline__ void team_sync(int team) {
+  asm volatile("bar.sync %0, %1;" ::"r"(team + 5), "r"(2 * WT) : "memory");
+}
+__device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async16z(uint32_t dst, const void* src, bool valid) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(valid ? 16 : 0) : "memory");
+}
+// this thread arrives on `full` once its earlier cp.async copies have landed
+__device__ __forceinline__ void cp_async_arrive(uint64_t* full) {
+  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(tc::smem_u32(full)) : "memory");
+}
+// Bounded wait for phase `parity` of an mbarrier.  A wait that gives up sets the workspace's error word
+// and `dead`, which ends every later wait at once; the kernel then runs to its end on whatever the buffers
+// hold.
+__device__ __forceinline__ void wait_bar(uint64_t* bar, uint32_t parity, GridBarrier* gb, volatile int* dead) {
+  const uint32_t a = tc::smem_u32(bar);
+  unsigned long long t0 = 0;
+  for (unsigned polls = 0;; ++polls) {
+    uint32_t done;
+    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                 : "=r"(done) : "r"(a), "r"(parity) : "memory");
+    if (done) return;
+    if ((polls & 63u) == 63u) {
+      if (*dead) return;
+      const unsigned long long now = global_ns();
+      if (t0 == 0) t0 = now;
+      if (now - t0 > BARRIER_TIMEOUT_NS) {
+        atomicOr(&gb->err, 1u);
+        *dead = 1;
+        return;
+      }
+    }
+  }
+}
+// use `seq` of a ring of `bars` barriers
+__device__ __forceinline__ void wait_full(uint64_t* full, unsigned seq, unsigned bars, GridBarrier* gb, volatile int* dead) {
+  wait_bar(full + seq % bars, (seq / bars) & 1u, gb, dead);
+}
+// Share of CTA blockIdx.x of `units` units (units < 2^22: the product fits 32 bits)
+__device__ __forceinline__ void share(unsigned units, int* begin, int* end) {
+  *begin = static_cast<int>(units * blockIdx.x / gridDim.x);
+  *end = static_cast<int>(units * (blockIdx.x + 1) / gridDim.x);
+}
+
+// Butterflies over bits [B0, 5) of the index of v[32] (packed pairs).
+template <int B0>
+__device__ __forceinline__ void bfly32(float2 (&v)[32]) {
+#pragma unroll
+  for (int b = B0 < 0 ? 0 : B0; b < 5; ++b)
+#pragma unroll
+    for (int i = 0; i < 32; ++i)
+      if ((i & (1 << b)) == 0) bf2(v[i], v[i + (1 << b)]);
+}
+
+// ---------------------------------------------------------------------------------------------
+// Rows of bf16 X on the tensor cores.  Both operands are K-major in 128-byte-swizzled panels of 64 k
+// (16-byte chunk j of row r at chunk j ^ (r mod 8)).
+//
+// H_128 (A: 128 rows, two panels of 16 KiB): entry (i, k) = (-1)^popcount(i & k).
+__device__ __forceinline__ void build_h(unsigned char* sh) {
+  for (int q = threadIdx.x; q < 128 * 16; q += THREADS) {
+    const int i = q >> 4, c = q & 15;  // k = 8 c ..
+    const uint32_t flip = (__popc(i & (8 * c)) & 1) ? 0x80008000u : 0u;
+    uint32_t w[4];
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      const uint32_t lo = (__popc(i & (2 * p)) & 1) ? 0xBF80u : 0x3F80u;
+      const uint32_t hi = (__popc(i & (2 * p + 1)) & 1) ? 0xBF80u : 0x3F80u;
+      w[p] = (lo | (hi << 16)) ^ flip;
+    }
+    *reinterpret_cast<uint4*>(sh + (c >> 3) * 16384 + i * 128 + (((c & 7) ^ (i & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+// X row (64 tile rows n of 128 contiguous elements, B: two panels of 8 KiB) by the worker's cp.async; elements
+// at offsets >= lim are zero.
+__device__ __forceinline__ void load_x_bf16(const unsigned short* src, int lim, uint32_t dst, int t) {
+  const int n = t >> 4, c = t & 15;
+  const uint32_t d = dst + (c >> 3) * 8192 + n * 128 + (((c & 7) ^ (n & 7)) << 4);
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int o = 8 * t + 1024 * i;
+    cp_async16z(d + 1024 * i, src + (o < lim ? o : 0), o < lim);
+  }
+}
+// D (TMEM columns d .. d + 63) = H_128 x row, one thread
+__device__ __forceinline__ void mma_row(uint32_t d, uint32_t h, uint32_t x) {
+#pragma unroll
+  for (int k = 0; k < 8; ++k)
+    tc::mma_bf16(d, tc::sw128_desc(h + (k >> 2) * 16384 + (k & 3) * 32), tc::sw128_desc(x + (k >> 2) * 8192 + (k & 3) * 32),
+                 tc::instr_desc(128, 64), k > 0);
+}
+// this thread's lane of D: element r = t + 128 n, pairs (n, n + 1)
+__device__ __forceinline__ void read_row(uint32_t ta, float2 (&v)[32]) {
+  float f[64];
+#pragma unroll
+  for (int c = 0; c < 64; c += 16) fast::tmem_ld16(ta + c, *reinterpret_cast<float(*)[16]>(f + c));
+  fast::tmem_wait_ld();
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = make_float2(f[2 * i], f[2 * i + 1]);
+}
+
+// ---------------------------------------------------------------------------------------------
+// Rows in registers.  Round A: thread t holds the quads (r0, r1) at 4 t + 512 v, v = 0..15 (r9..r12); round B:
+// lane l holds r0, r1, r2 = l mod 8, r9, r10 = l / 8, warp r11, r12, registers r3..r8 as pairs (s, s + 32).  In
+// the slot, word bits 3, 4 are XORed with r9, r10.
+__device__ __forceinline__ int quad_word(int t, int v) { return ((4 * t) ^ ((v & 3) << 3)) + 512 * v; }
+__device__ __forceinline__ void round_a(float2 (&a)[16][2]) {
+#pragma unroll
+  for (int v = 0; v < 16; ++v) {
+    bf_in(a[v][0]);
+    bf_in(a[v][1]);
+    bf2(a[v][0], a[v][1]);
+  }
+#pragma unroll
+  for (int h = 1; h < 16; h <<= 1)
+#pragma unroll
+    for (int v = 0; v < 16; ++v)
+      if ((v & h) == 0) {
+        bf2(a[v][0], a[v + h][0]);
+        bf2(a[v][1], a[v + h][1]);
+      }
+}
+__device__ __forceinline__ void round_b(float2 (&b)[32]) {
+#pragma unroll
+  for (int s = 0; s < 32; ++s) bf_in(b[s]);
+  bfly32<0>(b);
+  // r2 across lanes l, l ^ 4
+  const float2 sgn = (threadIdx.x & 4) ? make_float2(-1.f, -1.f) : make_float2(1.f, 1.f);
+#pragma unroll
+  for (int s = 0; s < 32; ++s) {
+    const float2 p = make_float2(__shfl_xor_sync(0xffffffffu, b[s].x, 4), __shfl_xor_sync(0xffffffffu, b[s].y, 4));
+    b[s] = fast::fma2(b[s], sgn, p);
+  }
+}
+// Slot word of round B's element s.
+struct RowB {
+  int q[4];
+  __device__ __forceinline__ RowB(int t) {
+    const int l = t & 31, h = l >> 3, w = t >> 5;
+    const int base = (l & 7) + 512 * (h + 4 * w);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) q[k] = base + 8 * (k ^ h);
+  }
+  __device__ __forceinline__ int word(int s) const { return q[s & 3] + 32 * (s >> 2); }
+};
+// A row of fp32 (lim elements present, the rest zero) into a slot, by one worker.
+__device__ __forceinline__ void load_row(const float* src, int lim, float* slot, int t, uint64_t* full) {
+  const uint32_t d = tc::smem_u32(slot);
+#pragma unroll
+  for (int v = 0; v < 16; ++v) {
+    const int o = 4 * t + 512 * v;
+    cp_async16z(d + 4 * quad_word(t, v), src + (o < lim ? o : 0), o < lim);
+  }
+  cp_async_arrive(full);
+}
+
+// Phase 1, fp32: the row in `slot` -> workspace row.  `done` is called once the slot is free.
+template <class Done>
+__device__ __forceinline__ void row_in(float* slot, float* ws_row, int t, int worker, const Done& done) {
+  {
+    float2 a[16][2];
+#pragma unroll
+    for (int v = 0; v < 16; ++v) {
+      const float4 q = *reinterpret_cast<const float4*>(slot + quad_word(t, v));
+      a[v][0] = make_float2(q.x, q.y);
+      a[v][1] = make_float2(q.z, q.w);
+    }
+    round_a(a);
+#pragma unroll
+    for (int v = 0; v < 16; ++v)
+      *reinterpret_cast<float4*>(slot + quad_word(t, v)) = make_float4(a[v][0].x, a[v][0].y, a[v][1].x, a[v][1].y);
+  }
+  worker_sync(worker);
+  const RowB rb(t);
+  float2 b[32];
+#pragma unroll
+  for (int s = 0; s < 32; ++s) b[s] = make_float2(slot[rb.word(s)], slot[rb.word(s + 32)]);
+  worker_sync(worker);
+  done();
+  round_b(b);
+  float* dst = ws_row + (t & 7) + 512 * (t >> 3);
+#pragma unroll
+  for (int s = 0; s < 32; ++s) {
+    __stcg(dst + 8 * s, b[s].x);
+    __stcg(dst + 8 * (s + 32), b[s].y);
+  }
+}
+
+// Phase 3: the workspace row in `slot` -> the first lim elements of Y's row at dst + e0.
+template <int D, class Done>
+__device__ __forceinline__ void row_out(float* slot, void* dst, long long e0, int lim, int t, int worker, const Done& done) {
+  {
+    const RowB rb(t);
+    float2 b[32];
+#pragma unroll
+    for (int s = 0; s < 32; ++s) b[s] = make_float2(slot[rb.word(s)], slot[rb.word(s + 32)]);
+    round_b(b);
+#pragma unroll
+    for (int s = 0; s < 32; ++s) {
+      slot[rb.word(s)] = b[s].x;
+      slot[rb.word(s + 32)] = b[s].y;
+    }
+  }
+  worker_sync(worker);
+  float2 a[16][2];
+#pragma unroll
+  for (int v = 0; v < 16; ++v) {
+    const float4 q = *reinterpret_cast<const float4*>(slot + quad_word(t, v));
+    a[v][0] = make_float2(q.x, q.y);
+    a[v][1] = make_float2(q.z, q.w);
+  }
+  worker_sync(worker);
+  done();
+  round_a(a);
+#pragma unroll
+  for (int v = 0; v < 16; ++v) {
+    const int o = 4 * t + 512 * v;
+    if (o < lim) {
+      if constexpr (D == DT_BF16) {
+        const __nv_bfloat162 h0 = __floats2bfloat162_rn(a[v][0].x, a[v][0].y), h1 = __floats2bfloat162_rn(a[v][1].x, a[v][1].y);
+        __stcs(reinterpret_cast<uint2*>(static_cast<unsigned short*>(dst) + e0 + o),
+               make_uint2(*reinterpret_cast<const uint32_t*>(&h0), *reinterpret_cast<const uint32_t*>(&h1)));
+      } else {
+        __stcs(reinterpret_cast<float4*>(static_cast<float*>(dst) + e0 + o),
+               make_float4(a[v][0].x, a[v][0].y, a[v][1].x, a[v][1].y));
+      }
+    }
+  }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Columns, Q <= 9: a warp lane is a column (a warp reads and writes 128-byte row segments) and a column's
+// rows meet in that lane's tensor memory, so nothing goes through shared memory.
+// Gains of one column: row(j), and rows2(j) = rows j and j + 1 (j even).
+template <int Q>
+struct LaneFull {
+  const float* p;
+  __device__ __forceinline__ LaneFull(const Params& P, const float*, int col) : p(static_cast<const float*>(P.g) + col) {}
+  __device__ __forceinline__ float2 rows2(int j) const { return make_float2(__ldg(p + (j << R)), __ldg(p + ((j + 1) << R))); }
+  __device__ __forceinline__ float row(int j) const { return __ldg(p + (j << R)); }
+};
+// Separable log gains: G[n, c] = et[n] ec[c] from two tables that phase 1 builds (tab); the token table is
+// stored so that a column's rows are consecutive, et[(column >> cb) 2^Q + row].
+template <int Q>
+struct LaneSep {
+  const float* p;
+  float e;
+  __device__ __forceinline__ LaneSep(const Params& P, const float* tab, int col)
+      : p(tab + (static_cast<long long>(col >> P.cbits) << Q)), e(tab[(1ll << (P.m - P.cbits)) + (col & ((1 << P.cbits) - 1))]) {}
+  __device__ __forceinline__ float2 rows2(int j) const { return mul2(*reinterpret_cast<const float2*>(p + j), make_float2(e, e)); }
+  __device__ __forceinline__ float row(int j) const { return p[j] * e; }
+};
+
+__device__ __forceinline__ void tmem_ld8(uint32_t ta, float (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]), "=f"(r[4]), "=f"(r[5]), "=f"(r[6]), "=f"(r[7])
+               : "r"(ta) : "memory");
+}
+__device__ __forceinline__ void tmem_st8(uint32_t ta, const float (&r)[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
+               ::"r"(ta), "f"(r[0]), "f"(r[1]), "f"(r[2]), "f"(r[3]), "f"(r[4]), "f"(r[5]), "f"(r[6]), "f"(r[7]) : "memory");
+}
+
+__device__ __forceinline__ void tmem_ld4(uint32_t ta, float (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=f"(r[0]), "=f"(r[1]), "=f"(r[2]), "=f"(r[3]) : "r"(ta) : "memory");
+}
+__device__ __forceinline__ void tmem_st4(uint32_t ta, const float (&r)[4]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};"
+               ::"r"(ta), "f"(r[0]), "f"(r[1]), "f"(r[2]), "f"(r[3]) : "memory");
+}
+
+// Staging of a warp's column blocks: NR rows of 32 columns (128 bytes a row), by the warp's own cp.async.
+template <int NR>
+__device__ __forceinline__ void stage_block(const float* src32, float* stg, int lane) {  // src32: the block's first column
+  const float* s = src32 + (static_cast<long long>(lane >> 3) << R) + 4 * (lane & 7);
+  const uint32_t d = tc::smem_u32(stg) + 16 * lane;
+#pragma unroll
+  for (int j = 0; j < NR / 4; ++j) cp_async16(d + 512 * j, s + (static_cast<long long>(4 * j) << R));
+}
+constexpr int WARP_STAGE = SLOT_BYTES / 4 / (THREADS / 32);  // floats of the slots per warp (12 KiB)
+
+// Columns of up to 64 rows, whole in a thread's registers; a warp's next blocks are staged behind it.
+template <int Q, class GainT>
+__device__ __forceinline__ void col_regs(float* ws, int cols, const Params& P, const float* tab, float* slots) {
+  constexpr int NR = 1 << Q, NP = NR / 2, m = R + Q;
+  constexpr int PER = 32 * (NR < 4 ? 4 : NR);
+  constexpr int RING = WARP_STAGE / PER > 3 ? 3 : WARP_STAGE / PER;  // blocks in flight
+  static_assert(RING >= 1, "a block fits the warp's staging area");
+  const float2 sc = make_float2(P.scale, P.scale);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int first = warp * gridDim.x + blockIdx.x, step = gridDim.x * (THREADS / 32), n = cols / 32;
+  float* stg = slots + warp * WARP_STAGE;
+  auto block = [&](int w) { return ws + (static_cast<long long>((32 * w) >> R) << m) + ((32 * w) & (TILE - 1)); };
+  auto stage = [&](int w, int slot) {
+    if (w < n) {
+      if constexpr (NR >= 4) {
+        stage_block<NR>(block(w), stg + slot * PER, lane);
+      } else {  // two rows: half the warp
+        if (lane < 8 * NR)
+          cp_async16(tc::smem_u32(stg + slot * PER) + 16 * lane, block(w) + (static_cast<long long>(lane >> 3) << R) + 4 * (lane & 7));
+      }
+    }
+    fast::cp_async_commit();
+  };
+#pragma unroll
+  for (int k = 0; k < RING; ++k) stage(first + k * step, k);
+  int slot = 0;
+  for (int w = first; w < n; w += step) {
+    float* base = block(w) + lane;
+    const GainT gain(P, tab, ((32 * w) & (TILE - 1)) + lane);
+    float2 v[NP], gg[NP < 16 ? NP : 16];
+#pragma unroll
+    for (int j = 0; j < NP && j < 16; ++j) gg[j] = gain.rows2(2 * j);
+    asm volatile("cp.async.wait_group %0;" ::"n"(RING - 1) : "memory");
+    __syncwarp();
+    const float* b = stg + slot * PER + lane;
+#pragma unroll
+    for (int j = 0; j < NP; ++j) v[j] = make_float2(b[64 * j], b[64 * j + 32]);
+    __syncwarp();
+    stage(w + RING * step, slot);
+    slot = slot + 1 == RING ? 0 : slot + 1;
+#pragma unroll
+    for (int j = 0; j < NP; ++j) bf_in(v[j]);
+    fast::bfly_all<NP>(v);
+#pragma unroll
+    for (int j = 0; j < NP && j < 16; ++j) v[j] = mul2(v[j], mul2(gg[j], sc));
+    if constexpr (NP > 16) {
+#pragma unroll
+      for (int j = 16; j < NP; ++j) gg[j - 16] = gain.rows2(2 * j);
+#pragma unroll
+      for (int j = 16; j < NP; ++j) v[j] = mul2(v[j], mul2(gg[j - 16], sc));
+    }
+#pragma unroll
+    for (int j = 0; j < NP; ++j) bf_in(v[j]);
+    fast::bfly_all<NP>(v);
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+      __stcg(base + ((2 * j) << R), v[j].x);
+      __stcg(base + ((2 * j + 1) << R), v[j].y);
+    }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+// Columns of 128, 256 and 512 rows: NW warps of a tensor-memory lane quarter hold 32 columns, two blocks of 64
+// rows of each per warp.  All four warps of a quarter run on one sub-partition of the SM, so columns are
+// given to as few warps as tensor memory (512 words a lane) allows: the groups then drift apart and one
+// group's loads overlap another's butterflies.
+//   round A  blocks of 64 rows, bits 0..5: workspace -> registers -> tensor memory (the second block staged
+//            in shared memory meanwhile);
+//   round B  bits 6.. across the NB blocks, 32 values a pass, each pass's gains loaded a pass ahead;
+//   round C  blocks of 64 rows, bits 0..5 again -> workspace.
+template <int Q>
+struct Lane {
+  static constexpr int NB = 1 << (Q - 6);           // blocks of 64 rows
+  static constexpr int NW = NB / 2;                 // warps per group of 32 columns
+  static constexpr int GROUPS = THREADS / 32 / NW;  // groups a CTA works on at a time
+  static constexpr int W = 32 / NB;                 // rows of each block per pass of round B: four passes
+};
+template <int NW>
+__device__ __forceinline__ void lane_sync(int group) {
+  fast::tmem_wait_st();
+  if constexpr (NW > 1) {
+    fast::tmem_fence_before();
+    asm volatile("bar.sync %0, %1;" ::"r"(group + 1), "r"(32 * NW) : "memory");
+    fast::tmem_fence_after();
+  }
+}
+// words ta .. ta + 2 N - 1 of this lane <-> N pairs
+template <int N>
+__device__ __forceinline__ void ld_pairs(uint32_t ta, float2* v) {
+  float f[2 * N];
+  if constexpr (N == 8) fast::tmem_ld16(ta, f);
+  else if constexpr (N == 4) tmem_ld8(ta, f);
+  else tmem_ld4(ta, f);
+#pragma unroll
+  for (int k = 0; k < N; ++k) v[k] = make_float2(f[2 * k], f[2 * k + 1]);
+}
+template <int N>
+__device__ __forceinline__ void st_pairs(uint32_t ta, const float2* v) {
+  float f[2 * N];
+#pragma unroll
+  for (int k = 0; k < N; ++k) f[2 * k] = v[k].x, f[2 * k + 1] = v[k].y;
+  if constexpr (N == 8) fast::tmem_st16(ta, f);
+  else if constexpr (N == 4) tmem_st8(ta, f);
+  else tmem_st4(ta, f);
+}
+template <int Q, class GainT>
+__device__ __forceinline__ void col_lanes(float* ws, int begin, int end, const Params& P, const float* tab, uint32_t tmem,
+                                          float* slots) {
+  using C = Lane<Q>;
+  constexpr int m = R + Q, NB = C::NB, NW = C::NW, W = C::W, WP = W / 2;
+  const float2 sc = make_float2(P.scale, P.scale);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quarter = warp & 3;
+  const int half = (warp >> 2) / NW, i = (warp >> 2) % NW;  // warps of a group share a quarter
+  const int group = quarter + 4 * half;
+  const uint32_t ta = tmem + (static_cast<uint32_t>(32 * quarter) << 16) + half * (64 * NB);
+  float* stg = slots + warp * WARP_STAGE;
+  auto block = [&](int g, int b) {  // first column, row 64 b of group g
+    return ws + (static_cast<long long>((32 * g) >> R) << m) + ((32 * g) & (TILE - 1)) + (static_cast<long long>(64 * b) << R);
+  };
+  if (begin + group < end) stage_block<64>(block(begin + group, i + NW), stg, lane);
+  for (int g = begin + group; g < end; g += C::GROUPS) {
+    const GainT gain(P, tab, ((32 * g) & (TILE - 1)) + lane);
+    auto round_ac = [&](float2 (&v)[32]) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j) bf_in(v[j]);
+      bfly32<0>(v);
+    };
+    {
+      float2 v[32];
+      const float* src = block(g, i) + lane;
+#pragma unroll
+      for (int j = 0; j < 32; ++j) v[j] = make_float2(__ldcg(src + ((2 * j) << R)), __ldcg(src + ((2 * j + 1) << R)));
+      round_ac(v);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) st_pairs<8>(ta + 64 * i + 16 * q, v + 8 * q);
+      fast::cp_async_wait_all();
+      __syncwarp();
+#pragma unroll
+      for (int j = 0; j < 32; ++j) v[j] = make_float2(stg[64 * j + lane], stg[64 * j + 32 + lane]);
+      __syncwarp();
+      if (g + C::GROUPS < end) stage_block<64>(block(g + C::GROUPS, i + NW), stg, lane);
+      round_ac(v);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) st_pairs<8>(ta + 64 * (i + NW) + 16 * q, v + 8 * q);
+    }
+    // round B: pair k = (s, low) is rows 64 s + (64 / NW) i + W pass + 2 low and + 1
+    const int low0 = (64 / NW) * i;
+    auto load_gains = [&](float2 (&gg)[16], int pass) {
+#pragma unroll
+      for (int k = 0; k < 16; ++k) gg[k] = gain.rows2(64 * (k / WP) + low0 + W * pass + 2 * (k % WP));
+    };
+    auto round_b_pass = [&](const float2 (&gg)[16], int pass) {
+      float2 v[16];
+#pragma unroll
+      for (int s = 0; s < NB; ++s) ld_pairs<WP>(ta + 64 * s + low0 + W * pass, v + WP * s);
+      fast::tmem_wait_ld();
+      auto across = [&] {
+#pragma unroll
+        for (int h = WP; h < 16; h <<= 1)
+#pragma unroll
+          for (int k = 0; k < 16; ++k)
+            if ((k & h) == 0) bf2(v[k], v[k + h]);
+      };
+      across();
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = mul2(v[k], mul2(gg[k], sc));
+      across();
+#pragma unroll
+      for (int s = 0; s < NB; ++s) st_pairs<WP>(ta + 64 * s + low0 + W * pass, v + WP * s);
+    };
+    float2 ga[16], gb[16];
+    load_gains(ga, 0);
+    lane_sync<NW>(group);
+#pragma unroll 1
+    for (int pass = 0; pass < 4; pass += 2) {
+      load_gains(gb, pass + 1);
+      round_b_pass(ga, pass);
+      if (pass == 0) load_gains(ga, 2);
+      round_b_pass(gb, pass + 1);
+    }
+    lane_sync<NW>(group);
+#pragma unroll 1
+    for (int it = 0; it < 2; ++it) {
+      float2 v[32];
+      float* dst = block(g, i + NW * it) + lane;
+      read_row(ta + 64 * (i + NW * it), v);
+      round_ac(v);
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        __stcg(dst + ((2 * j) << R), v[j].x);
+        __stcg(dst + ((2 * j + 1) << R), v[j].y);
+      }
+    }
+    // the next columns' round A writes only this warp's own blocks, which the others stopped reading at the
+    // second lane_sync
+  }
+}
+
+// ---------------------------------------------------------------------------------------------
+// Columns.  A unit is W = 2^(14-Q) adjacent columns of all 2^Q rows of a plane, two slots; its element e (row
+// e >> (14-Q), column e mod W) is word e, bit 4 XORed with bit 9.  A team's thread tt takes
+//   round A  the pairs at 2 tt + 512 i, i = 0..31 (word bits 9..13);
+//   round B  word bits 1, 2, 3, 9, 10 in the lane, 11..13 in the warp, 4..8 in the registers.
+// Word bit x is a row bit, and takes a butterfly, if x >= 14 - Q; Q <= 5 needs round A alone.
+constexpr int UNIT = 2 * TILE;
+template <int Q>
+struct Col {
+  static constexpr int W = 1 << (R + 1 - Q);
+  static constexpr int A0 = 5 - Q > 0 ? 5 - Q : 0;    // first row bit of round A's index
+  static constexpr int B0 = 10 - Q > 0 ? 10 - Q : 0;  // first row bit of round B's index
+  static constexpr bool TWO = Q > 5;
+  // plane offset of unit word e; additive over disjoint bits
+  __host__ __device__ static constexpr int off(int e) { return ((e >> (R + 1 - Q)) << R) + (e & (W - 1)); }
+};
+
+// Gains of a thread's pairs in the round that applies them: pair k sits at unit words e0 + STEP k and + 1.
+template <int Q>
+struct FullGain {
+  const float* p;
+  __device__ __forceinline__ FullGain(const Params& P, const float*, int col0, int e0)
+      : p(static_cast<const float*>(P.g) + col0 + Col<Q>::off(e0)) {}
+  template <int STEP>
+  __device__ __forceinline__ float2 at(int k) const {
+    return __ldg(reinterpret_cast<const float2*>(p + Col<Q>::off(STEP * k)));
+  }
+  __device__ __forceinline__ float2 row(int j) const { return __ldg(reinterpret_cast<const float2*>(p + (j << R))); }
+};
+// Separable log gains: G[n, c] = et[n] ec[c] from two tables that phase 1 builds (tab): the token table is
+// stored so that a column's rows are consecutive, et[(column >> cb) 2^Q + row].
+template <int Q>
+struct SepGain {
+  const float* et;
+  const float* ec;
+  int cb, c0, j0;
+  __device__ __forceinline__ SepGain(const Params& P, const float* tab, int col0, int e0)
+      : et(tab), ec(tab + (1ll << (P.m - P.cbits))), cb(P.cbits), c0(col0 + (e0 & (Col<Q>::W - 1))), j0(e0 >> (R + 1 - Q)) {}
+  template <int STEP>
+  __device__ __forceinline__ float2 at(int k) const {
+    const int e = STEP * k, c = c0 + (e & (Col<Q>::W - 1)), j = j0 + (e >> (R + 1 - Q)), ch = c & ((1 << cb) - 1);
+    const float t = et[(static_cast<long long>(c >> cb) << Q) + j];
+    return make_float2(t * ec[ch], t * ec[ch + 1]);
+  }
+  __device__ __forceinline__ float2 row(int j) const {
+    const int ch = c0 & ((1 << cb) - 1);
+    const float t = et[(static_cast<long long>(c0 >> cb) << Q) + j];
+    return make_float2(t * ec[ch], t * ec[ch + 1]);
+  }
+};
+
+// Unit u of the plane group (first element at `src`) into two slots, by one team.
+template <int Q>
+__device__ __forceinline__ void load_unit(const float* src, float* slot, int tt, uint64_t* full) {
+  using C = Col<Q>;
+  const float* s = src + C::off(4 * tt);
+  const uint32_t d = tc::smem_u32(slot) + 4 * ((4 * tt) ^ (((tt >> 7) & 1) << 4));
+#pragma unroll
+  for (int i = 0; i < 16; ++i) cp_async16(d + 4096 * i, s + C::off(1024 * i));
+  cp_async_arrive(full);
+}
+
+// Phase 2 of one unit: column bits, gain, column bits; the result to the workspace at `dst` (the unit's first
+// element).  `wait` is called before the slot is read, so that the first gains are on their way by then.
+template <int Q, class GainT, class Wait>
+__device__ __forceinline__ void col_unit(float* slot, float* dst, const Params& P, const float* tab, int col0, int tt,
+                                         int team, const Wait& wait) {
+  using C = Col<Q>;
+  const float2 sc = make_float2(P.scale, P.scale);
+  const int l = tt & 31;
+  const int e0 = C::TWO ? 2 * (l & 7) + 512 * (l >> 3) + 2048 * (tt >> 5) : 2 * tt;
+  constexpr int STEP = C::TWO ? 16 : 512;
+  const GainT gain(P, tab, col0, e0);
+  float2 gg[16];
+#pragma unroll
+  for (int k = 0; k < 16; ++k) gg[k] = gain.template at<STEP>(k);
+  wait();
+  float2 v[32];
+  const int a0 = 2 * tt, a1 = a0 ^ 16;
+#pragma unroll
+  for (int i = 0; i < 32; ++i) v[i] = *reinterpret_cast<const float2*>(slot + (i & 1 ? a1 : a0) + 512 * i);
+  bfly32<C::A0>(v);
+  const int b0 = e0 ^ (((l >> 3) & 1) << 4), b1 = b0 ^ 16;  // round B: bit 4 is the registers' lowest
+  if constexpr (C::TWO) {
+#pragma unroll
+    for (int i = 0; i < 32; ++i) *reinterpret_cast<float2*>(slot + (i & 1 ? a1 : a0) + 512 * i) = v[i];
+    team_sync(team);
+#pragma unroll
+    for (int k = 0; k < 32; ++k) v[k] = *reinterpret_cast<const float2*>(slot + (k & 1 ? b1 : b0) + 32 * (k >> 1));
+    bfly32<C::B0>(v);
+  }
+#pragma unroll
+  for (int k = 0; k < 16; ++k) v[k] = mul2(v[k], mul2(gg[k], sc));
+#pragma unroll
+  for (int k = 0; k < 16; ++k) gg[k] = gain.template at<STEP>(k + 16);
+#pragma unroll
+  for (int k = 0; k < 16; ++k) v[k + 16] = mul2(v[k + 16], mul2(gg[k], sc));
+  if constexpr (C::TWO) {
+    bfly32<C::B0>(v);
+#pragma unroll
+    for (int k = 0; k < 32; ++k) *reinterpret_cast<float2*>(slot + (k & 1 ? b1 : b0) + 32 * (k >> 1)) = v[k];
+    team_sync(team);
+#pragma unroll
+    for (int i = 0; i < 32; ++i) v[i] = *reinterpret_cast<const float2*>(slot + (i & 1 ? a1 : a0) + 512 * i);
+  }
+  bfly32<C::A0>(v);
+  float* o = dst + C::off(2 * tt);
+#pragma unroll
+  for (int i = 0; i < 32; ++i) __stcg(reinterpret_cast<float2*>(o + C::off(512 * i)), v[i]);
+}
+
+// ---------------------------------------------------------------------------------------------
+// Forward kernel: persistent grid (one CTA per SM, all resident), plane groups of P.gp planes.
+template <int D, int Q, bool SEP>
+__global__ void __launch_bounds__(THREADS, 1) k_forward_fast(Params P) {
+  extern __shared__ __align__(1024) unsigned char tri_smem[];
+  __shared__ uint64_t full_row[ROW_BARS], full_pair[PAIR_BARS], mma_done[WORKERS][2];
+  __shared__ int flag, dead;
+  __shared__ uint32_t tmem_slot;
+  constexpr int m = R + Q;
+  constexpr bool MMA = D == DT_BF16;
+  constexpr bool TMEM = MMA || (Q >= 7 && Q <= 9);
+  float* slots = reinterpret_cast<float*>(tri_smem);
+  const int worker = threadIdx.x / WT, t = threadIdx.x % WT;
+  const int team = threadIdx.x / (2 * WT), tt = threadIdx.x % (2 * WT);
+  float* ws = static_cast<float*>(P.ws);
+  const float* tab = ws + (static_cast<long long>(P.gp) << m);
+  if constexpr (TMEM) {
+    if (threadIdx.x < 32) fast::tmem_alloc_512(&tmem_slot);
+  }
+  if constexpr (MMA) {
+    build_h(tri_smem + SLOT_BYTES);
+    fence_async();
+  }
+  if (threadIdx.x == 0) {
+    dead = 0;
+    for (int i = 0; i < ROW_BARS; ++i) tc::mbar_init(&full_row[i], WT);
+    for (int i = 0; i < PAIR_BARS; ++i) tc::mbar_init(&full_pair[i], 2 * WT);
+    for (int i = 0; i < WORKERS; ++i)
+      for (int k = 0; k < 2; ++k) tc::mbar_init(&mma_done[i][k], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  {
+    int rb, re;
+    share(static_cast<unsigned>(min(static_cast<long long>(P.gp), P.B)) << Q, &rb, &re);
+    fast::l2_prefetch_first_rows<D, R, Q>(P.x, rb, re, P.lv);
+  }
+  fast::tmem_fence_before();
+  __syncthreads();
+  fast::tmem_fence_after();
+  // tensor memory is allocated before the wait: the previous kernel's CTA on this SM has left
+  pdl_wait();
+  GridSync gsync(P.bar, &flag);
+  // this CTA's share of G, fetched into L2 over phase 1's first rows
+  const long long g_chunks = (4ll << m) >> 4;
+  const long long g_begin = g_chunks * blockIdx.x / gridDim.x, g_end = g_chunks * (blockIdx.x + 1) / gridDim.x;
+  unsigned row_seq = 0, pair_seq = 0, mma_seq = 0;  // tiles taken by earlier phases
+  for (long long b0 = 0; b0 < P.B; b0 += P.gp) {
+    const int nb = static_cast<int>(min(static_cast<long long>(P.gp), P.B - b0));
+    int rb, re;
+    share(static_cast<unsigned>(nb) << Q, &rb, &re);
+    const int n = re - rb;
+    // phase 1: X -> workspace, row bits
+    if constexpr (SEP) {
+      if (b0 == 0) {  // once: the gain tables
+        float* tb = ws + (static_cast<long long>(P.gp) << m);
+        const long long n_t = 1ll << (m - P.cbits), n_tab = n_t + (1ll << P.cbits);
+        for (long long i = static_cast<long long>(blockIdx.x) * THREADS + threadIdx.x; i < n_tab;
+             i += static_cast<long long>(gridDim.x) * THREADS)
+          tb[i] = expf(i < n_t ? P.gt[fast::sep_token_of<R, Q>(i, P.cbits)] : P.gc[i - n_t]);
+      }
+    }
+    const int g_step = n > 0 ? static_cast<int>((g_end - g_begin + n - 1) / n) : 0;
+    auto prefetch_g = [&](int k) {  // one thread per row
+      if (SEP || b0 != 0) return;
+      const long long c0 = g_begin + static_cast<long long>(g_step) * k, c1 = min(c0 + g_step, g_end);
+      if (c1 > c0)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(static_cast<const char*>(P.g) + (c0 << 4)),
+                     "r"(static_cast<unsigned>((c1 - c0) << 4)) : "memory");
+    };
+    if constexpr (MMA) {
+      // the worker's i-th row (row worker + 4 i of the CTA's) is staged in its area i mod 3 and multiplied into
+      // its accumulator i mod 2
+      const int nw = (n - worker + WORKERS - 1) / WORKERS;
+      const uint32_t xs = tc::smem_u32(tri_smem) + worker * (XSLOTS * TILE * 2);
+      const uint32_t sh = tc::smem_u32(tri_smem) + SLOT_BYTES;
+      const uint32_t acc = tmem_slot + 128u * worker;
+      auto load = [&](int i) {
+        if (i < nw) {
+          long long e0;
+          int lim;
+          fast::row_loc<R, Q>(b0, rb + worker + WORKERS * i, P.lv, &e0, &lim);
+          load_x_bf16(static_cast<const unsigned short*>(P.x) + e0, lim, xs + (i % XSLOTS) * (TILE * 2), t);
+        }
+        fast::cp_async_commit();
+      };
+      // staged row i (at most `pending` later ones still in flight) -> its accumulator
+      auto multiply = [&](int i) {
+        fence_async();
+        fast::tmem_fence_before();
+        worker_sync(worker);
+        if (t == 0) {
+          fast::tmem_fence_after();
+          mma_row(acc + 64u * (i & 1), sh, xs + (i % XSLOTS) * (TILE * 2));
+          tc::mma_commit(&mma_done[worker][(mma_seq + i) & 1]);
+        }
+      };
+      for (int i = 0; i < XSLOTS; ++i) load(i);
+      if (nw > 0) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(XSLOTS - 1) : "memory");
+        multiply(0);
+      }
+      for (int i = 0; i < nw; ++i) {
+        if (t == 0) prefetch_g(worker + WORKERS * i);
+        if (i + 1 < nw) {
+          asm volatile("cp.async.wait_group %0;" ::"n"(XSLOTS - 2) : "memory");
+          multiply(i + 1);
+        }
+        wait_bar(&mma_done[worker][(mma_seq + i) & 1], ((mma_seq + i) >> 1) & 1u, P.bar, &dead);
+        __syncwarp();
+        fast::tmem_fence_after();
+        float2 v[32];
+        read_row(acc + 64u * (i & 1) + (static_cast<uint32_t>(32 * ((threadIdx.x >> 5) & 3)) << 16), v);
+        load(i + XSLOTS);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) bf_in(v[j]);
+        bfly32<0>(v);
+        float* dst = ws + (static_cast<long long>(rb + worker + WORKERS * i) << R) + t;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          __stcg(dst + 256 * j, v[j].x);
+          __stcg(dst + 256 * j + 128, v[j].y);
+        }
+      }
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+      mma_seq += nw > 0 ? nw : 0;
+      fast::tmem_fence_before();
+    } else {
+      auto load = [&](int k) {
+        long long e0;
+        int lim;
+        fast::row_loc<R, Q>(b0, rb + k, P.lv, &e0, &lim);
+        load_row(static_cast<const float*>(P.x) + e0, lim, slots + (row_seq + k) % SLOTS * TILE, t, &full_row[(row_seq + k) % ROW_BARS]);
+      };
+      for (int k = worker; k < SLOTS && k < n; k += WORKERS) load(k);
+      for (int k = worker; k < n; k += WORKERS) {
+        if (t == 0) prefetch_g(k);
+        wait_full(full_row, row_seq + k, ROW_BARS, P.bar, &dead);
+        row_in(slots + (row_seq + k) % SLOTS * TILE, ws + (static_cast<long long>(rb + k) << R), t, worker, [&] {
+          if (k + SLOTS < n) load(k + SLOTS);
+        });
+      }
+      row_seq += n;
+    }
+    if (!gsync()) break;
+    // phase 2: columns
+    {
+      using LaneT = typename std::conditional<SEP, LaneSep<Q>, LaneFull<Q>>::type;
+      if constexpr (Q <= 6) {
+        col_regs<Q, LaneT>(ws, nb << R, P, tab, slots);
+      } else if constexpr (Q <= 9) {
+        int gb, ge;
+        share(static_cast<unsigned>(nb) << (R - 5), &gb, &ge);
+        col_lanes<Q, LaneT>(ws, gb, ge, P, tab, tmem_slot, slots);
+        fast::tmem_fence_before();
+      } else {
+        using GainT = typename std::conditional<SEP, SepGain<Q>, FullGain<Q>>::type;
+        constexpr int UB = Q - 1;  // log2 of the units of a plane
+        int ub, ue;
+        share(static_cast<unsigned>(nb) << UB, &ub, &ue);
+        const int nu = ue - ub;
+        auto base = [&](int k, int* col0) {
+          const int u = ub + k, c = (u & ((1 << UB) - 1)) << (R + 1 - Q);
+          *col0 = c;
+          return ws + (static_cast<long long>(u >> UB) << m) + c;
+        };
+        auto load = [&](int k) {
+          int c;
+          const float* src = base(k, &c);
+          load_unit<Q>(src, slots + (pair_seq + k) % PAIRS * UNIT, tt, &full_pair[(pair_seq + k) % PAIR_BARS]);
+        };
+        for (int k = team; k < PAIRS && k < nu; k += 2) load(k);
+        for (int k = team; k < nu; k += 2) {
+          int col0;
+          float* dst = base(k, &col0);
+          col_unit<Q, GainT>(slots + (pair_seq + k) % PAIRS * UNIT, dst, P, tab, col0, tt, team,
+                             [&] { wait_full(full_pair, pair_seq + k, PAIR_BARS, P.bar, &dead); });
+          if (k + PAIRS < nu) {
+            team_sync(team);
+            load(k + PAIRS);
+          }
+        }
+        pair_seq += nu;
+      }
+    }
+    if (!gsync()) break;
+    // phase 3: workspace -> Y, row bits
+    {
+      auto load = [&](int k) {
+        load_row(ws + (static_cast<long long>(rb + k) << R), TILE, slots + (row_seq + k) % SLOTS * TILE, t,
+                 &full_row[(row_seq + k) % ROW_BARS]);
+      };
+      for (int k = worker; k < SLOTS && k < n; k += WORKERS) load(k);
+      for (int k = worker; k < n; k += WORKERS) {
+        long long e0;
+        int lim;
+        fast::row_loc<R, Q>(b0, rb + k, P.lv, &e0, &lim);
+        wait_full(full_row, row_seq + k, ROW_BARS, P.bar, &dead);
+        row_out<D>(slots + (row_seq + k) % SLOTS * TILE, P.y, e0, lim, t, worker, [&] {
+          if (k + SLOTS < n) load(k + SLOTS);
+        });
+      }
+      row_seq += n;
+    }
+    if (b0 + P.gp < P.B && !gsync()) break;
+  }
+  pdl_trigger();
+  if constexpr (TMEM) {
+    fast::tmem_fence_before();
+    __syncthreads();
+    fast::tmem_fence_after();
+    if (threadIdx.x < 32) fast::tmem_dealloc_512(tmem_slot);
+  }
+}
+
+}  // namespace tri
+}  // namespace whtmix
