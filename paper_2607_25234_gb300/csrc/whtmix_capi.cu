@@ -290,12 +290,12 @@ int dispatch_plan_l(bool backward, const Params& P, int sms, cudaStream_t stream
   return rc;
 }
 
-// The fast forward (whtmix_fast.cuh) covers fp32 / bf16 planes with 2^14 <= N*C <= 2^23.
+// The three-phase forward (whtmix_tri.cuh) covers fp32 / bf16 planes with 2^14 <= N*C <= 2^25.
 bool use_fast_forward(int dtype, int m) {
-  return (dtype == WHTMIX_F32 || dtype == WHTMIX_BF16) && m >= 14 && m <= 23;
+  return (dtype == WHTMIX_F32 || dtype == WHTMIX_BF16) && m >= 14 && m <= 25;
 }
 
-// The fast backward (whtmix_fast_bwd.cuh) covers fp32 / bf16 planes with 2^14 <= N*C <= 2^23.
+// The three-phase backward (whtmix_tri.cuh) covers fp32 / bf16 planes with 2^14 <= N*C <= 2^23.
 bool use_fast_backward(int dtype, int m) {
   return (dtype == WHTMIX_F32 || dtype == WHTMIX_BF16) && m >= 14 && m <= 23;
 }
@@ -410,7 +410,7 @@ long long sep_chunks(int m, int cbits) {
 }
 
 bool use_fast_separable(int dtype, int m, int cbits) {
-  return use_fast_forward(dtype, m) && cbits >= 1 && cbits <= fast::forward_row_bits(m);
+  return use_fast_forward(dtype, m) && cbits >= 1 && cbits <= 13;
 }
 
 // Zero padding / crop on the token axis for the shapes the fast kernels do not pad themselves:
@@ -469,7 +469,7 @@ struct Call {
 
 // The call runs the three-phase fast forward with the bf16 exchange workspace.
 bool x16_applies(const Call& c, int m) {
-  return c.ws16 && !c.backward && !c.separable && !c.w_in && use_fast_forward(c.dtype, m);
+  return c.ws16 && !c.backward && !c.separable && !c.w_in && m <= 23 && use_fast_forward(c.dtype, m);
 }
 
 // Workspace layout of a call: the kernel workspace (barrier header + plane group) first, then

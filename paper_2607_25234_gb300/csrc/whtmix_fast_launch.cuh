@@ -9,7 +9,6 @@
 #include <mutex>
 
 #include "whtmix_fast.cuh"
-#include "whtmix_fast_bwd.cuh"
 #include "whtmix_tri.cuh"
 
 namespace whtmix {
@@ -53,84 +52,48 @@ inline cudaError_t launch_persistent(const void* k, const Params& P, int sms, cu
   void* args[] = {&p};
   return launch_pdl(k, static_cast<unsigned>(sms), threads, smem, stream, args);
 }
-template <int D, int R, int Q, bool SEP, class WS = WsF32>
-cudaError_t launch_one(const Params& P, int sms, cudaStream_t stream) {
-  return launch_persistent(reinterpret_cast<const void*>(k_forward_fast<D, R, Q, SEP, WS>), P, sms, stream);
-}
-template <int D, int R, int Q>
-cudaError_t launch_bwd_one(const Params& P, int sms, cudaStream_t stream) {
-  return launch_persistent(reinterpret_cast<const void*>(k_backward_fast<D, R, Q>), P, sms, stream);
-}
-
-// The older three-phase kernel, for the 2^21-element planes and the bf16 exchange (WS = WsB16,
-// whtmix_forward_x16).
-// Rows of 2^13 elements at every size but 2^21; 2^23-element planes take 1024-row columns (two
-// lanes per column).  With 152 SMs, 1024 rows of 2^13 spread as 7 or 6 per CTA, where 512 rows of
-// 2^14 give 56 CTAs four rows against three; measured on the 2^22 planes, 2^13 rows with 512-row
-// columns beat 2^14 rows.  2^21-element planes take rows of 2^14 and 128-row columns, one column
-// per thread in registers, instead of 256-row columns in tensor memory: measured on sixteen such
-// planes (bf16), 138 us against 146 us per call.
-// SEP: separable log gains (P.gt, P.gc) instead of G; needs 1 <= P.cbits <= row bits.
-// WS: the workspace element (WsB16: whtmix_forward_x16).
-// The three-phase forward: rows of 2^13 at every size but 2^21, whose rows of 2^14 and 128-row columns stay with
-// the older kernel: next to the backward of a training step it measured no faster ([16, 8192, 256] bf16, forward
-// and backward: 465 us against 470).
-template <int D, int Q, bool SEP>
-cudaError_t launch_tri(const Params& P, int sms, cudaStream_t stream) {
-  return launch_persistent(reinterpret_cast<const void*>(tri::k_forward_fast<D, Q, SEP>), P, sms, stream, tri::THREADS,
-                           tri::smem_bytes<D>());
-}
-template <int D, bool SEP>
+// The three-phase kernels (whtmix_tri.cuh) of a 2^m-element plane: 2^(m-13) rows of 2^13.  SEP: separable log gains
+// (P.gt, P.gc) instead of G; needs 1 <= P.cbits <= 13.
+template <int D, bool SEP, int M = 14>
 cudaError_t launch_forward_tri(const Params& P, int sms, cudaStream_t stream) {
-  switch (P.m) {
-    case 14: return launch_tri<D, 1, SEP>(P, sms, stream);
-    case 15: return launch_tri<D, 2, SEP>(P, sms, stream);
-    case 16: return launch_tri<D, 3, SEP>(P, sms, stream);
-    case 17: return launch_tri<D, 4, SEP>(P, sms, stream);
-    case 18: return launch_tri<D, 5, SEP>(P, sms, stream);
-    case 19: return launch_tri<D, 6, SEP>(P, sms, stream);
-    case 20: return launch_tri<D, 7, SEP>(P, sms, stream);
-    case 21: return launch_one<D, 14, 7, SEP>(P, sms, stream);
-    case 22: return launch_tri<D, 9, SEP>(P, sms, stream);
-    case 23: return launch_tri<D, 10, SEP>(P, sms, stream);
-    default: return cudaErrorInvalidValue;
+  if constexpr (M <= 25) {
+    if (P.m != M) return launch_forward_tri<D, SEP, M + 1>(P, sms, stream);
+    return launch_persistent(reinterpret_cast<const void*>(tri::k_forward_fast<D, M - tri::R, SEP>), P, sms, stream,
+                             tri::THREADS, tri::smem_bytes<D>());
   }
+  return cudaErrorInvalidValue;
 }
-template <int D, bool SEP, class WS = WsF32>
-cudaError_t launch_forward(const Params& P, int sms, cudaStream_t stream) {
-  switch (P.m) {
-    case 14: return launch_one<D, 13, 1, SEP, WS>(P, sms, stream);
-    case 15: return launch_one<D, 13, 2, SEP, WS>(P, sms, stream);
-    case 16: return launch_one<D, 13, 3, SEP, WS>(P, sms, stream);
-    case 17: return launch_one<D, 13, 4, SEP, WS>(P, sms, stream);
-    case 18: return launch_one<D, 13, 5, SEP, WS>(P, sms, stream);
-    case 19: return launch_one<D, 13, 6, SEP, WS>(P, sms, stream);
-    case 20: return launch_one<D, 13, 7, SEP, WS>(P, sms, stream);
-    case 21: return launch_one<D, 14, 7, SEP, WS>(P, sms, stream);
-    case 22: return launch_one<D, 13, 9, SEP, WS>(P, sms, stream);
-    case 23: return launch_one<D, 13, 10, SEP, WS>(P, sms, stream);
-    default: return cudaErrorInvalidValue;
-  }
-}
-// Row bits of the fast forward for a 2^m-element plane.
-inline int forward_row_bits(int m) { return m == 21 ? 14 : 13; }
-
-// Backward: rows of 2^13 up to 2^20-element planes (columns of at most 128 rows, the transformed X
-// column of a 128-row column parked in TMEM) and rows of 2^14 from 2^21 (columns of 128, 256 and
-// 512 rows; the TMEM column pass for 256 and 512).
-template <int D>
+template <int D, int M = 14>
 cudaError_t launch_backward(const Params& P, int sms, cudaStream_t stream) {
+  if constexpr (M <= 23) {
+    if (P.m != M) return launch_backward<D, M + 1>(P, sms, stream);
+    return launch_persistent(reinterpret_cast<const void*>(tri::k_backward_fast<D, M - tri::R>), P, sms, stream,
+                             tri::THREADS, tri::smem_bytes<D>());
+  }
+  return cudaErrorInvalidValue;
+}
+
+// The bf16-exchange forward (whtmix_forward_x16; whtmix_fast.cuh).  Rows of 2^13 elements at every size but 2^21;
+// 2^23-element planes take 1024-row columns (two lanes per column).  With 152 SMs, 1024 rows of 2^13 spread as 7 or 6
+// per CTA, where 512 rows of 2^14 give 56 CTAs four rows against three; 2^21-element planes take rows of 2^14 and
+// 128-row columns, one column per thread in registers, instead of 256-row columns in tensor memory.
+template <int D, int R, int Q>
+cudaError_t launch_x16_one(const Params& P, int sms, cudaStream_t stream) {
+  return launch_persistent(reinterpret_cast<const void*>(k_forward_fast<D, R, Q, false, WsB16>), P, sms, stream);
+}
+template <int D>
+cudaError_t launch_forward_x16(const Params& P, int sms, cudaStream_t stream) {
   switch (P.m) {
-    case 14: return launch_bwd_one<D, 13, 1>(P, sms, stream);
-    case 15: return launch_bwd_one<D, 13, 2>(P, sms, stream);
-    case 16: return launch_bwd_one<D, 13, 3>(P, sms, stream);
-    case 17: return launch_bwd_one<D, 13, 4>(P, sms, stream);
-    case 18: return launch_bwd_one<D, 13, 5>(P, sms, stream);
-    case 19: return launch_bwd_one<D, 13, 6>(P, sms, stream);
-    case 20: return launch_bwd_one<D, 13, 7>(P, sms, stream);
-    case 21: return launch_bwd_one<D, 14, 7>(P, sms, stream);
-    case 22: return launch_bwd_one<D, 14, 8>(P, sms, stream);
-    case 23: return launch_bwd_one<D, 14, 9>(P, sms, stream);
+    case 14: return launch_x16_one<D, 13, 1>(P, sms, stream);
+    case 15: return launch_x16_one<D, 13, 2>(P, sms, stream);
+    case 16: return launch_x16_one<D, 13, 3>(P, sms, stream);
+    case 17: return launch_x16_one<D, 13, 4>(P, sms, stream);
+    case 18: return launch_x16_one<D, 13, 5>(P, sms, stream);
+    case 19: return launch_x16_one<D, 13, 6>(P, sms, stream);
+    case 20: return launch_x16_one<D, 13, 7>(P, sms, stream);
+    case 21: return launch_x16_one<D, 14, 7>(P, sms, stream);
+    case 22: return launch_x16_one<D, 13, 9>(P, sms, stream);
+    case 23: return launch_x16_one<D, 13, 10>(P, sms, stream);
     default: return cudaErrorInvalidValue;
   }
 }

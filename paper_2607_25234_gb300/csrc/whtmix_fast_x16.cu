@@ -5,10 +5,10 @@
 namespace whtmix {
 namespace fast {
 cudaError_t forward_x16_f32(const Params& P, int sms, cudaStream_t stream) {
-  return launch_forward<DT_F32, false, WsB16>(P, sms, stream);
+  return launch_forward_x16<DT_F32>(P, sms, stream);
 }
 cudaError_t forward_x16_bf16(const Params& P, int sms, cudaStream_t stream) {
-  return launch_forward<DT_BF16, false, WsB16>(P, sms, stream);
+  return launch_forward_x16<DT_BF16>(P, sms, stream);
 }
 }  // namespace fast
 }  // namespace whtmix

@@ -253,9 +253,10 @@ __device__ __forceinline__ void row_in(float* slot, float* ws_row, int t, int wo
   }
 }
 
-// Phase 3: the workspace row in `slot` -> the first lim elements of Y's row at dst + e0.
-template <int D, class Done>
-__device__ __forceinline__ void row_out(float* slot, void* dst, long long e0, int lim, int t, int worker, const Done& done) {
+// Phase 3: the row bits of the workspace row in `slot`, into the quads of round A.  `done` is called once the slot is
+// free.
+template <class Done>
+__device__ __forceinline__ void row_transform(float* slot, float2 (&a)[16][2], int t, int worker, const Done& done) {
   {
     const RowB rb(t);
     float2 b[32];
@@ -269,7 +270,6 @@ __device__ __forceinline__ void row_out(float* slot, void* dst, long long e0, in
     }
   }
   worker_sync(worker);
-  float2 a[16][2];
 #pragma unroll
   for (int v = 0; v < 16; ++v) {
     const float4 q = *reinterpret_cast<const float4*>(slot + quad_word(t, v));
@@ -279,6 +279,12 @@ __device__ __forceinline__ void row_out(float* slot, void* dst, long long e0, in
   worker_sync(worker);
   done();
   round_a(a);
+}
+// ... and out: the first lim elements of Y's row at dst + e0.
+template <int D, class Done>
+__device__ __forceinline__ void row_out(float* slot, void* dst, long long e0, int lim, int t, int worker, const Done& done) {
+  float2 a[16][2];
+  row_transform(slot, a, t, worker, done);
 #pragma unroll
   for (int v = 0; v < 16; ++v) {
     const int o = 4 * t + 512 * v;
@@ -376,9 +382,10 @@ __device__ __forceinline__ void col_regs(float* ws, int cols, const Params& P, c
   for (int w = first; w < n; w += step) {
     float* base = block(w) + lane;
     const GainT gain(P, tab, ((32 * w) & (TILE - 1)) + lane);
-    float2 v[NP], gg[NP < 16 ? NP : 16];
+    constexpr int NG = NP < 16 ? NP : 16;  // gains loaded at a time
+    float2 v[NP], gg[NG];
 #pragma unroll
-    for (int j = 0; j < NP && j < 16; ++j) gg[j] = gain.rows2(2 * j);
+    for (int j = 0; j < NG; ++j) gg[j] = gain.rows2(2 * j);
     asm volatile("cp.async.wait_group %0;" ::"n"(RING - 1) : "memory");
     __syncwarp();
     const float* b = stg + slot * PER + lane;
@@ -391,12 +398,13 @@ __device__ __forceinline__ void col_regs(float* ws, int cols, const Params& P, c
     for (int j = 0; j < NP; ++j) bf_in(v[j]);
     fast::bfly_all<NP>(v);
 #pragma unroll
-    for (int j = 0; j < NP && j < 16; ++j) v[j] = mul2(v[j], mul2(gg[j], sc));
-    if constexpr (NP > 16) {
+    for (int h = 0; h < NP; h += NG) {
+      if (h > 0) {
 #pragma unroll
-      for (int j = 16; j < NP; ++j) gg[j - 16] = gain.rows2(2 * j);
+        for (int j = 0; j < NG; ++j) gg[j] = gain.rows2(2 * (h + j));
+      }
 #pragma unroll
-      for (int j = 16; j < NP; ++j) v[j] = mul2(v[j], mul2(gg[j - 16], sc));
+      for (int j = 0; j < NG; ++j) v[h + j] = mul2(v[h + j], mul2(gg[j], sc));
     }
 #pragma unroll
     for (int j = 0; j < NP; ++j) bf_in(v[j]);
@@ -409,6 +417,11 @@ __device__ __forceinline__ void col_regs(float* ws, int cols, const Params& P, c
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
+
+// The column passes of 512 rows and up serve the backward in two more modes: SPECTRUM on the workspace of X (the
+// column bits alone) and then ADJOINT on the workspace of dY, which is FWD and on the way replaces the spectrum of X,
+// at the same positions of xws, by the dG term (W X)(W dY)/L.  Both take the same columns in the same thread.
+enum Mode { FWD, SPECTRUM, ADJOINT };
 
 // Columns of 128, 256 and 512 rows: NW warps of a tensor-memory lane quarter hold 32 columns, two blocks of 64
 // rows of each per warp.  All four warps of a quarter run on one sub-partition of the SM, so columns are
@@ -453,9 +466,9 @@ __device__ __forceinline__ void st_pairs(uint32_t ta, const float2* v) {
   else if constexpr (N == 4) tmem_st8(ta, f);
   else tmem_st4(ta, f);
 }
-template <int Q, class GainT>
+template <int Q, class GainT, Mode MODE = FWD>
 __device__ __forceinline__ void col_lanes(float* ws, int begin, int end, const Params& P, const float* tab, uint32_t tmem,
-                                          float* slots) {
+                                          float* slots, float* xws = nullptr) {
   using C = Lane<Q>;
   constexpr int m = R + Q, NB = C::NB, NW = C::NW, W = C::W, WP = W / 2;
   const float2 sc = make_float2(P.scale, P.scale);
@@ -512,25 +525,58 @@ __device__ __forceinline__ void col_lanes(float* ws, int begin, int end, const P
             if ((k & h) == 0) bf2(v[k], v[k + h]);
       };
       across();
+      // pair k's rows in this column
+      auto row = [&](int k) { return static_cast<long long>(64 * (k / WP) + low0 + W * pass + 2 * (k % WP)) << R; };
+      if constexpr (MODE == SPECTRUM) {
+        float* o = block(g, 0) + lane;
 #pragma unroll
-      for (int k = 0; k < 16; ++k) v[k] = mul2(v[k], mul2(gg[k], sc));
-      across();
+        for (int k = 0; k < 16; ++k) {
+          __stcg(o + row(k), v[k].x);
+          __stcg(o + row(k) + TILE, v[k].y);
+        }
+      } else {
+        if constexpr (MODE == ADJOINT) {
+          float* xp = xws + (block(g, 0) - ws) + lane;
+          float2 xh[16];
 #pragma unroll
-      for (int s = 0; s < NB; ++s) st_pairs<WP>(ta + 64 * s + low0 + W * pass, v + WP * s);
+          for (int k = 0; k < 16; ++k) xh[k] = make_float2(__ldcg(xp + row(k)), __ldcg(xp + row(k) + TILE));
+#pragma unroll
+          for (int k = 0; k < 16; ++k) {
+            const float2 pr = mul2(mul2(xh[k], v[k]), sc);
+            __stcg(xp + row(k), pr.x);
+            __stcg(xp + row(k) + TILE, pr.y);
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < 16; ++k) v[k] = mul2(v[k], mul2(gg[k], sc));
+        across();
+#pragma unroll
+        for (int s = 0; s < NB; ++s) st_pairs<WP>(ta + 64 * s + low0 + W * pass, v + WP * s);
+      }
     };
-    float2 ga[16], gb[16];
-    load_gains(ga, 0);
-    lane_sync<NW>(group);
+    if constexpr (MODE == FWD) {
+      float2 ga[16], gb[16];
+      load_gains(ga, 0);
+      lane_sync<NW>(group);
 #pragma unroll 1
-    for (int pass = 0; pass < 4; pass += 2) {
-      load_gains(gb, pass + 1);
-      round_b_pass(ga, pass);
-      if (pass == 0) load_gains(ga, 2);
-      round_b_pass(gb, pass + 1);
+      for (int pass = 0; pass < 4; pass += 2) {
+        load_gains(gb, pass + 1);
+        round_b_pass(ga, pass);
+        if (pass == 0) load_gains(ga, 2);
+        round_b_pass(gb, pass + 1);
+      }
+    } else {  // (the spectrum's registers leave no room to load gains a pass ahead)
+      lane_sync<NW>(group);
+#pragma unroll 1
+      for (int pass = 0; pass < 4; ++pass) {
+        float2 gg[16];
+        if constexpr (MODE == ADJOINT) load_gains(gg, pass);
+        round_b_pass(gg, pass);
+      }
     }
     lane_sync<NW>(group);
 #pragma unroll 1
-    for (int it = 0; it < 2; ++it) {
+    for (int it = 0; it < (MODE == SPECTRUM ? 0 : 2); ++it) {
       float2 v[32];
       float* dst = block(g, i + NW * it) + lane;
       read_row(ta + 64 * (i + NW * it), v);
@@ -546,54 +592,232 @@ __device__ __forceinline__ void col_lanes(float* ws, int begin, int end, const P
   }
 }
 
+// Backward columns of up to 256 rows, X and dY of a column in one pass: the spectrum of X waits on chip (in
+// registers up to 32 rows, else in tensor memory) while dY is transformed; the dG term (W X)(W dY)/L goes to X's
+// place in wsx, dY through gain and column bits to its own in wsd.  Against a pass over X that stores its spectrum
+// and a pass over dY that reads it back, the exchange is a third smaller.
+template <int Q>
+__device__ __forceinline__ void col_regs_bwd(float* wsx, float* wsd, int cols, const Params& P, uint32_t tmem, float* slots) {
+  constexpr int NR = 1 << Q, NP = NR / 2, m = R + Q;
+  constexpr int PER = 32 * (NR < 4 ? 4 : NR);
+  constexpr int RING = WARP_STAGE / PER > 3 ? 3 : WARP_STAGE / PER;  // blocks in flight: X, dY, X, ... in turn
+  const float2 sc = make_float2(P.scale, P.scale);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t ta = tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + 64 * (warp >> 2);
+  const int first = warp * gridDim.x + blockIdx.x, step = gridDim.x * (THREADS / 32), n = cols / 32;
+  float* stg = slots + warp * WARP_STAGE;
+  auto offset = [&](int w) { return (static_cast<long long>((32 * w) >> R) << m) + ((32 * w) & (TILE - 1)); };
+  int sw = first, sd = 0, sslot = 0;  // the next block to stage
+  auto stage = [&] {
+    if (sw < n) {
+      const float* b = (sd ? wsd : wsx) + offset(sw);
+      if constexpr (NR >= 4) {
+        stage_block<NR>(b, stg + sslot * PER, lane);
+      } else {
+        if (lane < 8 * NR)
+          cp_async16(tc::smem_u32(stg + sslot * PER) + 16 * lane, b + (static_cast<long long>(lane >> 3) << R) + 4 * (lane & 7));
+      }
+    }
+    fast::cp_async_commit();
+    sslot = sslot + 1 == RING ? 0 : sslot + 1;
+    sw += sd ? step : 0;
+    sd ^= 1;
+  };
+#pragma unroll
+  for (int k = 0; k < RING; ++k) stage();
+  int slot = 0;
+  auto take = [&](float2 (&v)[NP]) {  // the next staged block, its column bits done
+    asm volatile("cp.async.wait_group %0;" ::"n"(RING - 1) : "memory");
+    __syncwarp();
+    const float* b = stg + slot * PER + lane;
+#pragma unroll
+    for (int j = 0; j < NP; ++j) v[j] = make_float2(b[64 * j], b[64 * j + 32]);
+    __syncwarp();
+    stage();
+    slot = slot + 1 == RING ? 0 : slot + 1;
+#pragma unroll
+    for (int j = 0; j < NP; ++j) bf_in(v[j]);
+    fast::bfly_all<NP>(v);
+  };
+  constexpr int NG = NP < 16 ? NP : 16;  // pairs per batch of gains
+  for (int w = first; w < n; w += step) {
+    const long long o = offset(w) + lane;
+    const LaneFull<Q> gain(P, nullptr, ((32 * w) & (TILE - 1)) + lane);
+    float2 xh[NG];
+    float2 v[NP];
+    take(v);
+    if constexpr (NP > 16) {
+#pragma unroll
+      for (int q = 0; q < NP / 8; ++q) st_pairs<8>(ta + 16 * q, v + 8 * q);
+      fast::tmem_wait_st();
+    } else {
+#pragma unroll
+      for (int j = 0; j < NP; ++j) xh[j] = v[j];
+    }
+    take(v);
+#pragma unroll
+    for (int h = 0; h < NP; h += NG) {
+      if constexpr (NP > 16) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) ld_pairs<8>(ta + 2 * h + 16 * q, xh + 8 * q);
+        fast::tmem_wait_ld();
+      }
+      float2 gg[NG];
+#pragma unroll
+      for (int j = 0; j < NG; ++j) gg[j] = gain.rows2(2 * (h + j));
+#pragma unroll
+      for (int j = 0; j < NG; ++j) {
+        const float2 pr = mul2(mul2(xh[j], v[h + j]), sc);
+        __stcg(wsx + o + ((2 * (h + j)) << R), pr.x);
+        __stcg(wsx + o + ((2 * (h + j) + 1) << R), pr.y);
+      }
+#pragma unroll
+      for (int j = 0; j < NG; ++j) v[h + j] = mul2(v[h + j], mul2(gg[j], sc));
+    }
+#pragma unroll
+    for (int j = 0; j < NP; ++j) bf_in(v[j]);
+    fast::bfly_all<NP>(v);
+#pragma unroll
+    for (int j = 0; j < NP; ++j) {
+      __stcg(wsd + o + ((2 * j) << R), v[j].x);
+      __stcg(wsd + o + ((2 * j + 1) << R), v[j].y);
+    }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
+// 128 and 256 rows: NB = 2, 4 warps hold 32 columns, one block of 64 rows of X and of dY each.
+template <int Q>
+__device__ __forceinline__ void col_lanes_bwd(float* wsx, float* wsd, int begin, int end, const Params& P, uint32_t tmem,
+                                              float* slots) {
+  constexpr int m = R + Q, NB = 1 << (Q - 6), W = 32 / NB, WP = W / 2, GROUPS = THREADS / 32 / NB;
+  const float2 sc = make_float2(P.scale, P.scale);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quarter = warp & 3;
+  const int half = (warp >> 2) / NB, i = (warp >> 2) % NB, group = quarter + 4 * half;
+  // words of the lane: the spectrum of X, then dY
+  const uint32_t tx = tmem + (static_cast<uint32_t>(32 * quarter) << 16) + half * (128 * NB), td = tx + 64 * NB;
+  float* stg = slots + warp * WARP_STAGE;
+  auto offset = [&](int g) { return (static_cast<long long>((32 * g) >> R) << m) + ((32 * g) & (TILE - 1)); };
+  const long long own = static_cast<long long>(64 * i) << R;
+  if (begin + group < end) stage_block<64>(wsd + offset(begin + group) + own, stg, lane);
+  for (int g = begin + group; g < end; g += GROUPS) {
+    const long long o = offset(g) + lane;
+    const LaneFull<Q> gain(P, nullptr, ((32 * g) & (TILE - 1)) + lane);
+    auto rows64 = [&](float2 (&v)[32]) {
+#pragma unroll
+      for (int j = 0; j < 32; ++j) bf_in(v[j]);
+      bfly32<0>(v);
+    };
+    {
+      float2 v[32];
+      const float* src = wsx + o + own;
+#pragma unroll
+      for (int j = 0; j < 32; ++j) v[j] = make_float2(__ldcg(src + ((2 * j) << R)), __ldcg(src + ((2 * j + 1) << R)));
+      rows64(v);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) st_pairs<8>(tx + 64 * i + 16 * q, v + 8 * q);
+      fast::cp_async_wait_all();
+      __syncwarp();
+#pragma unroll
+      for (int j = 0; j < 32; ++j) v[j] = make_float2(stg[64 * j + lane], stg[64 * j + 32 + lane]);
+      __syncwarp();
+      if (g + GROUPS < end) stage_block<64>(wsd + offset(g + GROUPS) + own, stg, lane);
+      rows64(v);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) st_pairs<8>(td + 64 * i + 16 * q, v + 8 * q);
+    }
+    const int low0 = (64 / NB) * i;
+    auto across = [&](float2 (&v)[16]) {
+#pragma unroll
+      for (int h = WP; h < 16; h <<= 1)
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+          if ((k & h) == 0) bf2(v[k], v[k + h]);
+    };
+    float2 gg[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) gg[k] = gain.rows2(64 * (k / WP) + low0 + 2 * (k % WP));
+    lane_sync<NB>(group);
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {
+      const int low = low0 + W * pass;
+      float2 xh[16], v[16];
+#pragma unroll
+      for (int s = 0; s < NB; ++s) ld_pairs<WP>(tx + 64 * s + low, xh + WP * s);
+#pragma unroll
+      for (int s = 0; s < NB; ++s) ld_pairs<WP>(td + 64 * s + low, v + WP * s);
+      fast::tmem_wait_ld();
+      across(xh);
+      across(v);
+      float* xo = wsx + o + (static_cast<long long>(low) << R);
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        const float2 pr = mul2(mul2(xh[k], v[k]), sc);
+        __stcg(xo + ((64 * (k / WP) + 2 * (k % WP)) << R), pr.x);
+        __stcg(xo + ((64 * (k / WP) + 2 * (k % WP) + 1) << R), pr.y);
+      }
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[k] = mul2(v[k], mul2(gg[k], sc));
+      if (pass == 0) {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) gg[k] = gain.rows2(64 * (k / WP) + low0 + W + 2 * (k % WP));
+      }
+      across(v);
+#pragma unroll
+      for (int s = 0; s < NB; ++s) st_pairs<WP>(td + 64 * s + low, v + WP * s);
+    }
+    lane_sync<NB>(group);
+    {
+      float2 v[32];
+      float* dst = wsd + o + own;
+      read_row(td + 64 * i, v);
+      rows64(v);
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        __stcg(dst + ((2 * j) << R), v[j].x);
+        __stcg(dst + ((2 * j + 1) << R), v[j].y);
+      }
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------------------------
-// Columns.  A unit is W = 2^(14-Q) adjacent columns of all 2^Q rows of a plane, two slots; its element e (row
+// Columns, Q >= 10.  A unit is W = 2^(14-Q) adjacent columns of all 2^Q rows of a plane, two slots; its element e (row
 // e >> (14-Q), column e mod W) is word e, bit 4 XORed with bit 9.  A team's thread tt takes
 //   round A  the pairs at 2 tt + 512 i, i = 0..31 (word bits 9..13);
 //   round B  word bits 1, 2, 3, 9, 10 in the lane, 11..13 in the warp, 4..8 in the registers.
-// Word bit x is a row bit, and takes a butterfly, if x >= 14 - Q; Q <= 5 needs round A alone.
+// Word bit x is a row bit if x >= 14 - Q: ten of them in the registers of the two rounds, those below bit 4
+// (Q = 11, 12) across the lanes of round B by shuffles.
 constexpr int UNIT = 2 * TILE;
 template <int Q>
 struct Col {
+  static_assert(Q >= 10 && Q <= 12, "two rounds of five bits and at most two lane bits");
   static constexpr int W = 1 << (R + 1 - Q);
-  static constexpr int A0 = 5 - Q > 0 ? 5 - Q : 0;    // first row bit of round A's index
-  static constexpr int B0 = 10 - Q > 0 ? 10 - Q : 0;  // first row bit of round B's index
-  static constexpr bool TWO = Q > 5;
   // plane offset of unit word e; additive over disjoint bits
   __host__ __device__ static constexpr int off(int e) { return ((e >> (R + 1 - Q)) << R) + (e & (W - 1)); }
 };
 
-// Gains of a thread's pairs in the round that applies them: pair k sits at unit words e0 + STEP k and + 1.
+// Gains of a thread's round-B pairs: pair k sits at unit words e0 + 16 k and + 1.
 template <int Q>
 struct FullGain {
   const float* p;
   __device__ __forceinline__ FullGain(const Params& P, const float*, int col0, int e0)
       : p(static_cast<const float*>(P.g) + col0 + Col<Q>::off(e0)) {}
-  template <int STEP>
-  __device__ __forceinline__ float2 at(int k) const {
-    return __ldg(reinterpret_cast<const float2*>(p + Col<Q>::off(STEP * k)));
-  }
-  __device__ __forceinline__ float2 row(int j) const { return __ldg(reinterpret_cast<const float2*>(p + (j << R))); }
+  __device__ __forceinline__ float2 at(int k) const { return __ldg(reinterpret_cast<const float2*>(p + Col<Q>::off(16 * k))); }
 };
-// Separable log gains: G[n, c] = et[n] ec[c] from two tables that phase 1 builds (tab): the token table is
-// stored so that a column's rows are consecutive, et[(column >> cb) 2^Q + row].
 template <int Q>
-struct SepGain {
-  const float* et;
-  const float* ec;
-  int cb, c0, j0;
-  __device__ __forceinline__ SepGain(const Params& P, const float* tab, int col0, int e0)
-      : et(tab), ec(tab + (1ll << (P.m - P.cbits))), cb(P.cbits), c0(col0 + (e0 & (Col<Q>::W - 1))), j0(e0 >> (R + 1 - Q)) {}
-  template <int STEP>
-  __device__ __forceinline__ float2 at(int k) const {
-    const int e = STEP * k, c = c0 + (e & (Col<Q>::W - 1)), j = j0 + (e >> (R + 1 - Q)), ch = c & ((1 << cb) - 1);
-    const float t = et[(static_cast<long long>(c >> cb) << Q) + j];
-    return make_float2(t * ec[ch], t * ec[ch + 1]);
+struct SepGain {  // two channels of one token row range
+  const float* p;
+  float2 e;
+  __device__ __forceinline__ SepGain(const Params& P, const float* tab, int col0, int e0) {
+    const int c = col0 + (e0 & (Col<Q>::W - 1)), ch = c & ((1 << P.cbits) - 1);
+    const float* ec = tab + (1ll << (P.m - P.cbits));
+    p = tab + (static_cast<long long>(c >> P.cbits) << Q) + (e0 >> (R + 1 - Q));
+    e = make_float2(ec[ch], ec[ch + 1]);
   }
-  __device__ __forceinline__ float2 row(int j) const {
-    const int ch = c0 & ((1 << cb) - 1);
-    const float t = et[(static_cast<long long>(c0 >> cb) << Q) + j];
-    return make_float2(t * ec[ch], t * ec[ch + 1]);
+  __device__ __forceinline__ float2 at(int k) const {
+    const float t = p[(16 * k) >> (R + 1 - Q)];
+    return make_float2(t * e.x, t * e.y);
   }
 };
 
@@ -608,267 +832,477 @@ __device__ __forceinline__ void load_unit(const float* src, float* slot, int tt,
   cp_async_arrive(full);
 }
 
+// Butterfly over the row bit that lanes l and l ^ MASK differ in.
+template <int MASK>
+__device__ __forceinline__ void bfly_lanes(float2 (&v)[32]) {
+  const float2 sgn = (threadIdx.x & MASK) ? make_float2(-1.f, -1.f) : make_float2(1.f, 1.f);
+#pragma unroll
+  for (int k = 0; k < 32; ++k) {
+    const float2 p = make_float2(__shfl_xor_sync(0xffffffffu, v[k].x, MASK), __shfl_xor_sync(0xffffffffu, v[k].y, MASK));
+    v[k] = fast::fma2(v[k], sgn, p);
+  }
+}
+
 // Phase 2 of one unit: column bits, gain, column bits; the result to the workspace at `dst` (the unit's first
 // element).  `wait` is called before the slot is read, so that the first gains are on their way by then.
-template <int Q, class GainT, class Wait>
+template <int Q, class GainT, Mode MODE, class Wait>
 __device__ __forceinline__ void col_unit(float* slot, float* dst, const Params& P, const float* tab, int col0, int tt,
-                                         int team, const Wait& wait) {
+                                         int team, float* xdst, const Wait& wait) {
   using C = Col<Q>;
   const float2 sc = make_float2(P.scale, P.scale);
   const int l = tt & 31;
-  const int e0 = C::TWO ? 2 * (l & 7) + 512 * (l >> 3) + 2048 * (tt >> 5) : 2 * tt;
-  constexpr int STEP = C::TWO ? 16 : 512;
+  const int e0 = 2 * (l & 7) + 512 * (l >> 3) + 2048 * (tt >> 5);
   const GainT gain(P, tab, col0, e0);
   float2 gg[16];
+  if constexpr (MODE != SPECTRUM) {
 #pragma unroll
-  for (int k = 0; k < 16; ++k) gg[k] = gain.template at<STEP>(k);
+    for (int k = 0; k < 16; ++k) gg[k] = gain.at(k);
+  }
   wait();
   float2 v[32];
   const int a0 = 2 * tt, a1 = a0 ^ 16;
 #pragma unroll
   for (int i = 0; i < 32; ++i) v[i] = *reinterpret_cast<const float2*>(slot + (i & 1 ? a1 : a0) + 512 * i);
-  bfly32<C::A0>(v);
+  bfly32<0>(v);
   const int b0 = e0 ^ (((l >> 3) & 1) << 4), b1 = b0 ^ 16;  // round B: bit 4 is the registers' lowest
-  if constexpr (C::TWO) {
 #pragma unroll
-    for (int i = 0; i < 32; ++i) *reinterpret_cast<float2*>(slot + (i & 1 ? a1 : a0) + 512 * i) = v[i];
-    team_sync(team);
+  for (int i = 0; i < 32; ++i) *reinterpret_cast<float2*>(slot + (i & 1 ? a1 : a0) + 512 * i) = v[i];
+  team_sync(team);
 #pragma unroll
-    for (int k = 0; k < 32; ++k) v[k] = *reinterpret_cast<const float2*>(slot + (k & 1 ? b1 : b0) + 32 * (k >> 1));
-    bfly32<C::B0>(v);
-  }
+  for (int k = 0; k < 32; ++k) v[k] = *reinterpret_cast<const float2*>(slot + (k & 1 ? b1 : b0) + 32 * (k >> 1));
+  bfly32<0>(v);
+  if constexpr (Q >= 11) bfly_lanes<4>(v);
+  if constexpr (Q >= 12) bfly_lanes<2>(v);
+  if constexpr (MODE == SPECTRUM) {
+    float* o = dst + C::off(e0);
 #pragma unroll
-  for (int k = 0; k < 16; ++k) v[k] = mul2(v[k], mul2(gg[k], sc));
+    for (int k = 0; k < 32; ++k) __stcg(reinterpret_cast<float2*>(o + C::off(16 * k)), v[k]);
+  } else {
 #pragma unroll
-  for (int k = 0; k < 16; ++k) gg[k] = gain.template at<STEP>(k + 16);
+    for (int h = 0; h < 32; h += 16) {
+      if (h > 0) {
 #pragma unroll
-  for (int k = 0; k < 16; ++k) v[k + 16] = mul2(v[k + 16], mul2(gg[k], sc));
-  if constexpr (C::TWO) {
-    bfly32<C::B0>(v);
+        for (int k = 0; k < 16; ++k) gg[k] = gain.at(k + 16);
+      }
+      if constexpr (MODE == ADJOINT) {
+        float* xp = xdst + C::off(e0);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+          float2* x = reinterpret_cast<float2*>(xp + C::off(16 * (h + k)));
+          __stcg(x, mul2(mul2(__ldcg(x), v[h + k]), sc));
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 16; ++k) v[h + k] = mul2(v[h + k], mul2(gg[k], sc));
+    }
+    if constexpr (Q >= 12) bfly_lanes<2>(v);
+    if constexpr (Q >= 11) bfly_lanes<4>(v);
+    bfly32<0>(v);
 #pragma unroll
     for (int k = 0; k < 32; ++k) *reinterpret_cast<float2*>(slot + (k & 1 ? b1 : b0) + 32 * (k >> 1)) = v[k];
     team_sync(team);
 #pragma unroll
     for (int i = 0; i < 32; ++i) v[i] = *reinterpret_cast<const float2*>(slot + (i & 1 ? a1 : a0) + 512 * i);
-  }
-  bfly32<C::A0>(v);
-  float* o = dst + C::off(2 * tt);
+    bfly32<0>(v);
+    float* o = dst + C::off(2 * tt);
 #pragma unroll
-  for (int i = 0; i < 32; ++i) __stcg(reinterpret_cast<float2*>(o + C::off(512 * i)), v[i]);
+    for (int i = 0; i < 32; ++i) __stcg(reinterpret_cast<float2*>(o + C::off(512 * i)), v[i]);
+  }
 }
+
+// ---------------------------------------------------------------------------------------------
+// What the phases of one CTA share.
+struct Cta {
+  float* slots;
+  uint64_t *full_row, *full_pair;
+  uint64_t (*mma_done)[2];
+  volatile int* dead;
+  GridBarrier* bar;
+  uint32_t tmem;
+  int worker, t, team, tt;
+  unsigned row_seq, pair_seq, mma_seq;  // tiles taken from each ring so far
+};
+struct __align__(8) CtaShared {
+  uint64_t full_row[ROW_BARS], full_pair[PAIR_BARS], mma_done[WORKERS][2];
+  int flag, dead;
+  uint32_t tmem_slot;
+};
+__host__ __device__ constexpr bool uses_tmem(int dtype, int q) { return dtype == DT_BF16 || (q >= 6 && q <= 9); }
+
+// Before the launch wait: tensor memory, H_128, the barriers.
+template <int D, int Q>
+__device__ __forceinline__ Cta cta_begin(unsigned char* smem, CtaShared& sh, const Params& P) {
+  if constexpr (uses_tmem(D, Q)) {
+    if (threadIdx.x < 32) fast::tmem_alloc_512(&sh.tmem_slot);
+  }
+  if constexpr (D == DT_BF16) {
+    build_h(smem + SLOT_BYTES);
+    fence_async();
+  }
+  if (threadIdx.x == 0) {
+    sh.dead = 0;
+    for (int i = 0; i < ROW_BARS; ++i) tc::mbar_init(&sh.full_row[i], WT);
+    for (int i = 0; i < PAIR_BARS; ++i) tc::mbar_init(&sh.full_pair[i], 2 * WT);
+    for (int i = 0; i < WORKERS; ++i)
+      for (int k = 0; k < 2; ++k) tc::mbar_init(&sh.mma_done[i][k], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  fast::tmem_fence_before();
+  __syncthreads();
+  fast::tmem_fence_after();
+  return {reinterpret_cast<float*>(smem), sh.full_row, sh.full_pair, sh.mma_done, &sh.dead, P.bar,
+          uses_tmem(D, Q) ? sh.tmem_slot : 0u, static_cast<int>(threadIdx.x) / WT, static_cast<int>(threadIdx.x) % WT,
+          static_cast<int>(threadIdx.x) / (2 * WT), static_cast<int>(threadIdx.x) % (2 * WT), 0, 0, 0};
+}
+template <int D, int Q>
+__device__ __forceinline__ void cta_end(CtaShared& sh) {
+  if constexpr (uses_tmem(D, Q)) {
+    fast::tmem_fence_before();
+    __syncthreads();
+    fast::tmem_fence_after();
+    if (threadIdx.x < 32) fast::tmem_dealloc_512(sh.tmem_slot);
+  }
+}
+
+// Row bits of the CTA's n rows.  src(k, &p, &lim): row k's first element and how many are present; dst(k): its
+// workspace row; each(k): called by one thread per row.
+template <int D, class Src, class Dst, class Each>
+__device__ __forceinline__ void rows_in(Cta& c, int n, const Src& src, const Dst& dst, const Each& each) {
+  const int worker = c.worker, t = c.t;
+  if constexpr (D == DT_BF16) {
+    // the worker's i-th row (row worker + 4 i of the CTA's) is staged in its area i mod 3 and multiplied into its
+    // accumulator i mod 2
+    const int nw = (n - worker + WORKERS - 1) / WORKERS;
+    const uint32_t xs = tc::smem_u32(c.slots) + worker * (XSLOTS * TILE * 2);
+    const uint32_t sh = tc::smem_u32(c.slots) + SLOT_BYTES;
+    const uint32_t acc = c.tmem + 128u * worker;
+    auto load = [&](int i) {
+      if (i < nw) {
+        const void* p;
+        int lim;
+        src(worker + WORKERS * i, &p, &lim);
+        load_x_bf16(static_cast<const unsigned short*>(p), lim, xs + (i % XSLOTS) * (TILE * 2), t);
+      }
+      fast::cp_async_commit();
+    };
+    auto multiply = [&](int i) {  // a row that has been staged -> its accumulator
+      fence_async();
+      fast::tmem_fence_before();
+      worker_sync(worker);
+      if (t == 0) {
+        fast::tmem_fence_after();
+        mma_row(acc + 64u * (i & 1), sh, xs + (i % XSLOTS) * (TILE * 2));
+        tc::mma_commit(&c.mma_done[worker][(c.mma_seq + i) & 1]);
+      }
+    };
+    for (int i = 0; i < XSLOTS; ++i) load(i);
+    if (nw > 0) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(XSLOTS - 1) : "memory");
+      multiply(0);
+    }
+    for (int i = 0; i < nw; ++i) {
+      if (t == 0) each(worker + WORKERS * i);
+      if (i + 1 < nw) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(XSLOTS - 2) : "memory");
+        multiply(i + 1);
+      }
+      wait_bar(&c.mma_done[worker][(c.mma_seq + i) & 1], ((c.mma_seq + i) >> 1) & 1u, c.bar, c.dead);
+      __syncwarp();
+      fast::tmem_fence_after();
+      float2 v[32];
+      read_row(acc + 64u * (i & 1) + (static_cast<uint32_t>(32 * ((threadIdx.x >> 5) & 3)) << 16), v);
+      load(i + XSLOTS);
+#pragma unroll
+      for (int j = 0; j < 32; ++j) bf_in(v[j]);
+      bfly32<0>(v);
+      float* o = dst(worker + WORKERS * i) + t;
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        __stcg(o + 256 * j, v[j].x);
+        __stcg(o + 256 * j + 128, v[j].y);
+      }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    c.mma_seq += nw;
+    fast::tmem_fence_before();
+  } else {
+    auto load = [&](int k) {
+      const void* p;
+      int lim;
+      src(k, &p, &lim);
+      load_row(static_cast<const float*>(p), lim, c.slots + (c.row_seq + k) % SLOTS * TILE, t, &c.full_row[(c.row_seq + k) % ROW_BARS]);
+    };
+    for (int k = worker; k < SLOTS && k < n; k += WORKERS) load(k);
+    for (int k = worker; k < n; k += WORKERS) {
+      if (t == 0) each(k);
+      wait_full(c.full_row, c.row_seq + k, ROW_BARS, c.bar, c.dead);
+      row_in(c.slots + (c.row_seq + k) % SLOTS * TILE, dst(k), t, worker, [&] {
+        if (k + SLOTS < n) load(k + SLOTS);
+      });
+    }
+    c.row_seq += n;
+  }
+}
+
+// Row bits of the CTA's n workspace rows at wsr -> dst: loc(k, &e0, &lim) is row k's place in dst.
+template <int D, class Loc>
+__device__ __forceinline__ void rows_out(Cta& c, int n, const float* wsr, void* dst, const Loc& loc) {
+  auto load = [&](int k) {
+    load_row(wsr + (static_cast<long long>(k) << R), TILE, c.slots + (c.row_seq + k) % SLOTS * TILE, c.t,
+             &c.full_row[(c.row_seq + k) % ROW_BARS]);
+  };
+  for (int k = c.worker; k < SLOTS && k < n; k += WORKERS) load(k);
+  for (int k = c.worker; k < n; k += WORKERS) {
+    long long e0;
+    int lim;
+    loc(k, &e0, &lim);
+    wait_full(c.full_row, c.row_seq + k, ROW_BARS, c.bar, c.dead);
+    row_out<D>(c.slots + (c.row_seq + k) % SLOTS * TILE, dst, e0, lim, c.t, c.worker, [&] {
+      if (k + SLOTS < n) load(k + SLOTS);
+    });
+  }
+  c.row_seq += n;
+}
+
+// Column bits of nb planes of a workspace, all CTAs together.
+template <int Q, bool SEP, Mode MODE>
+__device__ __forceinline__ void columns(Cta& c, float* ws, int nb, const Params& P, const float* tab, float* xws = nullptr) {
+  constexpr int m = R + Q;
+  using LaneT = typename std::conditional<SEP, LaneSep<Q>, LaneFull<Q>>::type;
+  if constexpr (Q <= 6) {
+    col_regs<Q, LaneT>(ws, nb << R, P, tab, c.slots);
+  } else if constexpr (Q <= 9) {
+    int gb, ge;
+    share(static_cast<unsigned>(nb) << (R - 5), &gb, &ge);
+    col_lanes<Q, LaneT, MODE>(ws, gb, ge, P, tab, c.tmem, c.slots, xws);
+    fast::tmem_fence_before();
+  } else {
+    using GainT = typename std::conditional<SEP, SepGain<Q>, FullGain<Q>>::type;
+    constexpr int UB = Q - 1;  // log2 of the units of a plane
+    int ub, ue;
+    share(static_cast<unsigned>(nb) << UB, &ub, &ue);
+    const int nu = ue - ub;
+    auto offset = [&](int k, int* col0) {
+      const int u = ub + k;
+      *col0 = (u & ((1 << UB) - 1)) << (R + 1 - Q);
+      return (static_cast<long long>(u >> UB) << m) + *col0;
+    };
+    auto load = [&](int k) {
+      int col0;
+      const long long o = offset(k, &col0);
+      load_unit<Q>(ws + o, c.slots + (c.pair_seq + k) % PAIRS * UNIT, c.tt, &c.full_pair[(c.pair_seq + k) % PAIR_BARS]);
+    };
+    for (int k = c.team; k < PAIRS && k < nu; k += 2) load(k);
+    for (int k = c.team; k < nu; k += 2) {
+      int col0;
+      const long long o = offset(k, &col0);
+      col_unit<Q, GainT, MODE>(c.slots + (c.pair_seq + k) % PAIRS * UNIT, ws + o, P, tab, col0, c.tt, c.team, xws + o,
+                               [&] { wait_full(c.full_pair, c.pair_seq + k, PAIR_BARS, c.bar, c.dead); });
+      if (k + PAIRS < nu) {
+        team_sync(c.team);
+        load(k + PAIRS);
+      }
+    }
+    c.pair_seq += nu;
+    if constexpr (MODE == SPECTRUM) __syncthreads();  // the next pass refills the slots
+  }
+}
+
+// Backward columns of nb planes: the dG terms over wsx, dY through gain and back over wsd.
+template <int Q>
+__device__ __forceinline__ void columns_bwd(Cta& c, float* wsx, float* wsd, int nb, const Params& P) {
+  if constexpr (Q <= 6) {
+    col_regs_bwd<Q>(wsx, wsd, nb << R, P, c.tmem, c.slots);
+    fast::tmem_fence_before();
+  } else if constexpr (Q <= 8) {
+    int gb, ge;
+    share(static_cast<unsigned>(nb) << (R - 5), &gb, &ge);
+    col_lanes_bwd<Q>(wsx, wsd, gb, ge, P, c.tmem, c.slots);
+    fast::tmem_fence_before();
+  } else {
+    columns<Q, false, SPECTRUM>(c, wsx, nb, P, nullptr);
+    columns<Q, false, ADJOINT>(c, wsd, nb, P, nullptr, wsx);
+  }
+}
+
+// This CTA's share of G, fetched into L2 over phase 1's rows.
+struct GainPrefetch {
+  const char* g;
+  long long begin, end;  // 16-byte chunks
+  __device__ __forceinline__ GainPrefetch(const void* p, int m) : g(static_cast<const char*>(p)) {
+    const long long chunks = (4ll << m) >> 4;
+    begin = chunks * blockIdx.x / gridDim.x;
+    end = chunks * (blockIdx.x + 1) / gridDim.x;
+  }
+  __device__ __forceinline__ void operator()(int k, int n) const {  // piece k of n
+    const long long step = (end - begin + n - 1) / n, c0 = begin + step * k, c1 = min(c0 + step, end);
+    if (c1 > c0)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(g + (c0 << 4)), "r"(static_cast<unsigned>((c1 - c0) << 4)) : "memory");
+  }
+};
+// (planes that fill L2 by themselves read G from HBM in phase 2: a prefetch would push the workspace out)
+__host__ __device__ constexpr bool prefetches_gains(int q) { return q <= 10; }
 
 // ---------------------------------------------------------------------------------------------
 // Forward kernel: persistent grid (one CTA per SM, all resident), plane groups of P.gp planes.
 template <int D, int Q, bool SEP>
 __global__ void __launch_bounds__(THREADS, 1) k_forward_fast(Params P) {
   extern __shared__ __align__(1024) unsigned char tri_smem[];
-  __shared__ uint64_t full_row[ROW_BARS], full_pair[PAIR_BARS], mma_done[WORKERS][2];
-  __shared__ int flag, dead;
-  __shared__ uint32_t tmem_slot;
+  __shared__ CtaShared sh;
   constexpr int m = R + Q;
-  constexpr bool MMA = D == DT_BF16;
-  constexpr bool TMEM = MMA || (Q >= 7 && Q <= 9);
-  float* slots = reinterpret_cast<float*>(tri_smem);
-  const int worker = threadIdx.x / WT, t = threadIdx.x % WT;
-  const int team = threadIdx.x / (2 * WT), tt = threadIdx.x % (2 * WT);
+  constexpr int ES = D == DT_BF16 ? 2 : 4;
   float* ws = static_cast<float*>(P.ws);
-  const float* tab = ws + (static_cast<long long>(P.gp) << m);
-  if constexpr (TMEM) {
-    if (threadIdx.x < 32) fast::tmem_alloc_512(&tmem_slot);
-  }
-  if constexpr (MMA) {
-    build_h(tri_smem + SLOT_BYTES);
-    fence_async();
-  }
-  if (threadIdx.x == 0) {
-    dead = 0;
-    for (int i = 0; i < ROW_BARS; ++i) tc::mbar_init(&full_row[i], WT);
-    for (int i = 0; i < PAIR_BARS; ++i) tc::mbar_init(&full_pair[i], 2 * WT);
-    for (int i = 0; i < WORKERS; ++i)
-      for (int k = 0; k < 2; ++k) tc::mbar_init(&mma_done[i][k], 1);
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
+  float* tab = ws + (static_cast<long long>(P.gp) << m);
   {
     int rb, re;
     share(static_cast<unsigned>(min(static_cast<long long>(P.gp), P.B)) << Q, &rb, &re);
     fast::l2_prefetch_first_rows<D, R, Q>(P.x, rb, re, P.lv);
   }
-  fast::tmem_fence_before();
-  __syncthreads();
-  fast::tmem_fence_after();
+  Cta c = cta_begin<D, Q>(tri_smem, sh, P);
   // tensor memory is allocated before the wait: the previous kernel's CTA on this SM has left
   pdl_wait();
-  GridSync gsync(P.bar, &flag);
-  // this CTA's share of G, fetched into L2 over phase 1's first rows
-  const long long g_chunks = (4ll << m) >> 4;
-  const long long g_begin = g_chunks * blockIdx.x / gridDim.x, g_end = g_chunks * (blockIdx.x + 1) / gridDim.x;
-  unsigned row_seq = 0, pair_seq = 0, mma_seq = 0;  // tiles taken by earlier phases
+  GridSync gsync(P.bar, &sh.flag);
+  const GainPrefetch prefetch(P.g, m);
+  if constexpr (SEP) {  // the gain tables, part of the first phase 1
+    const long long n_t = 1ll << (m - P.cbits), n_tab = n_t + (1ll << P.cbits);
+    for (long long i = static_cast<long long>(blockIdx.x) * THREADS + threadIdx.x; i < n_tab;
+         i += static_cast<long long>(gridDim.x) * THREADS)
+      tab[i] = expf(i < n_t ? P.gt[fast::sep_token_of<R, Q>(i, P.cbits)] : P.gc[i - n_t]);
+  }
   for (long long b0 = 0; b0 < P.B; b0 += P.gp) {
     const int nb = static_cast<int>(min(static_cast<long long>(P.gp), P.B - b0));
     int rb, re;
     share(static_cast<unsigned>(nb) << Q, &rb, &re);
     const int n = re - rb;
     // phase 1: X -> workspace, row bits
-    if constexpr (SEP) {
-      if (b0 == 0) {  // once: the gain tables
-        float* tb = ws + (static_cast<long long>(P.gp) << m);
-        const long long n_t = 1ll << (m - P.cbits), n_tab = n_t + (1ll << P.cbits);
-        for (long long i = static_cast<long long>(blockIdx.x) * THREADS + threadIdx.x; i < n_tab;
-             i += static_cast<long long>(gridDim.x) * THREADS)
-          tb[i] = expf(i < n_t ? P.gt[fast::sep_token_of<R, Q>(i, P.cbits)] : P.gc[i - n_t]);
-      }
-    }
-    const int g_step = n > 0 ? static_cast<int>((g_end - g_begin + n - 1) / n) : 0;
-    auto prefetch_g = [&](int k) {  // one thread per row
-      if (SEP || b0 != 0) return;
-      const long long c0 = g_begin + static_cast<long long>(g_step) * k, c1 = min(c0 + g_step, g_end);
-      if (c1 > c0)
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(static_cast<const char*>(P.g) + (c0 << 4)),
-                     "r"(static_cast<unsigned>((c1 - c0) << 4)) : "memory");
-    };
-    if constexpr (MMA) {
-      // the worker's i-th row (row worker + 4 i of the CTA's) is staged in its area i mod 3 and multiplied into
-      // its accumulator i mod 2
-      const int nw = (n - worker + WORKERS - 1) / WORKERS;
-      const uint32_t xs = tc::smem_u32(tri_smem) + worker * (XSLOTS * TILE * 2);
-      const uint32_t sh = tc::smem_u32(tri_smem) + SLOT_BYTES;
-      const uint32_t acc = tmem_slot + 128u * worker;
-      auto load = [&](int i) {
-        if (i < nw) {
+    rows_in<D>(
+        c, n,
+        [&](int k, const void** p, int* lim) {
           long long e0;
-          int lim;
-          fast::row_loc<R, Q>(b0, rb + worker + WORKERS * i, P.lv, &e0, &lim);
-          load_x_bf16(static_cast<const unsigned short*>(P.x) + e0, lim, xs + (i % XSLOTS) * (TILE * 2), t);
-        }
-        fast::cp_async_commit();
-      };
-      // staged row i (at most `pending` later ones still in flight) -> its accumulator
-      auto multiply = [&](int i) {
-        fence_async();
-        fast::tmem_fence_before();
-        worker_sync(worker);
-        if (t == 0) {
-          fast::tmem_fence_after();
-          mma_row(acc + 64u * (i & 1), sh, xs + (i % XSLOTS) * (TILE * 2));
-          tc::mma_commit(&mma_done[worker][(mma_seq + i) & 1]);
-        }
-      };
-      for (int i = 0; i < XSLOTS; ++i) load(i);
-      if (nw > 0) {
-        asm volatile("cp.async.wait_group %0;" ::"n"(XSLOTS - 1) : "memory");
-        multiply(0);
-      }
-      for (int i = 0; i < nw; ++i) {
-        if (t == 0) prefetch_g(worker + WORKERS * i);
-        if (i + 1 < nw) {
-          asm volatile("cp.async.wait_group %0;" ::"n"(XSLOTS - 2) : "memory");
-          multiply(i + 1);
-        }
-        wait_bar(&mma_done[worker][(mma_seq + i) & 1], ((mma_seq + i) >> 1) & 1u, P.bar, &dead);
-        __syncwarp();
-        fast::tmem_fence_after();
-        float2 v[32];
-        read_row(acc + 64u * (i & 1) + (static_cast<uint32_t>(32 * ((threadIdx.x >> 5) & 3)) << 16), v);
-        load(i + XSLOTS);
-#pragma unroll
-        for (int j = 0; j < 32; ++j) bf_in(v[j]);
-        bfly32<0>(v);
-        float* dst = ws + (static_cast<long long>(rb + worker + WORKERS * i) << R) + t;
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          __stcg(dst + 256 * j, v[j].x);
-          __stcg(dst + 256 * j + 128, v[j].y);
-        }
-      }
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-      mma_seq += nw > 0 ? nw : 0;
-      fast::tmem_fence_before();
-    } else {
-      auto load = [&](int k) {
-        long long e0;
-        int lim;
-        fast::row_loc<R, Q>(b0, rb + k, P.lv, &e0, &lim);
-        load_row(static_cast<const float*>(P.x) + e0, lim, slots + (row_seq + k) % SLOTS * TILE, t, &full_row[(row_seq + k) % ROW_BARS]);
-      };
-      for (int k = worker; k < SLOTS && k < n; k += WORKERS) load(k);
-      for (int k = worker; k < n; k += WORKERS) {
-        if (t == 0) prefetch_g(k);
-        wait_full(full_row, row_seq + k, ROW_BARS, P.bar, &dead);
-        row_in(slots + (row_seq + k) % SLOTS * TILE, ws + (static_cast<long long>(rb + k) << R), t, worker, [&] {
-          if (k + SLOTS < n) load(k + SLOTS);
+          fast::row_loc<R, Q>(b0, rb + k, P.lv, &e0, lim);
+          *p = static_cast<const char*>(P.x) + e0 * ES;
+        },
+        [&](int k) { return ws + (static_cast<long long>(rb + k) << R); },
+        [&](int k) {
+          if (!SEP && prefetches_gains(Q) && b0 == 0) prefetch(k, n);
         });
-      }
-      row_seq += n;
-    }
     if (!gsync()) break;
     // phase 2: columns
-    {
-      using LaneT = typename std::conditional<SEP, LaneSep<Q>, LaneFull<Q>>::type;
-      if constexpr (Q <= 6) {
-        col_regs<Q, LaneT>(ws, nb << R, P, tab, slots);
-      } else if constexpr (Q <= 9) {
-        int gb, ge;
-        share(static_cast<unsigned>(nb) << (R - 5), &gb, &ge);
-        col_lanes<Q, LaneT>(ws, gb, ge, P, tab, tmem_slot, slots);
-        fast::tmem_fence_before();
-      } else {
-        using GainT = typename std::conditional<SEP, SepGain<Q>, FullGain<Q>>::type;
-        constexpr int UB = Q - 1;  // log2 of the units of a plane
-        int ub, ue;
-        share(static_cast<unsigned>(nb) << UB, &ub, &ue);
-        const int nu = ue - ub;
-        auto base = [&](int k, int* col0) {
-          const int u = ub + k, c = (u & ((1 << UB) - 1)) << (R + 1 - Q);
-          *col0 = c;
-          return ws + (static_cast<long long>(u >> UB) << m) + c;
-        };
-        auto load = [&](int k) {
-          int c;
-          const float* src = base(k, &c);
-          load_unit<Q>(src, slots + (pair_seq + k) % PAIRS * UNIT, tt, &full_pair[(pair_seq + k) % PAIR_BARS]);
-        };
-        for (int k = team; k < PAIRS && k < nu; k += 2) load(k);
-        for (int k = team; k < nu; k += 2) {
-          int col0;
-          float* dst = base(k, &col0);
-          col_unit<Q, GainT>(slots + (pair_seq + k) % PAIRS * UNIT, dst, P, tab, col0, tt, team,
-                             [&] { wait_full(full_pair, pair_seq + k, PAIR_BARS, P.bar, &dead); });
-          if (k + PAIRS < nu) {
-            team_sync(team);
-            load(k + PAIRS);
-          }
-        }
-        pair_seq += nu;
-      }
-    }
+    columns<Q, SEP, FWD>(c, ws, nb, P, tab);
     if (!gsync()) break;
     // phase 3: workspace -> Y, row bits
-    {
-      auto load = [&](int k) {
-        load_row(ws + (static_cast<long long>(rb + k) << R), TILE, slots + (row_seq + k) % SLOTS * TILE, t,
-                 &full_row[(row_seq + k) % ROW_BARS]);
-      };
-      for (int k = worker; k < SLOTS && k < n; k += WORKERS) load(k);
-      for (int k = worker; k < n; k += WORKERS) {
-        long long e0;
-        int lim;
-        fast::row_loc<R, Q>(b0, rb + k, P.lv, &e0, &lim);
-        wait_full(full_row, row_seq + k, ROW_BARS, P.bar, &dead);
-        row_out<D>(slots + (row_seq + k) % SLOTS * TILE, P.y, e0, lim, t, worker, [&] {
-          if (k + SLOTS < n) load(k + SLOTS);
-        });
-      }
-      row_seq += n;
-    }
+    rows_out<D>(c, n, ws + (static_cast<long long>(rb) << R), P.y,
+                [&](int k, long long* e0, int* lim) { fast::row_loc<R, Q>(b0, rb + k, P.lv, e0, lim); });
     if (b0 + P.gp < P.B && !gsync()) break;
   }
   pdl_trigger();
-  if constexpr (TMEM) {
-    fast::tmem_fence_before();
-    __syncthreads();
-    fast::tmem_fence_after();
-    if (threadIdx.x < 32) fast::tmem_dealloc_512(tmem_slot);
+  cta_end<D, Q>(sh);
+}
+
+// Backward kernel (planes of 2^14 .. 2^23 elements).  Against the previous one (8 warps, one column a thread or two passes
+// through tensor memory, dG summed plane after plane), forward and backward together: [16, 8192, 256] bf16 465 -> 379 us,
+// [8, 4096, 256] bf16 118 -> 91, [1, 65536, 128] bf16 186 -> 148, [4, 16384, 256] bf16 335 -> 243, [32, 1024, 64] bf16
+// 36.3 -> 32.5.  Per group of four 2^21-element planes now: phase 1 18 us, columns 22, rows out 9, dG 7, barriers 5; its
+// workspaces (64 MiB) and the streamed X, dY, dX do not fit L2 together (700 MB of HBM traffic a call against 218 MB),
+// and smaller groups lose more to phases than they save (48 MiB 437 us, 32 MiB 461).
+// Per group of planes the same three phases over X and dY
+// together,
+//   phase 1  rows of X and dY                                            X, dY -> wsx, wsd
+//   phase 2  columns: the spectrum of X in place, then dY through gain and back, the products
+//            (W X)(W dY)/L replacing the spectrum                        wsx, wsd -> wsx, wsd
+//   phase 3  rows of wsd -> dX; then dG at this CTA's positions: dG (0 for the first group) plus the
+//            group's products in ascending b, so that dG is summed over b = 0, 1, ..., B-1 in that order.
+// dG at plane positions [lb, le) (multiples of 4), NPOS positions of NPL planes loaded at a time: loaded one plane
+// after another the sum was bound by the latency of its loads (14 us instead of 7 for four 8 MiB planes).
+template <int NPOS, int NPL>
+__device__ __forceinline__ void dg_sum(float* dg, const float* wsx, int m, int nb, bool first, long long lb, long long le) {
+  for (long long l0 = lb + 4 * threadIdx.x; l0 < le; l0 += 4 * THREADS * NPOS) {
+    float4 acc[NPOS], p[NPOS][NPL];
+#pragma unroll
+    for (int i = 0; i < NPOS; ++i) {
+      const long long l = l0 + 4 * THREADS * i;
+      acc[i] = first || l >= le ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldcg(reinterpret_cast<const float4*>(dg + l));
+    }
+    for (int b = 0; b < nb; b += NPL) {
+#pragma unroll
+      for (int i = 0; i < NPOS; ++i)
+#pragma unroll
+        for (int k = 0; k < NPL; ++k) {
+          const long long l = l0 + 4 * THREADS * i;
+          if (l < le && b + k < nb) p[i][k] = __ldcg(reinterpret_cast<const float4*>(wsx + (static_cast<long long>(b + k) << m) + l));
+        }
+#pragma unroll
+      for (int i = 0; i < NPOS; ++i)
+#pragma unroll
+        for (int k = 0; k < NPL; ++k)
+          if (b + k < nb) {
+            acc[i].x += p[i][k].x;
+            acc[i].y += p[i][k].y;
+            acc[i].z += p[i][k].z;
+            acc[i].w += p[i][k].w;
+          }
+    }
+#pragma unroll
+    for (int i = 0; i < NPOS; ++i) {
+      const long long l = l0 + 4 * THREADS * i;
+      if (l < le) __stcg(reinterpret_cast<float4*>(dg + l), acc[i]);
+    }
   }
+}
+// (four loads in flight a thread: eight made the phases around it spill registers)
+__device__ __forceinline__ void dg_reduce(float* dg, const float* wsx, int m, int nb, bool first, long long lb, long long le) {
+  if (nb == 1) dg_sum<4, 1>(dg, wsx, m, nb, first, lb, le);
+  else dg_sum<1, 4>(dg, wsx, m, nb, first, lb, le);
+}
+template <int D, int Q>
+__global__ void __launch_bounds__(THREADS, 1) k_backward_fast(Params P) {
+  extern __shared__ __align__(1024) unsigned char tri_smem[];
+  __shared__ CtaShared sh;
+  constexpr int m = R + Q;
+  constexpr int ES = D == DT_BF16 ? 2 : 4;
+  float* wsx = static_cast<float*>(P.ws);
+  float* wsd = wsx + (static_cast<long long>(P.gp) << m);
+  Cta c = cta_begin<D, Q>(tri_smem, sh, P);
+  pdl_wait();
+  GridSync gsync(P.bar, &sh.flag);
+  const GainPrefetch prefetch(P.g, m);
+  const long long L = 1ll << m;
+  const long long lb = ((L >> 2) * blockIdx.x / gridDim.x) << 2, le = ((L >> 2) * (blockIdx.x + 1) / gridDim.x) << 2;
+  for (long long b0 = 0; b0 < P.B; b0 += P.gp) {
+    const int nb = static_cast<int>(min(static_cast<long long>(P.gp), P.B - b0));
+    const int rows = nb << Q;
+    {
+      int ub, ue;
+      share(2u * static_cast<unsigned>(rows), &ub, &ue);
+      const int n = ue - ub;
+      rows_in<D>(
+          c, n,
+          [&](int k, const void** p, int* lim) {
+            const int u = ub + k;
+            long long e0;
+            fast::row_loc<R, Q>(b0, u < rows ? u : u - rows, P.lv, &e0, lim);
+            *p = static_cast<const char*>(u < rows ? P.x : P.dy) + e0 * ES;
+          },
+          [&](int k) {
+            const int u = ub + k;
+            return u < rows ? wsx + (static_cast<long long>(u) << R) : wsd + (static_cast<long long>(u - rows) << R);
+          },
+          [&](int k) {
+            if (b0 == 0) prefetch(k, n);
+          });
+    }
+    if (!gsync()) break;
+    columns_bwd<Q>(c, wsx, wsd, nb, P);
+    if (!gsync()) break;
+    int rb, re;
+    share(static_cast<unsigned>(rows), &rb, &re);
+    rows_out<D>(c, re - rb, wsd + (static_cast<long long>(rb) << R), P.dx,
+                [&](int k, long long* e0, int* lim) { fast::row_loc<R, Q>(b0, rb + k, P.lv, e0, lim); });
+    dg_reduce(static_cast<float*>(P.dg), wsx, m, nb, b0 == 0, lb, le);
+    if (b0 + P.gp < P.B && !gsync()) break;
+  }
+  pdl_trigger();
+  cta_end<D, Q>(sh);
 }
 
 }  // namespace tri
