@@ -7,23 +7,23 @@
 //   phase 3  every row: its 13 bits again                               workspace -> Y
 // with the bounded device-wide barrier between phases.  The workspace is in natural order.
 //
-// One CTA of 16 warps per SM, 64 elements a thread (128 registers).  A worker of 128 threads holds a row,
-// a team of two workers 2^(14-Q) adjacent columns; a ring of shared-memory slots keeps the next tiles in
-// flight, so that loads, butterflies and stores of different tiles overlap.
+// One CTA of 16 warps per SM, 64 elements a thread (128 registers).  A worker of 128 threads holds a row; a ring of
+// shared-memory slots keeps the next rows in flight, so that loads, butterflies and stores of different rows overlap.
 //   rows of bf16 X  the 7 low bits on the tensor cores: D[i, n] = sum_k H_128[i, k] x[128 n + k] (M = 128,
 //            N = 64, K = 128; bf16 times +-1 is exact, fp32 accumulation), then lane i of the worker reads its
 //            64 values n from tensor memory and runs the other 6 bits in registers: no exchange at all;
 //   other rows  two register rounds with one exchange inside the slot: A on bits {0, 1, 9..12} (16-byte
 //            vectors), B on bits {3..8} and, by one shuffle stage, bit 2;
-//   columns  rounds of five bits each, in place in the slot.
+//   columns  a warp lane is a column (a warp reads and writes whole row segments): up to 64 rows in a thread's registers,
+//            taller columns in that lane's tensor memory, which the warps of a lane quarter share.
 // Slots are XOR-swizzled so that every access is conflict-free.
 //
 // What bounds it: the fp32 workspace crosses between SMs through L2 twice (32 MiB each way at 2^23 elements;
 // measured without arithmetic: 4.4 us to write it, 5.9 to read and write it by columns, 1.8 to read it back,
 // 1.4 per barrier), and within an SM the shared-memory data path (one 128-byte wavefront a cycle) more than the
 // additions.  Measured against the previous kernel (8 warps, 128 elements a thread, columns read straight from
-// L2): [32, 4096, 64] f32 40.6 -> 32.9 us, [1, 4096, 64] bf16 11.6 -> 9.7, [1, 65536, 128] bf16 41.9 -> 39.7, with
-// log gains 39.2 -> 37.9, [1, 32768, 128] bf16 28.4 -> 27.1, [8, 4096, 256] f32 42.6 -> 36.3; of that the tensor-core
+// L2): [32, 4096, 64] f32 40.6 -> 32.9 us, [1, 4096, 64] bf16 11.6 -> 9.7, [1, 65536, 128] bf16 41.9 -> 38.0, with
+// log gains 39.2 -> 35.5, [1, 32768, 128] bf16 28.4 -> 27.1, [8, 4096, 256] f32 42.6 -> 36.3; of that the tensor-core
 // rows took phase 1 of the 2^23-element plane from 13.5 to 8.7 us.
 #pragma once
 
@@ -43,8 +43,7 @@ constexpr int WORKERS = 4;
 constexpr int WT = 128;              // threads per worker
 constexpr int R = 13;                // row bits
 constexpr int TILE = 1 << R;         // elements per row
-constexpr int SLOTS = 6;             // ring of rows; the column ring is three pairs of slots
-constexpr int PAIRS = SLOTS / 2;
+constexpr int SLOTS = 6;             // ring of rows
 constexpr int XSLOTS = 3;            // bf16 X rows (16 KiB) staged per worker
 constexpr int H_BYTES = 128 * 128 * 2;  // H_128 in bf16, the tensor cores' A operand
 constexpr int SLOT_BYTES = SLOTS * TILE * 4;
@@ -53,16 +52,12 @@ static_assert(WORKERS * XSLOTS * TILE * 2 <= SLOT_BYTES, "the X staging areas sh
 template <int D>
 constexpr size_t smem_bytes() { return SLOT_BYTES + (D == DT_BF16 ? H_BYTES : 0); }
 
-// Mbarriers of the rings: two per slot, taken in turn, so that all uses of one barrier belong to one
-// worker or team (12 is a multiple of four workers, 6 of two teams) and no wait can start two phases ahead.
+// Mbarriers of the ring: two per slot, taken in turn, so that all uses of one barrier belong to one worker (12 is a
+// multiple of four workers) and no wait can start two phases ahead.
 constexpr int ROW_BARS = 2 * SLOTS;
-constexpr int PAIR_BARS = 2 * PAIRS;
 
 __device__ __forceinline__ void worker_sync(int worker) {
   asm volatile("bar.sync %0, %1;" ::"r"(worker + 1), "r"(WT) : "memory");
-}
-__device__ __forceinline__ void team_sync(int team) {
-  asm volatile("bar.sync %0, %1;" ::"r"(team + 5), "r"(2 * WT) : "memory");
 }
 __device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
@@ -302,8 +297,7 @@ __device__ __forceinline__ void row_out(float* slot, void* dst, long long e0, in
 }
 
 // ---------------------------------------------------------------------------------------------
-// Columns, Q <= 9: a warp lane is a column (a warp reads and writes 128-byte row segments) and a column's
-// rows meet in that lane's tensor memory, so nothing goes through shared memory.
+// Columns.
 // Gains of one column: row(j), and rows2(j) = rows j and j + 1 (j even).
 template <int Q>
 struct LaneFull {
@@ -423,20 +417,30 @@ __device__ __forceinline__ void col_regs(float* ws, int cols, const Params& P, c
 // at the same positions of xws, by the dG term (W X)(W dY)/L.  Both take the same columns in the same thread.
 enum Mode { FWD, SPECTRUM, ADJOINT };
 
-// Columns of 128, 256 and 512 rows: NW warps of a tensor-memory lane quarter hold 32 columns, two blocks of 64
-// rows of each per warp.  All four warps of a quarter run on one sub-partition of the SM, so columns are
-// given to as few warps as tensor memory (512 words a lane) allows: the groups then drift apart and one
-// group's loads overlap another's butterflies.
+// Columns of 128 rows and up.  NW warps of a tensor-memory lane quarter hold a group of columns, 64 NB rows of each (up to
+// 512, bits 0..8 of the row), two blocks of 64 rows per warp.  All four warps of a quarter run on one sub-partition of the
+// SM, so columns are given to as few warps as tensor memory (512 words a lane) allows: the groups then drift apart and
+// one group's loads overlap another's butterflies.
 //   round A  blocks of 64 rows, bits 0..5: workspace -> registers -> tensor memory (the second block staged
 //            in shared memory meanwhile);
 //   round B  bits 6.. across the NB blocks, 32 values a pass, each pass's gains loaded a pass ahead;
 //   round C  blocks of 64 rows, bits 0..5 again -> workspace.
+// Taller columns (Q >= 10) are 16 to a group: the upper half of the lanes holds row bit 9, whose butterfly is a shuffle
+// in round B.  For Q = 11 and 12 the NQ = 2 or 4 quarters of a set hold row bits 10 (and 11) of the same columns: in round
+// B the warps at the same place of their quarters trade values through shared memory, each then holding all NQ of 16 / NQ
+// row pairs, and trade them back after the gain.  Against units of 2^14 elements in shared memory (8 columns of 1024 or 2048
+// rows, 4 of 4096: 32- and 16-byte row segments, each a whole wavefront of the SM's data path): 2^23 elements 39.6 -> 38.0 us
+// (log gains 37.9 -> 35.5, backward included 148 -> 132), 2^24 116 -> 101, 2^25 526 -> 222 (generic engine: 967).
 template <int Q>
 struct Lane {
-  static constexpr int NB = 1 << (Q - 6);           // blocks of 64 rows
-  static constexpr int NW = NB / 2;                 // warps per group of 32 columns
-  static constexpr int GROUPS = THREADS / 32 / NW;  // groups a CTA works on at a time
-  static constexpr int W = 32 / NB;                 // rows of each block per pass of round B: four passes
+  static constexpr bool TALL = Q >= 10;
+  static constexpr int NB = TALL ? 8 : 1 << (Q - 6);  // blocks of 64 rows
+  static constexpr int NW = NB / 2;                   // warps per group
+  static constexpr int NQ = Q <= 10 ? 1 : 1 << (Q - 10);        // quarters per set
+  static constexpr int GROUPS = THREADS / 32 / NW / NQ;         // groups a CTA works on at a time
+  static constexpr int W = 32 / NB;                   // rows of each block per pass of round B: four passes
+  static constexpr int COLS = TALL ? 16 : 32;         // columns per group
+  static constexpr int LOG_GROUPS = TALL ? R - 4 : R - 5;       // log2 of the groups of a plane
 };
 template <int NW>
 __device__ __forceinline__ void lane_sync(int group) {
@@ -470,19 +474,33 @@ template <int Q, class GainT, Mode MODE = FWD>
 __device__ __forceinline__ void col_lanes(float* ws, int begin, int end, const Params& P, const float* tab, uint32_t tmem,
                                           float* slots, float* xws = nullptr) {
   using C = Lane<Q>;
-  constexpr int m = R + Q, NB = C::NB, NW = C::NW, W = C::W, WP = W / 2;
+  constexpr int m = R + Q, NB = C::NB, NW = C::NW, W = C::W, WP = W / 2, NQ = C::NQ, COLS = C::COLS;
+  static_assert(MODE == FWD || NQ == 1, "the backward modes: Q <= 10");
   const float2 sc = make_float2(P.scale, P.scale);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quarter = warp & 3;
   const int half = (warp >> 2) / NW, i = (warp >> 2) % NW;  // warps of a group share a quarter
-  const int group = quarter + 4 * half;
+  const int bar = quarter + 4 * half, group = bar / NQ, sub = quarter % NQ;  // this warp's quarter of the set
   const uint32_t ta = tmem + (static_cast<uint32_t>(32 * quarter) << 16) + half * (64 * NB);
   float* stg = slots + warp * WARP_STAGE;
-  auto block = [&](int g, int b) {  // first column, row 64 b of group g
-    return ws + (static_cast<long long>((32 * g) >> R) << m) + ((32 * g) & (TILE - 1)) + (static_cast<long long>(64 * b) << R);
+  const int lcol = lane & (COLS - 1);
+  const int row0 = (C::TALL ? 512 * (lane >> 4) : 0) + 1024 * sub;  // this lane's first row
+  auto first_col = [&](int g) { return (COLS * g) & (TILE - 1); };
+  auto plane = [&](int g) { return ws + (static_cast<long long>((COLS * g) >> R) << m) + first_col(g); };
+  // this lane's column of group g, from its row 64 b on
+  auto block = [&](int g, int b) { return plane(g) + lcol + (static_cast<long long>(row0 + 64 * b) << R); };
+  auto stage = [&](int g) {
+    if constexpr (C::TALL) {  // lanes 0..3 and 4..7 of a row copy the two halves
+      const float* src = plane(g) + 4 * (lane & 3) + (static_cast<long long>(1024 * sub + 512 * ((lane >> 2) & 1) + 64 * (i + NW) + (lane >> 3)) << R);
+      const uint32_t d = tc::smem_u32(stg) + 16 * lane;
+#pragma unroll
+      for (int j = 0; j < 16; ++j) cp_async16(d + 512 * j, src + (static_cast<long long>(4 * j) << R));
+    } else {
+      stage_block<64>(plane(g) + (static_cast<long long>(64 * (i + NW)) << R), stg, lane);
+    }
   };
-  if (begin + group < end) stage_block<64>(block(begin + group, i + NW), stg, lane);
+  if (begin + group < end) stage(begin + group);
   for (int g = begin + group; g < end; g += C::GROUPS) {
-    const GainT gain(P, tab, ((32 * g) & (TILE - 1)) + lane);
+    const GainT gain(P, tab, first_col(g) + lcol);
     auto round_ac = [&](float2 (&v)[32]) {
 #pragma unroll
       for (int j = 0; j < 32; ++j) bf_in(v[j]);
@@ -490,7 +508,7 @@ __device__ __forceinline__ void col_lanes(float* ws, int begin, int end, const P
     };
     {
       float2 v[32];
-      const float* src = block(g, i) + lane;
+      const float* src = block(g, i);
 #pragma unroll
       for (int j = 0; j < 32; ++j) v[j] = make_float2(__ldcg(src + ((2 * j) << R)), __ldcg(src + ((2 * j + 1) << R)));
       round_ac(v);
@@ -501,17 +519,28 @@ __device__ __forceinline__ void col_lanes(float* ws, int begin, int end, const P
 #pragma unroll
       for (int j = 0; j < 32; ++j) v[j] = make_float2(stg[64 * j + lane], stg[64 * j + 32 + lane]);
       __syncwarp();
-      if (g + C::GROUPS < end) stage_block<64>(block(g + C::GROUPS, i + NW), stg, lane);
+      if (g + C::GROUPS < end) stage(g + C::GROUPS);
       round_ac(v);
 #pragma unroll
       for (int q = 0; q < 4; ++q) st_pairs<8>(ta + 64 * (i + NW) + 16 * q, v + 8 * q);
     }
-    // round B: pair k = (s, low) is rows 64 s + (64 / NW) i + W pass + 2 low and + 1
+    // round B: pair k of a pass is rows pair_row(k) and + 1 of this lane; after the trade between quarters, rows of quarter
+    // k / (16 / NQ) at the place of pair (16 / NQ) sub + k mod (16 / NQ)
     const int low0 = (64 / NW) * i;
+    constexpr int KQ = 16 / NQ;
+    auto pair_row = [&](int k, int pass) { return 64 * (k / WP) + low0 + W * pass + 2 * (k % WP); };
     auto load_gains = [&](float2 (&gg)[16], int pass) {
 #pragma unroll
-      for (int k = 0; k < 16; ++k) gg[k] = gain.rows2(64 * (k / WP) + low0 + W * pass + 2 * (k % WP));
+      for (int k = 0; k < 16; ++k) {
+        if constexpr (NQ == 1) {
+          gg[k] = gain.rows2(row0 + pair_row(k, pass));
+        } else {
+          const int kk = k % KQ, r = 64 * (sub * (KQ / WP) + kk / WP) + low0 + W * pass + 2 * (kk % WP);
+          gg[k] = gain.rows2(row0 - 1024 * sub + 1024 * (k / KQ) + r);
+        }
+      }
     };
+    auto trade_sync = [&] { asm volatile("bar.sync %0, %1;" ::"r"(5 + i * (4 / NQ) + group % (4 / NQ)), "r"(32 * NQ) : "memory"); };
     auto round_b_pass = [&](const float2 (&gg)[16], int pass) {
       float2 v[16];
 #pragma unroll
@@ -524,31 +553,68 @@ __device__ __forceinline__ void col_lanes(float* ws, int begin, int end, const P
           for (int k = 0; k < 16; ++k)
             if ((k & h) == 0) bf2(v[k], v[k + h]);
       };
+      auto lane_bit = [&] {  // row bit 9: lanes l, l ^ 16
+        if constexpr (C::TALL) {
+          const float2 sgn = (lane & 16) ? make_float2(-1.f, -1.f) : make_float2(1.f, 1.f);
+#pragma unroll
+          for (int k = 0; k < 16; ++k) {
+            const float2 p = make_float2(__shfl_xor_sync(0xffffffffu, v[k].x, 16), __shfl_xor_sync(0xffffffffu, v[k].y, 16));
+            v[k] = fast::fma2(v[k], sgn, p);
+          }
+        }
+      };
       across();
-      // pair k's rows in this column
-      auto row = [&](int k) { return static_cast<long long>(64 * (k / WP) + low0 + W * pass + 2 * (k % WP)) << R; };
+      lane_bit();
       if constexpr (MODE == SPECTRUM) {
-        float* o = block(g, 0) + lane;
+        float* o = block(g, 0);
 #pragma unroll
         for (int k = 0; k < 16; ++k) {
-          __stcg(o + row(k), v[k].x);
-          __stcg(o + row(k) + TILE, v[k].y);
+          __stcg(o + (static_cast<long long>(pair_row(k, pass)) << R), v[k].x);
+          __stcg(o + (static_cast<long long>(pair_row(k, pass) + 1) << R), v[k].y);
         }
       } else {
         if constexpr (MODE == ADJOINT) {
-          float* xp = xws + (block(g, 0) - ws) + lane;
+          float* xp = xws + (block(g, 0) - ws);
           float2 xh[16];
 #pragma unroll
-          for (int k = 0; k < 16; ++k) xh[k] = make_float2(__ldcg(xp + row(k)), __ldcg(xp + row(k) + TILE));
+          for (int k = 0; k < 16; ++k)
+            xh[k] = make_float2(__ldcg(xp + (static_cast<long long>(pair_row(k, pass)) << R)),
+                                __ldcg(xp + (static_cast<long long>(pair_row(k, pass) + 1) << R)));
 #pragma unroll
           for (int k = 0; k < 16; ++k) {
             const float2 pr = mul2(mul2(xh[k], v[k]), sc);
-            __stcg(xp + row(k), pr.x);
-            __stcg(xp + row(k) + TILE, pr.y);
+            __stcg(xp + (static_cast<long long>(pair_row(k, pass)) << R), pr.x);
+            __stcg(xp + (static_cast<long long>(pair_row(k, pass) + 1) << R), pr.y);
           }
+        }
+        // the trade areas lie behind the staged blocks
+        auto area = [&](int s) { return reinterpret_cast<float2*>(slots + (warp - sub + s) * WARP_STAGE + 64 * 32) + lane; };
+        auto quarters = [&] {
+#pragma unroll
+          for (int h = KQ; h < 16; h <<= 1)
+#pragma unroll
+            for (int k = 0; k < 16; ++k)
+              if ((k & h) == 0) bf2(v[k], v[k + h]);
+        };
+        if constexpr (NQ > 1) {
+#pragma unroll
+          for (int k = 0; k < 16; ++k) area(sub)[32 * k] = v[k];
+          trade_sync();
+#pragma unroll
+          for (int k = 0; k < 16; ++k) v[k] = area(k / KQ)[32 * (KQ * sub + k % KQ)];
+          quarters();
         }
 #pragma unroll
         for (int k = 0; k < 16; ++k) v[k] = mul2(v[k], mul2(gg[k], sc));
+        if constexpr (NQ > 1) {
+          quarters();
+#pragma unroll
+          for (int k = 0; k < 16; ++k) area(k / KQ)[32 * (KQ * sub + k % KQ)] = v[k];
+          trade_sync();
+#pragma unroll
+          for (int k = 0; k < 16; ++k) v[k] = area(sub)[32 * k];
+        }
+        lane_bit();
         across();
 #pragma unroll
         for (int s = 0; s < NB; ++s) st_pairs<WP>(ta + 64 * s + low0 + W * pass, v + WP * s);
@@ -557,7 +623,7 @@ __device__ __forceinline__ void col_lanes(float* ws, int begin, int end, const P
     if constexpr (MODE == FWD) {
       float2 ga[16], gb[16];
       load_gains(ga, 0);
-      lane_sync<NW>(group);
+      lane_sync<NW>(bar);
 #pragma unroll 1
       for (int pass = 0; pass < 4; pass += 2) {
         load_gains(gb, pass + 1);
@@ -566,7 +632,7 @@ __device__ __forceinline__ void col_lanes(float* ws, int begin, int end, const P
         round_b_pass(gb, pass + 1);
       }
     } else {  // (the spectrum's registers leave no room to load gains a pass ahead)
-      lane_sync<NW>(group);
+      lane_sync<NW>(bar);
 #pragma unroll 1
       for (int pass = 0; pass < 4; ++pass) {
         float2 gg[16];
@@ -574,11 +640,11 @@ __device__ __forceinline__ void col_lanes(float* ws, int begin, int end, const P
         round_b_pass(gg, pass);
       }
     }
-    lane_sync<NW>(group);
+    lane_sync<NW>(bar);
 #pragma unroll 1
     for (int it = 0; it < (MODE == SPECTRUM ? 0 : 2); ++it) {
       float2 v[32];
-      float* dst = block(g, i + NW * it) + lane;
+      float* dst = block(g, i + NW * it);
       read_row(ta + 64 * (i + NW * it), v);
       round_ac(v);
 #pragma unroll
@@ -782,152 +848,23 @@ __device__ __forceinline__ void col_lanes_bwd(float* wsx, float* wsd, int begin,
 }
 
 // ---------------------------------------------------------------------------------------------
-// Columns, Q >= 10.  A unit is W = 2^(14-Q) adjacent columns of all 2^Q rows of a plane, two slots; its element e (row
-// e >> (14-Q), column e mod W) is word e, bit 4 XORed with bit 9.  A team's thread tt takes
-//   round A  the pairs at 2 tt + 512 i, i = 0..31 (word bits 9..13);
-//   round B  word bits 1, 2, 3, 9, 10 in the lane, 11..13 in the warp, 4..8 in the registers.
-// Word bit x is a row bit if x >= 14 - Q: ten of them in the registers of the two rounds, those below bit 4
-// (Q = 11, 12) across the lanes of round B by shuffles.
-constexpr int UNIT = 2 * TILE;
-template <int Q>
-struct Col {
-  static_assert(Q >= 10 && Q <= 12, "two rounds of five bits and at most two lane bits");
-  static constexpr int W = 1 << (R + 1 - Q);
-  // plane offset of unit word e; additive over disjoint bits
-  __host__ __device__ static constexpr int off(int e) { return ((e >> (R + 1 - Q)) << R) + (e & (W - 1)); }
-};
-
-// Gains of a thread's round-B pairs: pair k sits at unit words e0 + 16 k and + 1.
-template <int Q>
-struct FullGain {
-  const float* p;
-  __device__ __forceinline__ FullGain(const Params& P, const float*, int col0, int e0)
-      : p(static_cast<const float*>(P.g) + col0 + Col<Q>::off(e0)) {}
-  __device__ __forceinline__ float2 at(int k) const { return __ldg(reinterpret_cast<const float2*>(p + Col<Q>::off(16 * k))); }
-};
-template <int Q>
-struct SepGain {  // two channels of one token row range
-  const float* p;
-  float2 e;
-  __device__ __forceinline__ SepGain(const Params& P, const float* tab, int col0, int e0) {
-    const int c = col0 + (e0 & (Col<Q>::W - 1)), ch = c & ((1 << P.cbits) - 1);
-    const float* ec = tab + (1ll << (P.m - P.cbits));
-    p = tab + (static_cast<long long>(c >> P.cbits) << Q) + (e0 >> (R + 1 - Q));
-    e = make_float2(ec[ch], ec[ch + 1]);
-  }
-  __device__ __forceinline__ float2 at(int k) const {
-    const float t = p[(16 * k) >> (R + 1 - Q)];
-    return make_float2(t * e.x, t * e.y);
-  }
-};
-
-// Unit u of the plane group (first element at `src`) into two slots, by one team.
-template <int Q>
-__device__ __forceinline__ void load_unit(const float* src, float* slot, int tt, uint64_t* full) {
-  using C = Col<Q>;
-  const float* s = src + C::off(4 * tt);
-  const uint32_t d = tc::smem_u32(slot) + 4 * ((4 * tt) ^ (((tt >> 7) & 1) << 4));
-#pragma unroll
-  for (int i = 0; i < 16; ++i) cp_async16(d + 4096 * i, s + C::off(1024 * i));
-  cp_async_arrive(full);
-}
-
-// Butterfly over the row bit that lanes l and l ^ MASK differ in.
-template <int MASK>
-__device__ __forceinline__ void bfly_lanes(float2 (&v)[32]) {
-  const float2 sgn = (threadIdx.x & MASK) ? make_float2(-1.f, -1.f) : make_float2(1.f, 1.f);
-#pragma unroll
-  for (int k = 0; k < 32; ++k) {
-    const float2 p = make_float2(__shfl_xor_sync(0xffffffffu, v[k].x, MASK), __shfl_xor_sync(0xffffffffu, v[k].y, MASK));
-    v[k] = fast::fma2(v[k], sgn, p);
-  }
-}
-
-// Phase 2 of one unit: column bits, gain, column bits; the result to the workspace at `dst` (the unit's first
-// element).  `wait` is called before the slot is read, so that the first gains are on their way by then.
-template <int Q, class GainT, Mode MODE, class Wait>
-__device__ __forceinline__ void col_unit(float* slot, float* dst, const Params& P, const float* tab, int col0, int tt,
-                                         int team, float* xdst, const Wait& wait) {
-  using C = Col<Q>;
-  const float2 sc = make_float2(P.scale, P.scale);
-  const int l = tt & 31;
-  const int e0 = 2 * (l & 7) + 512 * (l >> 3) + 2048 * (tt >> 5);
-  const GainT gain(P, tab, col0, e0);
-  float2 gg[16];
-  if constexpr (MODE != SPECTRUM) {
-#pragma unroll
-    for (int k = 0; k < 16; ++k) gg[k] = gain.at(k);
-  }
-  wait();
-  float2 v[32];
-  const int a0 = 2 * tt, a1 = a0 ^ 16;
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = *reinterpret_cast<const float2*>(slot + (i & 1 ? a1 : a0) + 512 * i);
-  bfly32<0>(v);
-  const int b0 = e0 ^ (((l >> 3) & 1) << 4), b1 = b0 ^ 16;  // round B: bit 4 is the registers' lowest
-#pragma unroll
-  for (int i = 0; i < 32; ++i) *reinterpret_cast<float2*>(slot + (i & 1 ? a1 : a0) + 512 * i) = v[i];
-  team_sync(team);
-#pragma unroll
-  for (int k = 0; k < 32; ++k) v[k] = *reinterpret_cast<const float2*>(slot + (k & 1 ? b1 : b0) + 32 * (k >> 1));
-  bfly32<0>(v);
-  if constexpr (Q >= 11) bfly_lanes<4>(v);
-  if constexpr (Q >= 12) bfly_lanes<2>(v);
-  if constexpr (MODE == SPECTRUM) {
-    float* o = dst + C::off(e0);
-#pragma unroll
-    for (int k = 0; k < 32; ++k) __stcg(reinterpret_cast<float2*>(o + C::off(16 * k)), v[k]);
-  } else {
-#pragma unroll
-    for (int h = 0; h < 32; h += 16) {
-      if (h > 0) {
-#pragma unroll
-        for (int k = 0; k < 16; ++k) gg[k] = gain.at(k + 16);
-      }
-      if constexpr (MODE == ADJOINT) {
-        float* xp = xdst + C::off(e0);
-#pragma unroll
-        for (int k = 0; k < 16; ++k) {
-          float2* x = reinterpret_cast<float2*>(xp + C::off(16 * (h + k)));
-          __stcg(x, mul2(mul2(__ldcg(x), v[h + k]), sc));
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < 16; ++k) v[h + k] = mul2(v[h + k], mul2(gg[k], sc));
-    }
-    if constexpr (Q >= 12) bfly_lanes<2>(v);
-    if constexpr (Q >= 11) bfly_lanes<4>(v);
-    bfly32<0>(v);
-#pragma unroll
-    for (int k = 0; k < 32; ++k) *reinterpret_cast<float2*>(slot + (k & 1 ? b1 : b0) + 32 * (k >> 1)) = v[k];
-    team_sync(team);
-#pragma unroll
-    for (int i = 0; i < 32; ++i) v[i] = *reinterpret_cast<const float2*>(slot + (i & 1 ? a1 : a0) + 512 * i);
-    bfly32<0>(v);
-    float* o = dst + C::off(2 * tt);
-#pragma unroll
-    for (int i = 0; i < 32; ++i) __stcg(reinterpret_cast<float2*>(o + C::off(512 * i)), v[i]);
-  }
-}
-
-// ---------------------------------------------------------------------------------------------
 // What the phases of one CTA share.
 struct Cta {
   float* slots;
-  uint64_t *full_row, *full_pair;
+  uint64_t* full_row;
   uint64_t (*mma_done)[2];
   volatile int* dead;
   GridBarrier* bar;
   uint32_t tmem;
-  int worker, t, team, tt;
-  unsigned row_seq, pair_seq, mma_seq;  // tiles taken from each ring so far
+  int worker, t;
+  unsigned row_seq, mma_seq;  // rows taken from the ring, and multiplied, so far
 };
 struct __align__(8) CtaShared {
-  uint64_t full_row[ROW_BARS], full_pair[PAIR_BARS], mma_done[WORKERS][2];
+  uint64_t full_row[ROW_BARS], mma_done[WORKERS][2];
   int flag, dead;
   uint32_t tmem_slot;
 };
-__host__ __device__ constexpr bool uses_tmem(int dtype, int q) { return dtype == DT_BF16 || (q >= 6 && q <= 9); }
+__host__ __device__ constexpr bool uses_tmem(int dtype, int q) { return dtype == DT_BF16 || q >= 6; }
 
 // Before the launch wait: tensor memory, H_128, the barriers.
 template <int D, int Q>
@@ -942,7 +879,6 @@ __device__ __forceinline__ Cta cta_begin(unsigned char* smem, CtaShared& sh, con
   if (threadIdx.x == 0) {
     sh.dead = 0;
     for (int i = 0; i < ROW_BARS; ++i) tc::mbar_init(&sh.full_row[i], WT);
-    for (int i = 0; i < PAIR_BARS; ++i) tc::mbar_init(&sh.full_pair[i], 2 * WT);
     for (int i = 0; i < WORKERS; ++i)
       for (int k = 0; k < 2; ++k) tc::mbar_init(&sh.mma_done[i][k], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -950,9 +886,8 @@ __device__ __forceinline__ Cta cta_begin(unsigned char* smem, CtaShared& sh, con
   fast::tmem_fence_before();
   __syncthreads();
   fast::tmem_fence_after();
-  return {reinterpret_cast<float*>(smem), sh.full_row, sh.full_pair, sh.mma_done, &sh.dead, P.bar,
-          uses_tmem(D, Q) ? sh.tmem_slot : 0u, static_cast<int>(threadIdx.x) / WT, static_cast<int>(threadIdx.x) % WT,
-          static_cast<int>(threadIdx.x) / (2 * WT), static_cast<int>(threadIdx.x) % (2 * WT), 0, 0, 0};
+  return {reinterpret_cast<float*>(smem), sh.full_row, sh.mma_done, &sh.dead, P.bar, uses_tmem(D, Q) ? sh.tmem_slot : 0u,
+          static_cast<int>(threadIdx.x) / WT, static_cast<int>(threadIdx.x) % WT, 0, 0};
 }
 template <int D, int Q>
 __device__ __forceinline__ void cta_end(CtaShared& sh) {
@@ -1067,44 +1002,14 @@ __device__ __forceinline__ void rows_out(Cta& c, int n, const float* wsr, void* 
 // Column bits of nb planes of a workspace, all CTAs together.
 template <int Q, bool SEP, Mode MODE>
 __device__ __forceinline__ void columns(Cta& c, float* ws, int nb, const Params& P, const float* tab, float* xws = nullptr) {
-  constexpr int m = R + Q;
   using LaneT = typename std::conditional<SEP, LaneSep<Q>, LaneFull<Q>>::type;
   if constexpr (Q <= 6) {
     col_regs<Q, LaneT>(ws, nb << R, P, tab, c.slots);
-  } else if constexpr (Q <= 9) {
+  } else {
     int gb, ge;
-    share(static_cast<unsigned>(nb) << (R - 5), &gb, &ge);
+    share(static_cast<unsigned>(nb) << Lane<Q>::LOG_GROUPS, &gb, &ge);
     col_lanes<Q, LaneT, MODE>(ws, gb, ge, P, tab, c.tmem, c.slots, xws);
     fast::tmem_fence_before();
-  } else {
-    using GainT = typename std::conditional<SEP, SepGain<Q>, FullGain<Q>>::type;
-    constexpr int UB = Q - 1;  // log2 of the units of a plane
-    int ub, ue;
-    share(static_cast<unsigned>(nb) << UB, &ub, &ue);
-    const int nu = ue - ub;
-    auto offset = [&](int k, int* col0) {
-      const int u = ub + k;
-      *col0 = (u & ((1 << UB) - 1)) << (R + 1 - Q);
-      return (static_cast<long long>(u >> UB) << m) + *col0;
-    };
-    auto load = [&](int k) {
-      int col0;
-      const long long o = offset(k, &col0);
-      load_unit<Q>(ws + o, c.slots + (c.pair_seq + k) % PAIRS * UNIT, c.tt, &c.full_pair[(c.pair_seq + k) % PAIR_BARS]);
-    };
-    for (int k = c.team; k < PAIRS && k < nu; k += 2) load(k);
-    for (int k = c.team; k < nu; k += 2) {
-      int col0;
-      const long long o = offset(k, &col0);
-      col_unit<Q, GainT, MODE>(c.slots + (c.pair_seq + k) % PAIRS * UNIT, ws + o, P, tab, col0, c.tt, c.team, xws + o,
-                               [&] { wait_full(c.full_pair, c.pair_seq + k, PAIR_BARS, c.bar, c.dead); });
-      if (k + PAIRS < nu) {
-        team_sync(c.team);
-        load(k + PAIRS);
-      }
-    }
-    c.pair_seq += nu;
-    if constexpr (MODE == SPECTRUM) __syncthreads();  // the next pass refills the slots
   }
 }
 
@@ -1201,7 +1106,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_forward_fast(Params P) {
 
 // Backward kernel (planes of 2^14 .. 2^23 elements).  Against the previous one (8 warps, one column a thread or two passes
 // through tensor memory, dG summed plane after plane), forward and backward together: [16, 8192, 256] bf16 465 -> 379 us,
-// [8, 4096, 256] bf16 118 -> 91, [1, 65536, 128] bf16 186 -> 148, [4, 16384, 256] bf16 335 -> 243, [32, 1024, 64] bf16
+// [8, 4096, 256] bf16 118 -> 91, [1, 65536, 128] bf16 186 -> 132, [4, 16384, 256] bf16 335 -> 243, [32, 1024, 64] bf16
 // 36.3 -> 32.5.  Per group of four 2^21-element planes now: phase 1 18 us, columns 22, rows out 9, dG 7, barriers 5; its
 // workspaces (64 MiB) and the streamed X, dY, dX do not fit L2 together (700 MB of HBM traffic a call against 218 MB),
 // and smaller groups lose more to phases than they save (48 MiB 437 us, 32 MiB 461).

@@ -1,0 +1,46 @@
+"""GPU parity at the edges of the kernels' ranges that the shape sweeps do not reach: planes of 2^24 and 2^25 elements
+(columns of 2048 and 4096 rows, shared by two and four tensor-memory lane quarters).  Bounds as in _checks.py."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from _checks import Guarded, check, ref_inputs, to_dev
+from paper_2607_25234_gb300 import inputs, whtmix
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    from paper_2607_25234_gb300 import build
+    build.build()
+    oracle.build()
+    torch.cuda.set_device(0)
+
+
+@pytest.mark.parametrize("B,n,N,C,dtype", [(1, 1 << 17, 1 << 17, 128, "f32"), (2, 70001, 1 << 17, 128, "bf16"),
+                                           (1, 1 << 12, 1 << 12, 1 << 13, "bf16"), (1, 259200, 1 << 18, 128, "bf16"),
+                                           (1, (1 << 18) - 3, 1 << 18, 128, "f32")])
+def test_tall_columns_forward(B, n, N, C, dtype):
+    d = inputs.make_inputs(B, N, C, dtype, seed=n, n_valid=n)
+    x, g = to_dev(d["x"], dtype), to_dev(d["g"], "f32")
+    y = Guarded((B, n, C), x.dtype)
+    whtmix.forward_padded(x[:, :n].contiguous(), g, out=y.t)
+    whtmix.sync()
+    r = ref_inputs(d, dtype)
+    check(y.t, oracle.forward(r["x"], r["g"])[:, :n], dtype, f"Y [{B},{n} of {N},{C}] {dtype}")
+    y.assert_intact("Y")
+
+
+@pytest.mark.parametrize("N,C,dtype", [(1 << 17, 128, "bf16"), (1 << 13, 1 << 11, "f32"), (1 << 18, 128, "f32")])
+def test_tall_columns_log_gains(N, C, dtype):
+    d = inputs.make_inputs(1, N, C, dtype, seed=N + C)
+    g_t, g_c = inputs.make_log_gains(N, C, seed=3)
+    x = to_dev(d["x"], dtype)
+    y = Guarded(x.shape, x.dtype)
+    whtmix.forward_separable(x, torch.from_numpy(g_t).cuda(), torch.from_numpy(g_c).cuda(), out=y.t)
+    whtmix.sync()
+    ref = oracle.forward_separable(ref_inputs(d, dtype)["x"], g_t.astype(np.float64), g_c.astype(np.float64))
+    check(y.t, ref, dtype, f"separable Y [1,{N},{C}] {dtype}")
+    y.assert_intact("Y")
