@@ -1,11 +1,12 @@
 """GPU parity at the edges of the kernels' ranges that the shape sweeps do not reach: planes of 2^24 and 2^25 elements
-(columns of 2048 and 4096 rows, shared by two and four tensor-memory lane quarters).  Bounds as in _checks.py."""
+(columns of 2048 and 4096 rows, shared by two and four tensor-memory lane quarters), and the block, the small planes and the log
+gain gradients at theirs.  Bounds as in _checks.py."""
 import numpy as np
 import pytest
 import torch
 
 import oracle
-from _checks import Guarded, check, ref_inputs, to_dev
+from _checks import Guarded, check, check_grad, ref_inputs, to_dev
 from paper_2607_25234_gb300 import inputs, whtmix
 
 pytestmark = pytest.mark.gpu
@@ -44,3 +45,23 @@ def test_tall_columns_log_gains(N, C, dtype):
     ref = oracle.forward_separable(ref_inputs(d, dtype)["x"], g_t.astype(np.float64), g_c.astype(np.float64))
     check(y.t, ref, dtype, f"separable Y [1,{N},{C}] {dtype}")
     y.assert_intact("Y")
+
+
+# one and two channel blocks of 32 and a part of one; token counts below, at and past a block of 32 and of a chunk
+@pytest.mark.parametrize("B,n,N,C,dtype", [(3, 5, 8, 4, "f32"), (2, 17, 32, 64, "f32"), (2, 4000, 4096, 32, "f32"),
+                                           (1, 1 << 14, 1 << 14, 2, "bf16"), (1, 2, 2, 1 << 13, "f32"), (2, 8192, 8192, 256, "bf16")])
+def test_log_gain_gradients_in_one_pass(B, n, N, C, dtype):
+    d = inputs.make_inputs(B, N, C, dtype, seed=n + C, n_valid=n, with_dy=True)
+    g_t, g_c = inputs.make_log_gains(N, C, seed=5)
+    x, dy = (to_dev(d[k], dtype)[:, :n].contiguous() for k in ("x", "dy"))
+    out = [Guarded((B, n, C), x.dtype), Guarded((N,), torch.float32), Guarded((C,), torch.float32)]
+    whtmix.backward_separable(x, torch.from_numpy(g_t).cuda(), torch.from_numpy(g_c).cuda(), dy, dx=out[0].t, dg_t=out[1].t,
+                              dg_c=out[2].t)
+    whtmix.sync()
+    r = ref_inputs(d, dtype)
+    dx, dgt, dgc = oracle.backward_separable(r["x"], g_t.astype(np.float64), g_c.astype(np.float64), r["dy"])
+    check(out[0].t, dx[:, :n], dtype, "dX")
+    check_grad(out[1].t, dgt, "f32", "dg_t")
+    check_grad(out[2].t, dgc, "f32", "dg_c")
+    for o, name in zip(out, ("dX", "dg_t", "dg_c")):
+        o.assert_intact(name)
