@@ -44,7 +44,7 @@ REASONS = {0x1: "gpu_idle", 0x2: "applications_clocks_setting", 0x4: "sw_power_c
 KERNEL_FAMILY_SOURCES = {
     "k_forward_fast": ("whtmix_kernels.cuh", "whtmix_fast.cuh", "whtmix_fast_launch.cuh", "whtmix_tri.cuh"),
     "k_backward_fast": ("whtmix_kernels.cuh", "whtmix_fast.cuh", "whtmix_fast_launch.cuh", "whtmix_tri.cuh"),
-    "k_block_fast": ("whtmix_kernels.cuh", "whtmix_fast.cuh", "whtmix_block.cuh", "whtmix_block.cu"),
+    "k_block_fast": ("whtmix_kernels.cuh", "whtmix_fast.cuh", "whtmix_tri.cuh", "whtmix_block.cuh", "whtmix_block.cu"),
     "k_forward_plane": ("whtmix_kernels.cuh", "whtmix_fast.cuh", "whtmix_plane.cuh", "whtmix_plane.cu"),
 }
 
@@ -52,14 +52,14 @@ KERNEL_FAMILY_SOURCES = {
 def block_fused(w) -> bool:
     """True where whtmix_block_forward runs the whole block as one fused launch (mirrors the C ABI)."""
     m = (w.N * w.C).bit_length() - 1
-    return w.block and w.dtype == "bf16" and w.C == 128 and 21 <= m <= 23
+    return w.block and w.dtype == "bf16" and w.C in (64, 128) and 17 <= m <= 23
 
 
 def kernel_name(w) -> str:
     """The kernel one whtmix_forward call launches for this workload (mirrors the C ABI's dispatch)."""
     m = (w.N * w.C).bit_length() - 1
     if block_fused(w):
-        return f"k_block_fast<bf16, R=14, Q={m - 14}>"
+        return f"k_block_fast<bf16, R=13, Q={m - 13}>"
     padded_ok = w.n_valid is None or (w.n_valid * w.C * (2 if w.dtype == "bf16" else 4)) % 16 == 0
     if (w.dtype in ("f32", "bf16") and 14 <= m <= 16 and (m < 16 or w.B >= 80) and w.gains == "full"
             and not w.block and (not w.padded_io or padded_ok)):

@@ -24,7 +24,7 @@ cudaError_t forward_f32(const Params& P, cudaStream_t stream);
 cudaError_t forward_bf16(const Params& P, cudaStream_t stream);
 }  // namespace pln
 namespace blk {
-// Fused block (whtmix_block.cu): bf16, C = 128, 2^21 <= N C <= 2^23, full gains, N_valid = N.
+// Fused block (whtmix_block.cu): bf16, C = 64 or 128, 2^17 <= N C <= 2^23, full gains, N_valid = N.
 cudaError_t forward_bf16(const Params& P, const void* w_in, const void* w_out, int sms, cudaStream_t stream);
 }  // namespace blk
 namespace proj {
@@ -805,9 +805,10 @@ Call separable_call(bool backward, const void* x, const float* gt, const float* 
   return c;
 }
 
-// The fused block kernel covers 128 channels and planes of 2^21 to 2^23 elements (rows of 128
-// tokens x 128 channels, columns of 128 to 512 rows).
-bool use_fused_block(int64_t C, int m) { return C == 128 && m >= 21 && m <= 23; }
+// The fused block kernel covers 64 and 128 channels and planes of 2^17 to 2^23 elements.  Against three launches (projection,
+// mixer, projection): [1, 1024, 128] 19.9 -> 13.7 us, [8, 4096, 128] 31.3 -> 25.6, [32, 4096, 64] 50.5 -> 38.1,
+// [16, 8192, 128] 92.5 -> 72.9.  Smaller planes run one per CTA between the projections.
+bool use_fused_block(int64_t C, int m) { return (C == 64 || C == 128) && m >= 17 && m <= 23; }
 
 }  // namespace
 

@@ -65,3 +65,27 @@ def test_log_gain_gradients_in_one_pass(B, n, N, C, dtype):
     check_grad(out[2].t, dgc, "f32", "dg_c")
     for o, name in zip(out, ("dX", "dg_t", "dg_c")):
         o.assert_intact(name)
+
+
+def bf16_dev(a):
+    return torch.from_numpy(inputs.f32_to_bf16_bits(a).view(np.int16)).cuda().view(torch.bfloat16)
+
+
+# the smallest and largest plane of the fused block for each channel count, one per kind of column pass between, and a
+# batch of several plane groups
+@pytest.mark.parametrize("B,N,C", [(1, 1024, 128), (3, 2048, 64), (2, 8192, 64), (5, 8192, 128), (1, 1 << 17, 64), (9, 1 << 15, 64)])
+def test_fused_block(B, N, C):
+    d = inputs.make_inputs(B, N, C, "bf16", seed=B + N + C)
+    w_in, w_out = ((inputs.normal(s + C, C * C) / np.sqrt(C)).reshape(C, C).astype(np.float32) for s in (90, 91))
+    x, g = to_dev(d["x"], "bf16"), to_dev(d["g"], "f32")
+    y = Guarded(x.shape, torch.bfloat16)
+    whtmix.block_forward(x, bf16_dev(w_in), g, bf16_dev(w_out), out=y.t)
+    whtmix.sync()
+    y.assert_intact("block Y")
+    x64, g64 = inputs.as_float64(d["x"], "bf16"), d["g"].astype(np.float64)
+    wi, wo = (inputs.as_float64(inputs.f32_to_bf16_bits(w), "bf16") for w in (w_in, w_out))
+    m = oracle.forward(x64 @ wi.T, g64)
+    ref, got = m @ wo.T, y.t.double().cpu().numpy()
+    # M's and Y's roundings to bf16 (half an ulp, 2^-8 of a value) and the fp32 sums before them
+    bound = 2.0 ** -8 * np.abs(ref) + (2.0 ** -8 + 1e-5) * (np.abs(m) @ np.abs(wo).T) + 1e-5 * np.sqrt(np.mean(ref ** 2))
+    assert (np.abs(got - ref) <= bound).all(), float(np.max(np.abs(got - ref) / bound))
