@@ -22,6 +22,7 @@ namespace pln {
 // One plane per CTA in tensor memory (whtmix_plane.cu): fp32 / bf16 planes of 2^14 .. 2^16 elements.
 cudaError_t forward_f32(const Params& P, cudaStream_t stream);
 cudaError_t forward_bf16(const Params& P, cudaStream_t stream);
+void* error_header(int dev);  // their error header on the current device, null if none was launched there
 }  // namespace pln
 namespace blk {
 // Fused block (whtmix_block.cu): bf16, C = 64 or 128, 2^17 <= N C <= 2^23, full gains, N_valid = N.
@@ -49,12 +50,11 @@ thread_local int g_last_cuda_error = 0;
 
 constexpr size_t HEADER_BYTES = sizeof(GridBarrier);
 constexpr size_t WS_TARGET_BYTES = 64ull << 20;  // plane-group workspace, L2-resident (126 MiB L2)
-constexpr int64_t PLANE_MIN_BATCH_16 = 80;
-// Smallest batch for which the one-plane-per-CTA forward beats the three-phase kernel: a plane of
-// 2^16 elements is four rows for one CTA (two per worker, one after the other), so a small batch
-// leaves most SMs idle (measured on [B, 512, 128] bf16, back to back: B = 64 three-phase 24.6 us
-// against 26.6, B = 96 30.8 against 26.7, B = 128 36.0 against 28.7); 2^14 and 2^15 planes are one
-// row per worker.
+constexpr int64_t PLANE_MIN_BATCH_16 = 48;
+// Smallest batch for which the one-plane-per-CTA forward beats the three-phase kernel: a plane of 2^16 elements takes a CTA the
+// same 15 us whether one or all SMs have one, where the three-phase kernel spreads a small batch over every SM (measured on
+// [B, 512, 128] bf16, back to back: B = 40 three-phase 14.7 us against 15.2, B = 64 17.9 against 15.2).  2^14 and 2^15
+// planes take less than the three-phase kernel's phases and barriers.
 int64_t plane_kernel_min_batch(int m) { return m == 16 ? PLANE_MIN_BATCH_16 : 1; }
 
 int cuda_fail(cudaError_t e) {
@@ -1048,14 +1048,14 @@ int whtmix_sync(void* stream_v) {
   int dev = 0;
   e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return cuda_fail(e);
-  void* ptrs[2] = {nullptr, whtmix::noalloc_scratch_of(dev)};
+  void* ptrs[3] = {nullptr, whtmix::noalloc_scratch_of(dev), pln::error_header(dev)};
   {
     std::lock_guard<std::mutex> lk(g_mu);
     auto it = g_ws.find(std::make_tuple(dev, stream, 0));
     if (it != g_ws.end()) ptrs[0] = it->second.ptr;
   }
-  // the stream's library-managed workspace, then the no-allocation scratch of this device (both
-  // keep a set error word until it is reported here)
+  // the stream's library-managed workspace, then this device's no-allocation scratch and the
+  // one-plane-per-CTA kernels' header (all keep a set error word until it is reported here)
   int rc = WHTMIX_OK;
   for (void* ptr : ptrs) {
     if (!ptr) continue;

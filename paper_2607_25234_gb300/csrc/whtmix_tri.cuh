@@ -119,8 +119,9 @@ __device__ __forceinline__ void bfly32(float2 (&v)[32]) {
 // (16-byte chunk j of row r at chunk j ^ (r mod 8)).
 //
 // H_128 (A: 128 rows, two panels of 16 KiB): entry (i, k) = (-1)^popcount(i & k).
+template <int NT = THREADS>
 __device__ __forceinline__ void build_h(unsigned char* sh) {
-  for (int q = threadIdx.x; q < 128 * 16; q += THREADS) {
+  for (int q = threadIdx.x; q < 128 * 16; q += NT) {
     const int i = q >> 4, c = q & 15;  // k = 8 c ..
     const uint32_t flip = (__popc(i & (8 * c)) & 1) ? 0x80008000u : 0u;
     uint32_t w[4];

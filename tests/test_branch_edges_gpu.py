@@ -89,3 +89,34 @@ def test_fused_block(B, N, C):
     # M's and Y's roundings to bf16 (half an ulp, 2^-8 of a value) and the fp32 sums before them
     bound = 2.0 ** -8 * np.abs(ref) + (2.0 ** -8 + 1e-5) * (np.abs(m) @ np.abs(wo).T) + 1e-5 * np.sqrt(np.mean(ref ** 2))
     assert (np.abs(got - ref) <= bound).all(), float(np.max(np.abs(got - ref) / bound))
+
+
+def run_padded(B, n, N, C, dtype, backward):
+    d = inputs.make_inputs(B, N, C, dtype, seed=n + N, n_valid=n, with_dy=backward)
+    x, g = to_dev(d["x"], dtype)[:, :n].contiguous(), to_dev(d["g"], "f32")
+    r = ref_inputs(d, dtype)
+    y = Guarded((B, n, C), x.dtype)
+    whtmix.forward_padded(x, g, out=y.t)
+    whtmix.sync()
+    check(y.t, oracle.forward(r["x"], r["g"])[:, :n], dtype, f"Y [{B},{n} of {N},{C}] {dtype}")
+    y.assert_intact("Y")
+    if not backward:
+        return
+    dy = to_dev(d["dy"], dtype)[:, :n].contiguous()
+    dx, dg = Guarded((B, n, C), x.dtype), Guarded((N, C), torch.float32)
+    whtmix.backward_padded(x, g, dy, dx=dx.t, dg=dg.t)
+    whtmix.sync()
+    ref_dx, ref_dg = oracle.backward(r["x"], r["g"], r["dy"])
+    check(dx.t, ref_dx[:, :n], dtype, f"dX [{B},{n} of {N},{C}] {dtype}")
+    check_grad(dg.t, ref_dg, dtype, f"dG [{B},{n} of {N},{C}] {dtype}")
+    dx.assert_intact("dX")
+    dg.assert_intact("dG")
+
+
+# one plane a CTA (2^14, 2^15, and 2^16 from its smallest batch): whole, cut inside a 16-byte chunk's row, one token stored;
+# more planes than SMs
+@pytest.mark.parametrize("B,n,N,C", [(1, 256, 256, 64), (3, 249, 256, 64), (2, 1, 512, 64), (3, 1023, 1024, 32), (48, 512, 512, 128),
+                                     (49, 333, 512, 128), (310, 128, 128, 128), (160, 500, 512, 64)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_plane_in_tensor_memory(B, n, N, C, dtype):
+    run_padded(B, n, N, C, dtype, False)
