@@ -24,6 +24,11 @@ cudaError_t forward_f32(const Params& P, cudaStream_t stream);
 cudaError_t forward_bf16(const Params& P, cudaStream_t stream);
 void* error_header(int dev);  // their error header on the current device, null if none was launched there
 }  // namespace pln
+namespace sml {
+// Planes of 2^10 .. 2^13 elements (whtmix_small.cu), forward and backward.
+cudaError_t run_f32(bool backward, const Params& P, cudaStream_t stream);
+cudaError_t run_bf16(bool backward, const Params& P, cudaStream_t stream);
+}  // namespace sml
 namespace blk {
 // Fused block (whtmix_block.cu): bf16, C = 64 or 128, 2^17 <= N C <= 2^23, full gains, N_valid = N.
 cudaError_t forward_bf16(const Params& P, const void* w_in, const void* w_out, int sms, cudaStream_t stream);
@@ -300,6 +305,11 @@ bool use_fast_backward(int dtype, int m) {
   return (dtype == WHTMIX_F32 || dtype == WHTMIX_BF16) && m >= 14 && m <= 23;
 }
 
+// The small-plane kernels (whtmix_small.cuh) cover fp32 / bf16 planes of 2^10 .. 2^13 elements; they read and write planes of any
+// whole number of 4-element vectors, so that these pad without copies.
+bool use_small(int dtype, int m) { return dtype != WHTMIX_I32 && m >= 10 && m <= TILE_BITS; }
+bool small_pads(int dtype, int m, size_t lv) { return use_small(dtype, m) && lv % 4 == 0; }
+
 // ws16: the three-phase forward exchanges bf16 (whtmix_forward_x16); P.ws is then sized for it.
 template <int D>
 int dispatch(bool backward, const Params& P, int sms, cudaStream_t stream, bool ws16 = false) {
@@ -307,6 +317,12 @@ int dispatch(bool backward, const Params& P, int sms, cudaStream_t stream, bool 
   const int m = P.m;
   const size_t tile_bytes = sizeof(A) * TILE;
   if (m > MAX_PLANE_BITS_M) return dispatch_plan_l<D>(backward, P, sms, stream);
+  if constexpr (D != DT_I32) {
+    if (use_small(D, m)) {
+      const cudaError_t e = D == DT_BF16 ? sml::run_bf16(backward, P, stream) : sml::run_f32(backward, P, stream);
+      return e == cudaSuccess ? WHTMIX_OK : cuda_fail(e);
+    }
+  }
   if (!backward) {
     if constexpr (D != DT_I32) {
       if (use_fast_forward(D, m)) {
@@ -546,7 +562,7 @@ Layout plan_call(const Call& c, int m) {
   const size_t lv = static_cast<size_t>(c.n_valid) * static_cast<size_t>(c.C);
   // the fast kernels pad and crop in their row passes when every stored plane starts 16-byte aligned
   const bool fast = c.backward ? use_fast_backward(c.dtype, m) : use_fast_forward(c.dtype, m);
-  l.pad_copy = lv < L && !(fast && (lv * es) % 16 == 0);
+  l.pad_copy = lv < L && !(fast && (lv * es) % 16 == 0) && !small_pads(c.dtype, m, lv);
   l.fast_sep = c.separable && !c.backward && !l.pad_copy && use_fast_separable(c.dtype, m, cbits);
   // whtmix_workspace_bytes for a plain call
   l.base = workspace_bytes(c.B, m, c.backward, c.group_target, x16_applies(c, m) ? 2 : 4);

@@ -120,3 +120,12 @@ def run_padded(B, n, N, C, dtype, backward):
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_plane_in_tensor_memory(B, n, N, C, dtype):
     run_padded(B, n, N, C, dtype, False)
+
+
+# tiles of 8, 4, 2 planes and one: a short last tile, padding in vectors of four elements and (one or two channels) not,
+# more planes than a round of the dG sum
+@pytest.mark.parametrize("B,n,N,C", [(1, 32, 32, 32), (9, 31, 32, 32), (5, 64, 64, 32), (130, 61, 64, 32), (257, 64, 64, 64), (3, 33, 64, 64),
+                                     (2, 128, 128, 64), (5, 1, 128, 64), (3, 1021, 2048, 2), (4, 4093, 4096, 1), (2, 1, 1, 1 << 13)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_small_planes(B, n, N, C, dtype):
+    run_padded(B, n, N, C, dtype, True)
