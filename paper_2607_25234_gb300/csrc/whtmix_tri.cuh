@@ -472,7 +472,7 @@ __device__ __forceinline__ void st_pairs(uint32_t ta, const float2* v) {
   else tmem_st4(ta, f);
 }
 template <int Q, class GainT, Mode MODE = FWD>
-__device__ __forceinline__ void col_lanes(float* ws, int begin, int end, const Params& P, const float* tab, uint32_t tmem,
+__device__ __forceinline__ void col_lanes(float* ws, int begin, int end, int total, const Params& P, const float* tab, uint32_t tmem,
                                           float* slots, float* xws = nullptr) {
   using C = Lane<Q>;
   constexpr int m = R + Q, NB = C::NB, NW = C::NW, W = C::W, WP = W / 2, NQ = C::NQ, COLS = C::COLS;
@@ -499,8 +499,13 @@ __device__ __forceinline__ void col_lanes(float* ws, int begin, int end, const P
       stage_block<64>(plane(g) + (static_cast<long long>(64 * (i + NW)) << R), stg, lane);
     }
   };
-  if (begin + group < end) stage(begin + group);
-  for (int g = begin + group; g < end; g += C::GROUPS) {
+  // neighbouring CTAs take neighbouring groups where the plane lies in HBM (the rows' segments then fall into the same DRAM pages at
+  // the same time), else each CTA a contiguous range
+  const int first = NQ > 1 ? static_cast<int>(blockIdx.x) * C::GROUPS + group : begin + group;
+  const int step = NQ > 1 ? static_cast<int>(gridDim.x) * C::GROUPS : C::GROUPS;
+  if constexpr (NQ > 1) end = total;
+  if (first < end) stage(first);
+  for (int g = first; g < end; g += step) {
     const GainT gain(P, tab, first_col(g) + lcol);
     auto round_ac = [&](float2 (&v)[32]) {
 #pragma unroll
@@ -520,7 +525,7 @@ __device__ __forceinline__ void col_lanes(float* ws, int begin, int end, const P
 #pragma unroll
       for (int j = 0; j < 32; ++j) v[j] = make_float2(stg[64 * j + lane], stg[64 * j + 32 + lane]);
       __syncwarp();
-      if (g + C::GROUPS < end) stage(g + C::GROUPS);
+      if (g + step < end) stage(g + step);
       round_ac(v);
 #pragma unroll
       for (int q = 0; q < 4; ++q) st_pairs<8>(ta + 64 * (i + NW) + 16 * q, v + 8 * q);
@@ -1009,7 +1014,7 @@ __device__ __forceinline__ void columns(Cta& c, float* ws, int nb, const Params&
   } else {
     int gb, ge;
     share(static_cast<unsigned>(nb) << Lane<Q>::LOG_GROUPS, &gb, &ge);
-    col_lanes<Q, LaneT, MODE>(ws, gb, ge, P, tab, c.tmem, c.slots, xws);
+    col_lanes<Q, LaneT, MODE>(ws, gb, ge, nb << Lane<Q>::LOG_GROUPS, P, tab, c.tmem, c.slots, xws);
     fast::tmem_fence_before();
   }
 }
