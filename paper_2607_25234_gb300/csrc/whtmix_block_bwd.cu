@@ -3,15 +3,15 @@
 //     dW[o, i] = sum over tokens t of A[t, o] B[t, i]      (dW_out = dY^T M, dW_in = dZ^T X)
 // on the 5th-generation tensor cores, and the weight transposes the projections need.
 //
-// A and B are [T, C] bf16 token rows; the contraction runs over the tokens.  k_wgrad splits the
-// tokens into one chunk per CTA (one persistent CTA per SM, 128 threads): per K tile of 64 tokens
-// the CTA reads the token rows of both operands, transposes 8 x 8 blocks in registers and stages
-// the A rows (output channels o, 128 per MMA tile) and the B rows (input channels i) in the tensor
-// core's 128-byte-swizzled K-major layout, double-buffered, with the next tile's loads in flight;
-// one thread issues tcgen05.mma (kind::f16, M = 128, N = C, K = 16) into a TMEM accumulator per
-// 128 rows of o, committed to an mbarrier per buffer.  Each thread then reads its row o of the
-// accumulator (tcgen05.ld) into the chunk's fp32 partial [C, C]; k_wgrad_reduce adds the partials
-// in a fixed order, so dW is the same bit for bit on every run.
+// A and B are [T, C] bf16 token rows; the contraction runs over the tokens.  k_wgrad splits the tokens into one chunk per
+// CTA (one persistent CTA per SM, 128 threads): K tiles of 64 tokens of both operands are copied as they are by 16-byte
+// cp.async into 128-byte-swizzled panels of 64 channels, up to five tiles ahead, and multiplied from there as
+// M-major and N-major operands (the channels are contiguous, the contraction runs down the panel's rows), so nothing is
+// transposed; one thread issues tcgen05.mma (kind::f16, M = 128, N = C, K = 16) into a TMEM accumulator per 128 rows of
+// o.  Each thread then reads its row o of the accumulator (tcgen05.ld) into the chunk's fp32 partial [C, C];
+// k_wgrad_reduce adds the partials in a fixed order, so dW is the same bit for bit on every run.
+// A chunk is a few tiles (3.4 at 32768 tokens), so its time is the latency of its chain: with 8 x 8 transposes in registers
+// and one tile ahead it took 13.2 us, now 9.0 (32768 tokens, C = 128; whole block_train step [8, 4096, 128] 140 -> 124).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -29,65 +29,62 @@ constexpr int WG_THREADS = 128;    // one thread per TMEM lane = per output row 
 constexpr int TR_THREADS = 256;
 constexpr size_t SMEM_MIN = 120 * 1024;  // more than half an SM: one CTA per SM, so TMEM allocation never waits
 
-// out[c, t] = in[t, c] for t < T, 0 for T <= t < Tp (both bf16; C a multiple of 64, Tp of 64):
-// the weights' transposes.
-__global__ void __launch_bounds__(TR_THREADS) k_transpose(const uint16_t* __restrict__ in, uint16_t* __restrict__ out,
-                                                          long long T, int C, long long Tp) {
+// out0 = in0^T and out1 = in1^T, bf16 [C, C], C a multiple of 64: both weights' transposes in one launch.
+__global__ void __launch_bounds__(TR_THREADS) k_transpose2(const uint16_t* __restrict__ in0, uint16_t* __restrict__ out0,
+                                                           const uint16_t* __restrict__ in1, uint16_t* __restrict__ out1, int C) {
   __shared__ uint16_t tile[64][66];
   pdl_wait();
-  const long long ntt = Tp / 64;
-  const int nct = C / 64, tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
-  for (long long blk = blockIdx.x; blk < ntt * nct; blk += gridDim.x) {
-    const long long tt = blk / nct;
-    const int ct = static_cast<int>(blk - tt * nct);
-    for (int r = ty; r < 64; r += TR_THREADS / 64) {
-      const long long t = tt * 64 + r;
-      tile[r][tx] = t < T ? in[t * C + ct * 64 + tx] : static_cast<uint16_t>(0);
-    }
-    __syncthreads();
-    for (int r = ty; r < 64; r += TR_THREADS / 64) out[static_cast<long long>(ct * 64 + r) * Tp + tt * 64 + tx] = tile[tx][r];
-    __syncthreads();
-  }
+  const int n = C / 64, blk = blockIdx.x % (n * n), tx = threadIdx.x & 63, ty = threadIdx.x >> 6;
+  const int r0 = 64 * (blk / n), c0 = 64 * (blk % n);
+  const uint16_t* in = static_cast<int>(blockIdx.x) < n * n ? in0 : in1;
+  uint16_t* out = static_cast<int>(blockIdx.x) < n * n ? out0 : out1;
+#pragma unroll
+  for (int r = ty; r < 64; r += TR_THREADS / 64) tile[r][tx] = in[(r0 + r) * C + c0 + tx];
+  __syncthreads();
+#pragma unroll
+  for (int r = ty; r < 64; r += TR_THREADS / 64) out[(c0 + r) * C + r0 + tx] = tile[tx][r];
   pdl_trigger();
 }
 
-// Partial weight gradient of token chunk blockIdx.x: part[chunk][o][i] = sum over the chunk's
-// tokens t of A[t][o] B[t][i], with A and B the [T, C] token rows as given.  C in {64, 128, 256}.
-//
-// A K tile of KT = 64 tokens of an operand becomes C rows (channels) of 128 bytes (64 tokens) in
-// the tensor core's 128-byte-swizzled K-major layout: in each 1024-byte group of 8 rows, the
-// 16-byte chunk j (tokens 8j .. 8j + 7) of row r sits at chunk position j ^ (r mod 8).  Thread
-// work item (r8, k) reads the 8 x 8 block of channels 8 r8 .. + 7 and tokens 8 k .. + 7 as eight
-// 16-byte token rows, transposes it in registers (byte permutes of token pairs) and writes the
-// eight 16-byte channel rows; the eight items of a row group land in eight different bank groups.
+// Shared-memory descriptor of an M- or N-major operand in 128-byte-swizzled panels of 64 channels (rows of 128 bytes, one
+// token each; 16-byte chunk j of token t at chunk j ^ (t mod 8)): `panel` bytes to the next 64 channels, 1024 to the next 8
+// tokens.
+__device__ __forceinline__ uint64_t mn_desc(uint32_t addr, uint32_t panel) {
+  return static_cast<uint64_t>((addr & 0x3FFFFu) >> 4) | (static_cast<uint64_t>(panel >> 4) << 16) |
+         (static_cast<uint64_t>(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
+}
+// instr_desc with A and B M- and N-major
+constexpr uint32_t MN_MAJOR = (1u << 15) | (1u << 16);
+
+template <int C>
+struct Wg {
+  static constexpr int MT = C > 128 ? C / 128 : 1;             // MMA tiles of 128 output rows
+  static constexpr uint32_t PANEL = KT * 128, OPERAND = C / 64 * PANEL, STAGE = 2 * OPERAND;
+  static constexpr int STAGES = C == 256 ? 3 : 6;
+  static constexpr size_t SMEM = STAGES * STAGE + 1024 > SMEM_MIN ? STAGES * STAGE + 1024 : SMEM_MIN;  // 1024: alignment slack
+  static constexpr uint32_t TCOLS = MT * C;                    // 64, 128 or 512 TMEM columns
+};
+
+// Partial weight gradient of token chunk blockIdx.x: part[chunk][o][i] = sum over the chunk's tokens t of A[t][o] B[t][i], with A
+// and B the [T, C] token rows as given.  C in {64, 128, 256}.
 template <int C>
 __global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad(const uint16_t* __restrict__ A, const uint16_t* __restrict__ B,
                                                          float* __restrict__ part, long long T, int nchunk,
                                                          unsigned int* err) {
-  constexpr int MT = C > 128 ? C / 128 : 1;          // MMA tiles of 128 output rows
-  constexpr int AR = MT * 128;                       // staged A rows (rows >= C stay zero)
-  constexpr uint32_t A_BYTES = AR * KT * 2, B_BYTES = C * KT * 2, STAGE = A_BYTES + B_BYTES;
-  constexpr uint32_t TCOLS = MT * C;                 // 64, 128 or 512 TMEM columns
-  constexpr int ITEMS = C / WG_THREADS > 0 ? C / WG_THREADS : 1;  // 8 x 8 blocks per operand per thread
+  using G = Wg<C>;
+  constexpr int MT = G::MT, S = G::STAGES;
+  constexpr uint32_t TCOLS = G::TCOLS;
   static_assert(C == 64 || C == 128 || C == 256, "channels");
   extern __shared__ __align__(1024) unsigned char smem_raw[];
-  __shared__ uint64_t mbar[2];
+  __shared__ uint64_t mbar[S];
   __shared__ uint32_t tmem_slot;
   // the swizzle pattern is a function of the address: stage buffers start on 1024-byte boundaries
-  unsigned char* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
+  const uint32_t smem = (smem_u32(smem_raw) + 1023u) & ~1023u;
   const int tid = threadIdx.x, warp = tid >> 5;
   if (tid < 32) tmem_alloc(&tmem_slot, TCOLS);
   if (tid == 0) {
-    mbar_init(&mbar[0], 1);
-    mbar_init(&mbar[1], 1);
+    for (int i = 0; i < S; ++i) mbar_init(&mbar[i], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  }
-  if constexpr (AR > C) {  // A rows C .. AR - 1 of both buffers: zero once, never written again
-    for (int q = tid; q < 2 * (AR - C) * 8; q += WG_THREADS) {
-      const int b = q / ((AR - C) * 8), rem = q % ((AR - C) * 8);
-      *reinterpret_cast<uint4*>(smem + b * STAGE + C * 128 + rem * 16) = make_uint4(0u, 0u, 0u, 0u);
-    }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -96,89 +93,54 @@ __global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad(const uint16_t* __restr
   const uint32_t tmem = tmem_slot;
   const long long ntiles = (T + KT - 1) / KT;
   const long long k0 = ntiles * blockIdx.x / nchunk, k1 = ntiles * (blockIdx.x + 1) / nchunk;
-  const bool has_item = tid < C;  // C work items per operand and tile: C = 64 leaves threads 64 .. 127 idle
+  const int n = static_cast<int>(k1 - k0);
 
-  // the 8 x 8 blocks of tile kt, item n of this thread: n-th work item tid + 128 n = 8 r8 + k
-  uint4 ra[ITEMS][8], rb[ITEMS][8];
-  auto load = [&](long long kt) {
+  auto load = [&](int i) {  // tile i of the chunk into stage i mod S; tokens past T are zero
+    if (i < n) {
+      const uint32_t st = smem + (i % S) * G::STAGE;
 #pragma unroll
-    for (int n = 0; n < ITEMS; ++n) {
-      const int item = tid + WG_THREADS * n, r8 = item >> 3, k = item & 7;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const long long t = kt * KT + 8 * k + j;
-        const bool live = has_item && t < T;
-        const long long off = (live ? t : 0) * C + 8 * r8;
-        ra[n][j] = live ? __ldcs(reinterpret_cast<const uint4*>(A + off)) : make_uint4(0u, 0u, 0u, 0u);
-        rb[n][j] = live ? __ldcs(reinterpret_cast<const uint4*>(B + off)) : make_uint4(0u, 0u, 0u, 0u);
+      for (int j = 0; j < C * KT / 8 / WG_THREADS; ++j) {
+        const int q = tid + WG_THREADS * j, tok = q / (C / 8), c = q % (C / 8);
+        const long long t = (k0 + i) * KT + tok;
+        const bool in = t < T;
+        const long long off = (in ? t : 0) * C + 8 * c;
+        const uint32_t d = st + (c >> 3) * G::PANEL + tok * 128 + (((c & 7) ^ (tok & 7)) << 4);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(A + off), "r"(in ? 16 : 0) : "memory");
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d + G::OPERAND), "l"(B + off), "r"(in ? 16 : 0) : "memory");
       }
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  // transpose one 8 x 8 block (v[j] = token j's 8 channels) and store its 8 channel rows
-  auto put = [&](unsigned char* base, const uint4 (&v)[8], int r8, int k) {
-    uint32_t o[8][4];
-#pragma unroll
-    for (int j = 0; j < 8; j += 2) {
-      const uint32_t a[4] = {v[j].x, v[j].y, v[j].z, v[j].w}, b[4] = {v[j + 1].x, v[j + 1].y, v[j + 1].z, v[j + 1].w};
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        o[2 * q][j / 2] = __byte_perm(a[q], b[q], 0x5410);      // channel 2q, tokens j, j + 1
-        o[2 * q + 1][j / 2] = __byte_perm(a[q], b[q], 0x7632);  // channel 2q + 1, tokens j, j + 1
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < 8; ++c)
-      *reinterpret_cast<uint4*>(base + (r8 * 8 + c) * 128 + ((k ^ c) << 4)) = make_uint4(o[c][0], o[c][1], o[c][2], o[c][3]);
-  };
-  auto store = [&](int buf) {
-    unsigned char* sa = smem + buf * STAGE;
-    unsigned char* sb = sa + A_BYTES;
-    if (has_item) {
-#pragma unroll
-      for (int n = 0; n < ITEMS; ++n) {
-        const int item = tid + WG_THREADS * n;
-        put(sa, ra[n], item >> 3, item & 7);
-        put(sb, rb[n], item >> 3, item & 7);
-      }
-    }
-    // generic-proxy shared-memory writes -> visible to the tensor core (async proxy)
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  };
+  // the products of tile i have completed (all threads; false if the wait gave up)
+  auto done = [&](int i) { return __syncthreads_and(mbar_wait(&mbar[i % S], (i / S) & 1) ? 1 : 0) != 0; };
 
-  const uint32_t idesc = instr_desc(128, C);
-  uint32_t parity[2] = {0u, 0u};
+  const uint32_t idesc = instr_desc(128, C) | MN_MAJOR;
   bool ok = true;
-  if (k1 > k0) load(k0);
-  for (long long kt = k0; kt < k1; ++kt) {
-    const int buf = static_cast<int>((kt - k0) & 1);
-    if (kt - k0 >= 2) {  // buffer buf is free once the MMAs of tile kt - 2 (its last reader) completed
-      ok = __syncthreads_and(mbar_wait(&mbar[buf], parity[buf]) ? 1 : 0) != 0;
-      parity[buf] ^= 1u;
-      if (!ok) break;
-    }
-    store(buf);
-    if (kt + 1 < k1) load(kt + 1);  // in flight while this tile is handed to the tensor core
+  for (int i = 0; i < S - 1; ++i) load(i);
+  for (int i = 0; i < n; ++i) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(S - 2) : "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
     if (tid == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t sa = smem_u32(smem + buf * STAGE), sb = sa + A_BYTES;
+      const uint32_t sa = smem + (i % S) * G::STAGE, sb = sa + G::OPERAND;
 #pragma unroll
       for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-        for (int ks = 0; ks < KT / 16; ++ks)  // K steps of 16 tokens: 32 bytes along the swizzled rows
-          mma_bf16(tmem + mt * C, sw128_desc(sa + mt * (128 * 128) + ks * 32), sw128_desc(sb + ks * 32), idesc,
-                   (kt > k0 || ks > 0) ? 1u : 0u);
-      mma_commit(&mbar[buf]);
+        for (int ks = 0; ks < KT / 16; ++ks)  // K steps of 16 tokens: 2048 bytes down the panels
+          // (C = 64: rows 64 .. 127 of the product read the only panel again and are not used)
+          mma_bf16(tmem + mt * C, mn_desc(sa + 2 * mt * G::PANEL + ks * 2048, C > 64 ? G::PANEL : 0),
+                   mn_desc(sb + ks * 2048, C > 64 ? G::PANEL : 0), idesc, (i > 0 || ks > 0) ? 1u : 0u);
+      mma_commit(&mbar[i % S]);
     }
-  }
-  if (ok && k1 > k0) {  // the last two tiles' commits cover every MMA issued
-    const long long n = k1 - k0;
-    for (long long kt = (n >= 2 ? k1 - 2 : k0); kt < k1 && ok; ++kt) {
-      const int b = static_cast<int>((kt - k0) & 1);
-      ok = __syncthreads_and(mbar_wait(&mbar[b], parity[b]) ? 1 : 0) != 0;
-      parity[b] ^= 1u;
+    if (i + S - 1 < n && i > 0) {  // the stage of tile i - 1 is next
+      ok = done(i - 1);
+      if (!ok) break;
     }
+    load(i + S - 1);
   }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  if (ok && n > 0) ok = done(n - 1);  // the last commit covers every product issued before it
   if (!ok && tid == 0) atomicOr(err, 1u << 13);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   // row o = mt * 128 + tid of the accumulator -> this chunk's partial (zeros for an empty chunk)
@@ -195,7 +157,7 @@ __global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad(const uint16_t* __restr
         float4* dst = reinterpret_cast<float4*>(pc + static_cast<long long>(o) * C + c0);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const bool live = ok && k1 > k0;
+          const bool live = ok && n > 0;
           dst[q] = live ? make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]) : make_float4(0.f, 0.f, 0.f, 0.f);
         }
       }
@@ -255,21 +217,17 @@ int wgrad_chunks(long long T, int sms) {
   return static_cast<int>(nt < sms ? (nt < 1 ? 1 : nt) : sms);
 }
 
-cudaError_t transpose(const void* in, void* out, long long T, int C, long long Tp, int sms, cudaStream_t stream) {
-  const long long blocks = (Tp / 64) * (C / 64);
-  const unsigned grid = static_cast<unsigned>(blocks < 8ll * sms ? (blocks < 1 ? 1 : blocks) : 8ll * sms);
-  const uint16_t* i = static_cast<const uint16_t*>(in);
-  uint16_t* o = static_cast<uint16_t*>(out);
-  void* args[] = {&i, &o, &T, &C, &Tp};
-  return launch_pdl(reinterpret_cast<const void*>(k_transpose), grid, TR_THREADS, 0, stream, args);
+cudaError_t transpose2(const void* in0, void* out0, const void* in1, void* out1, int C, cudaStream_t stream) {
+  const uint16_t *i0 = static_cast<const uint16_t*>(in0), *i1 = static_cast<const uint16_t*>(in1);
+  uint16_t *o0 = static_cast<uint16_t*>(out0), *o1 = static_cast<uint16_t*>(out1);
+  void* args[] = {&i0, &o0, &i1, &o1, &C};
+  return launch_pdl(reinterpret_cast<const void*>(k_transpose2), static_cast<unsigned>(2 * (C / 64) * (C / 64)), TR_THREADS, 0, stream, args);
 }
 
 template <int C>
 cudaError_t wgrad_c(const void* a_tok, const void* b_tok, float* part, float* out, long long T, int sms, unsigned int* err,
                     cudaStream_t stream) {
-  constexpr int MT = C > 128 ? C / 128 : 1;
-  constexpr size_t need = 2ull * (MT * 128 + C) * KT * 2 + 1024;  // two stages, 1024-byte alignment slack
-  const size_t smem = need > SMEM_MIN ? need : SMEM_MIN;
+  constexpr size_t smem = Wg<C>::SMEM;
   const void* k = reinterpret_cast<const void*>(k_wgrad<C>);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;

@@ -41,7 +41,7 @@ cudaError_t project(const void* x, const void* w, void* z, long long T, int C, b
 namespace bbwd {
 // whtmix_block_bwd.cu: the block backward's weight transposes and weight gradients on the tensor cores
 int wgrad_chunks(long long T, int sms);
-cudaError_t transpose(const void* in, void* out, long long T, int C, long long Tp, int sms, cudaStream_t stream);
+cudaError_t transpose2(const void* in0, void* out0, const void* in1, void* out1, int C, cudaStream_t stream);
 cudaError_t wgrad(const void* a_tok, const void* b_tok, float* part, float* out, long long T, int C, int sms,
                   unsigned int* err, cudaStream_t stream);
 }  // namespace bbwd
@@ -995,12 +995,12 @@ int whtmix_block_backward(const void* x, const void* w_in, const void* gains, co
   }
   rc = device_check(&dev, &sms);
   if (rc != WHTMIX_OK) return rc;
-  // slot-1 layout: Z, M, dM [T, C] bf16; a transposed weight [C, C] bf16; the per-chunk partials
+  // slot-1 layout: Z, M, dM [T, C] bf16; the transposed weights [C, C] bf16; the per-chunk partials
   // [chunks, C, C] fp32 of a weight gradient
   const int chunks = bbwd::wgrad_chunks(T, sms);
-  size_t off[5], total = 0;
-  const size_t sizes[5] = {pb, pb, pb, wb, static_cast<size_t>(chunks) * wgb};
-  for (int i = 0; i < 5; ++i) {
+  size_t off[6], total = 0;
+  const size_t sizes[6] = {pb, pb, pb, wb, wb, static_cast<size_t>(chunks) * wgb};
+  for (int i = 0; i < 6; ++i) {
     off[i] = total;
     total += align256(sizes[i]);
   }
@@ -1008,8 +1008,8 @@ int whtmix_block_backward(const void* x, const void* w_in, const void* gains, co
   rc = cached_workspace(dev, stream, total, &w1, 1);
   if (rc != WHTMIX_OK) return rc;
   char* base = static_cast<char*>(w1);
-  void *Z = base + off[0], *M = base + off[1], *dM = base + off[2], *WT = base + off[3];
-  float* part = reinterpret_cast<float*>(base + off[4]);
+  void *Z = base + off[0], *M = base + off[1], *dM = base + off[2], *WoT = base + off[3], *WiT = base + off[4];
+  float* part = reinterpret_cast<float*>(base + off[5]);
   auto err_word = [&](unsigned int** e) -> int {  // the slot-0 header's error word, read by whtmix_sync
     void* w0 = nullptr;
     const int r = cached_workspace(dev, stream, HEADER_BYTES, &w0, 0);
@@ -1028,12 +1028,12 @@ int whtmix_block_backward(const void* x, const void* w_in, const void* gains, co
     e = (call);                            \
     if (e != cudaSuccess) return cuda_fail(e); \
   } while (0)
+  WHTMIX_CUDA_STEP(bbwd::transpose2(w_out, WoT, w_in, WiT, static_cast<int>(C), stream));
   // Eq. 1 and the mixer: Z = X W_in^T, M = mix(Z) (bf16 activations, as the forward's)
   WHTMIX_STEP(whtmix_project(x, w_in, Z, T, C, WHTMIX_BF16, stream));
   WHTMIX_STEP(run(full_call(false, Z, gains, nullptr, M, nullptr, B, N, N, C, dtype), nullptr, 0, false, stream));
   // Eq. 4 backward: dM = dY W_out (the projection with W_out^T), dW_out = dY^T M
-  WHTMIX_CUDA_STEP(bbwd::transpose(w_out, WT, C, static_cast<int>(C), C, sms, stream));
-  WHTMIX_STEP(whtmix_project(dy, WT, dM, T, C, WHTMIX_BF16, stream));
+  WHTMIX_STEP(whtmix_project(dy, WoT, dM, T, C, WHTMIX_BF16, stream));
   WHTMIX_STEP(err_word(&err));
   WHTMIX_CUDA_STEP(bbwd::wgrad(dy, M, part, static_cast<float*>(dw_out), T, static_cast<int>(C), sms, err, stream));
   // the mixer's backward: dZ (into dx) and dG
@@ -1041,8 +1041,7 @@ int whtmix_block_backward(const void* x, const void* w_in, const void* gains, co
   // Eq. 1 backward: dW_in = dZ^T X, then dX = dZ W_in in place
   WHTMIX_STEP(err_word(&err));
   WHTMIX_CUDA_STEP(bbwd::wgrad(dx, x, part, static_cast<float*>(dw_in), T, static_cast<int>(C), sms, err, stream));
-  WHTMIX_CUDA_STEP(bbwd::transpose(w_in, WT, C, static_cast<int>(C), C, sms, stream));
-  WHTMIX_STEP(whtmix_project(dx, WT, dx, T, C, WHTMIX_BF16, stream));
+  WHTMIX_STEP(whtmix_project(dx, WiT, dx, T, C, WHTMIX_BF16, stream));
 #undef WHTMIX_STEP
 #undef WHTMIX_CUDA_STEP
   return WHTMIX_OK;
