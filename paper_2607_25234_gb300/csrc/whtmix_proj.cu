@@ -10,8 +10,8 @@
 // stores it.  Both operands are K-major (X rows are tokens with their channels contiguous, W rows
 // are output channels with their input channels contiguous), laid out in shared memory as the
 // tensor core's no-swizzle canonical form: 8-row x 16-byte core matrices, the K-adjacent core
-// matrix 128 bytes on, the next group of 8 rows (C / 8) x 128 bytes on.  bf16 output at C = 64 and
-// 128 takes the pipelined, warp-specialised k_proj_pipe below instead (TMA in and out).
+// matrix 128 bytes on, the next group of 8 rows (C / 8) x 128 bytes on.  bf16 output takes
+// other kernels below: the pipelined, warp-specialised k_proj_pipe (TMA in and out) at C = 64 and 128, k_proj_wide at 256.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -40,10 +40,15 @@ __global__ void __launch_bounds__(THREADS, 1) k_proj(const __nv_bfloat16* x, con
   unsigned char* sw = smem;                     // W: C x C bf16, canonical layout
   unsigned char* sx = smem + C * C * 2;         // X tile: 128 x C bf16, canonical layout
   const int tid = threadIdx.x;
+  // 16 bytes to shared memory, zeros if not `in`; every copy of W and of a tile is in flight at once (through registers, four
+  // at a time, C = 256 spent 15 of its 21 us on W)
+  auto copy16 = [](uint32_t dst, const void* src, bool in) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+  };
   // W once per CTA
   for (int i = tid; i < C * C / 8; i += THREADS) {
     const int r = i / (C / 8), k = (i % (C / 8)) * 8;
-    *reinterpret_cast<uint4*>(sw + core_off(r, k, C)) = *reinterpret_cast<const uint4*>(w + static_cast<long long>(r) * C + k);
+    copy16(smem_u32(sw) + core_off(r, k, C), w + static_cast<long long>(r) * C + k, true);
   }
   if (tid < 32) tmem_alloc(&tmem_slot, C);
   if (tid == 0) {
@@ -64,10 +69,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_proj(const __nv_bfloat16* x, con
     // X tile; tokens past T are zero
     for (int i = tid; i < TILE_T * C / 8; i += THREADS) {
       const int r = i / (C / 8), k = (i % (C / 8)) * 8;
-      uint4 v = make_uint4(0u, 0u, 0u, 0u);
-      if (t0 + r < T) v = *reinterpret_cast<const uint4*>(x + (t0 + r) * C + k);
-      *reinterpret_cast<uint4*>(sx + core_off(r, k, C)) = v;
+      const bool in = t0 + r < T;
+      copy16(smem_u32(sx) + core_off(r, k, C), x + (in ? t0 + r : 0) * C + k, in);
     }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     // generic-proxy shared-memory writes -> visible to the tensor core (async proxy)
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     __syncthreads();
@@ -289,6 +294,107 @@ __global__ void __launch_bounds__(P2_THREADS, 1) k_proj_pipe(const __grid_consta
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * C) : "memory");
 }
 
+// C = 256, bf16 out: the transposed product Z^T = W X^T, so that a warp's lanes are 32 consecutive output channels and its
+// stores whole 64-byte segments.  256 threads, a persistent CTA per SM; W (two M tiles of 128 channels, K = 256) stays in
+// shared memory, tiles of 64 tokens (N) pass through three stages; both K-major in 128-byte-swizzled panels of 64 k.  Warps 0-3
+// take the first M tile's accumulator, 4-7 the second's.  Against k_proj, whose lanes are tokens (512-byte strides) and whose
+// staging is 32-way bank-conflicted at this width: 16384 tokens (17 MB) 20.5 -> 8.9 us.
+constexpr int PW_THREADS = 256, PW_T = 64, PW_STAGES = 3;
+constexpr int PW_C = 256, PW_WPANEL = PW_C * 128, PW_XPANEL = PW_T * 128, PW_STAGE = 4 * PW_XPANEL;
+constexpr size_t PW_SMEM = 4 * PW_WPANEL + PW_STAGES * PW_STAGE;
+__global__ void __launch_bounds__(PW_THREADS, 1) k_proj_wide(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ w,
+                                                             __nv_bfloat16* z, long long T, unsigned int* err) {  // z may be x
+  extern __shared__ __align__(1024) unsigned char smem[];
+  __shared__ uint64_t mbar[2];
+  __shared__ uint32_t tmem_slot;
+  const int tid = threadIdx.x, warp = tid >> 5;
+  if (tid < 32) tmem_alloc(&tmem_slot, 256);  // two accumulators of 2 x 64 columns
+  if (tid == 0) {
+    mbar_init(&mbar[0], 1);
+    mbar_init(&mbar[1], 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  pdl_wait();
+  const uint32_t sw = smem_u32(smem), sx = sw + 4 * PW_WPANEL;
+  // 16-byte chunk q of a [rows, 256] operand (32 a row) in panels of `panel` bytes
+  auto place = [](int q, int panel) {
+    const int r = q >> 5, c = q & 31;
+    return static_cast<uint32_t>((c >> 3) * panel + r * 128 + (((c & 7) ^ (r & 7)) << 4));
+  };
+  auto copy16 = [](uint32_t dst, const void* src, bool in) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(in ? 16 : 0) : "memory");
+  };
+  const long long ntiles = (T + PW_T - 1) / PW_T;
+  const int n = blockIdx.x < ntiles ? static_cast<int>((ntiles - blockIdx.x + gridDim.x - 1) / gridDim.x) : 0;
+  auto first_token = [&](int i) { return (blockIdx.x + static_cast<long long>(i) * gridDim.x) * PW_T; };
+  auto load = [&](int i) {
+    if (i < n) {
+      const long long t0 = first_token(i);
+#pragma unroll
+      for (int j = 0; j < PW_T * 32 / PW_THREADS; ++j) {
+        const int q = tid + PW_THREADS * j;
+        const bool in = t0 + (q >> 5) < T;
+        copy16(sx + (i % PW_STAGES) * PW_STAGE + place(q, PW_XPANEL), x + (in ? t0 * PW_C + 8ll * q : 0), in);
+      }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+#pragma unroll
+  for (int j = 0; j < PW_C * 32 / PW_THREADS; ++j) {
+    const int q = tid + PW_THREADS * j;
+    copy16(sw + place(q, PW_WPANEL), w + 8ll * q, true);
+  }
+  load(0);
+  load(1);
+  const uint32_t tmem = tmem_slot;
+  bool ok = true;
+  for (int i = 0; i < n && ok; ++i) {
+    asm volatile("cp.async.wait_group 1;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (tid == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t st = sx + (i % PW_STAGES) * PW_STAGE;
+#pragma unroll
+      for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+        for (int ks = 0; ks < PW_C / 16; ++ks)
+          mma_bf16(tmem + 128 * (i & 1) + 64 * mt, sw128_desc(sw + (ks >> 2) * PW_WPANEL + mt * (128 * 128) + (ks & 3) * 32),
+                   sw128_desc(st + (ks >> 2) * PW_XPANEL + (ks & 3) * 32), instr_desc(128, PW_T), ks > 0 ? 1u : 0u);
+      mma_commit(&mbar[i & 1]);
+    }
+    load(i + 2);  // into the stage of tile i - 1, whose products every thread has waited for
+    ok = __syncthreads_and(mbar_wait(&mbar[i & 1], (i >> 1) & 1) ? 1 : 0) != 0;
+    if (!ok) {
+      if (tid == 0) atomicOr(err, 1u);
+      break;
+    }
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const long long t0 = first_token(i);
+    const uint32_t d = tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + 128 * (i & 1) + 64 * (warp >> 2);
+    __nv_bfloat16* o = z + t0 * PW_C + tid;  // lane = output channel tid
+#pragma unroll
+    for (int c0 = 0; c0 < PW_T; c0 += 16) {
+      float v[16];
+      tmem_ld16(d + c0, v);
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+      for (int k = 0; k < 16; ++k)
+        if (t0 + c0 + k < T) o[(c0 + k) * PW_C] = __float2bfloat16_rn(v[k]);
+    }
+  }
+  asm volatile("cp.async.wait_group 0;" ::: "memory");
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  pdl_trigger();
+  if (tid < 32) tmem_dealloc(tmem, 256);
+}
+
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link against libcuda).
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
@@ -347,6 +453,16 @@ cudaError_t launch_c(const void* x, const void* w, void* z, long long T, unsigne
   return cudaGetLastError();
 }
 
+cudaError_t launch_wide(const void* x, const void* w, void* z, long long T, unsigned int* err, int sms, cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(k_proj_wide, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(PW_SMEM));
+  if (e != cudaSuccess) return e;
+  const long long ntiles = (T + PW_T - 1) / PW_T;
+  const __nv_bfloat16 *xb = static_cast<const __nv_bfloat16*>(x), *wb = static_cast<const __nv_bfloat16*>(w);
+  __nv_bfloat16* zb = static_cast<__nv_bfloat16*>(z);
+  void* args[] = {&xb, &wb, &zb, &T, &err};
+  return launch_pdl(reinterpret_cast<const void*>(k_proj_wide), static_cast<unsigned>(ntiles < sms ? ntiles : sms), PW_THREADS, PW_SMEM, s, args);
+}
+
 // Z = X W^T for T tokens of C channels (C = 64, 128 or 256); err: device word set on a timeout.
 cudaError_t project(const void* x, const void* w, void* z, long long T, int C, bool out_f32, unsigned int* err, int sms,
                     cudaStream_t s) {
@@ -358,7 +474,7 @@ cudaError_t project(const void* x, const void* w, void* z, long long T, int C, b
   switch (C) {
     case 64: return out_f32 ? launch_c<64, true>(x, w, z, T, err, sms, s) : launch_c<64, false>(x, w, z, T, err, sms, s);
     case 128: return out_f32 ? launch_c<128, true>(x, w, z, T, err, sms, s) : launch_c<128, false>(x, w, z, T, err, sms, s);
-    case 256: return out_f32 ? launch_c<256, true>(x, w, z, T, err, sms, s) : launch_c<256, false>(x, w, z, T, err, sms, s);
+    case 256: return out_f32 ? launch_c<256, true>(x, w, z, T, err, sms, s) : launch_wide(x, w, z, T, err, sms, s);
     default: return cudaErrorInvalidValue;
   }
 }

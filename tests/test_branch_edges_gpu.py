@@ -91,6 +91,25 @@ def test_fused_block(B, N, C):
     assert (np.abs(got - ref) <= bound).all(), float(np.max(np.abs(got - ref) / bound))
 
 
+# C = 256 to bf16, tiles of 64 tokens through three stages: one token, the edges of a tile, and two, three and four tiles a CTA
+@pytest.mark.parametrize("T", [1, 63, 64, 65, 152 * 64 + 1, 2 * 152 * 64 + 77, 3 * 152 * 64 + 64])
+def test_wide_projection(T):
+    C = 256
+    x, w = inputs.normal(60, T * C).reshape(T, C), (inputs.normal(61, C * C) / 16).reshape(C, C)
+    xd, wd = bf16_dev(x.astype(np.float32)), bf16_dev(w.astype(np.float32))
+    z = Guarded((T, C), torch.bfloat16)
+    whtmix.project(xd, wd, out=z.t)
+    own = xd.clone()
+    whtmix.project(own, wd, out=own)
+    whtmix.sync()
+    z.assert_intact("Z")
+    assert torch.equal(own, z.t)
+    xe, we = xd.double().cpu().numpy(), wd.double().cpu().numpy()
+    want, got = xe @ we.T, z.t.double().cpu().numpy()
+    tol = np.abs(want) * 2.0 ** -8 + 1e-6 * (np.abs(xe) @ np.abs(we).T)  # half an ulp of bf16, and the fp32 sum
+    assert (np.abs(got - want) <= tol).all(), float(np.max(np.abs(got - want) / tol))
+
+
 def run_padded(B, n, N, C, dtype, backward):
     d = inputs.make_inputs(B, N, C, dtype, seed=n + N, n_valid=n, with_dy=backward)
     x, g = to_dev(d["x"], dtype)[:, :n].contiguous(), to_dev(d["g"], "f32")
