@@ -7,9 +7,9 @@
 // CTA (one persistent CTA per SM, 128 threads): K tiles of 64 tokens of both operands are copied as they are by 16-byte
 // cp.async into 128-byte-swizzled panels of 64 channels, up to five tiles ahead, and multiplied from there as
 // M-major and N-major operands (the channels are contiguous, the contraction runs down the panel's rows), so nothing is
-// transposed; one thread issues tcgen05.mma (kind::f16, M = 128, N = C, K = 16) into a TMEM accumulator per 128 rows of
-// o.  Each thread then reads its row o of the accumulator (tcgen05.ld) into the chunk's fp32 partial [C, C];
-// k_wgrad_reduce adds the partials in a fixed order, so dW is the same bit for bit on every run.
+// transposed; one thread issues tcgen05.mma (kind::f16, M = 128, N = C, K = 16) into a TMEM accumulator per 128 input
+// channels i.  A lane of the accumulator is an i, a column an o, so that a warp stores 32 consecutive floats of the chunk's
+// fp32 partial [C, C] at a time (with the roles swapped, 32 rows at a stride: 16384 tokens of 256 channels 16.9 us, so 11.8); k_wgrad_reduce adds the partials in a fixed order, so dW is the same bit for bit on every run.
 // A chunk is a few tiles (3.4 at 32768 tokens), so its time is the latency of its chain: with 8 x 8 transposes in registers
 // and one tile ahead it took 13.2 us, now 9.0 (32768 tokens, C = 128; whole block_train step [8, 4096, 128] 140 -> 124).
 #include <cuda_bf16.h>
@@ -25,7 +25,7 @@ namespace bbwd {
 using namespace tc;
 
 constexpr int KT = 64;             // tokens per K tile (one 128-byte row of bf16 per operand row)
-constexpr int WG_THREADS = 128;    // one thread per TMEM lane = per output row o of an MMA tile
+constexpr int WG_THREADS = 128;    // one thread per TMEM lane
 constexpr int TR_THREADS = 256;
 constexpr size_t SMEM_MIN = 120 * 1024;  // more than half an SM: one CTA per SM, so TMEM allocation never waits
 
@@ -58,7 +58,7 @@ constexpr uint32_t MN_MAJOR = (1u << 15) | (1u << 16);
 
 template <int C>
 struct Wg {
-  static constexpr int MT = C > 128 ? C / 128 : 1;             // MMA tiles of 128 output rows
+  static constexpr int MT = C > 128 ? C / 128 : 1;             // MMA tiles of 128 input channels
   static constexpr uint32_t PANEL = KT * 128, OPERAND = C / 64 * PANEL, STAGE = 2 * OPERAND;
   static constexpr int STAGES = C == 256 ? 3 : 6;
   static constexpr size_t SMEM = STAGES * STAGE + 1024 > SMEM_MIN ? STAGES * STAGE + 1024 : SMEM_MIN;  // 1024: alignment slack
@@ -129,8 +129,8 @@ __global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad(const uint16_t* __restr
 #pragma unroll
         for (int ks = 0; ks < KT / 16; ++ks)  // K steps of 16 tokens: 2048 bytes down the panels
           // (C = 64: rows 64 .. 127 of the product read the only panel again and are not used)
-          mma_bf16(tmem + mt * C, mn_desc(sa + 2 * mt * G::PANEL + ks * 2048, C > 64 ? G::PANEL : 0),
-                   mn_desc(sb + ks * 2048, C > 64 ? G::PANEL : 0), idesc, (i > 0 || ks > 0) ? 1u : 0u);
+          mma_bf16(tmem + mt * C, mn_desc(sb + 2 * mt * G::PANEL + ks * 2048, C > 64 ? G::PANEL : 0),
+                   mn_desc(sa + ks * 2048, C > 64 ? G::PANEL : 0), idesc, (i > 0 || ks > 0) ? 1u : 0u);
       mma_commit(&mbar[i % S]);
     }
     if (i + S - 1 < n && i > 0) {  // the stage of tile i - 1 is next
@@ -143,23 +143,20 @@ __global__ void __launch_bounds__(WG_THREADS, 1) k_wgrad(const uint16_t* __restr
   if (ok && n > 0) ok = done(n - 1);  // the last commit covers every product issued before it
   if (!ok && tid == 0) atomicOr(err, 1u << 13);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  // row o = mt * 128 + tid of the accumulator -> this chunk's partial (zeros for an empty chunk)
+  // lane i = mt * 128 + tid, column o of the accumulator -> this chunk's partial (zeros for an empty chunk)
   float* pc = part + static_cast<long long>(blockIdx.x) * C * C;
-#pragma unroll 1
+  const bool live = ok && n > 0;
+#pragma unroll
   for (int mt = 0; mt < MT; ++mt) {
-    const int o = mt * 128 + tid;
-#pragma unroll 1
+    const int i = mt * 128 + tid;
+#pragma unroll 4
     for (int c0 = 0; c0 < C; c0 += 16) {
       float v[16];
       tmem_ld16(tmem + (static_cast<uint32_t>(32 * warp) << 16) + mt * C + c0, v);
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-      if (o < C) {
-        float4* dst = reinterpret_cast<float4*>(pc + static_cast<long long>(o) * C + c0);
+      if (i < C) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const bool live = ok && n > 0;
-          dst[q] = live ? make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
+        for (int q = 0; q < 16; ++q) pc[(c0 + q) * C + i] = live ? v[q] : 0.f;
       }
     }
   }
@@ -211,10 +208,12 @@ __global__ void __launch_bounds__(TR_THREADS) k_wgrad_reduce(const float4* __res
 
 // ---- host ----
 
-// Token chunks of one weight gradient over T tokens: one per SM, at most one per K tile.
-int wgrad_chunks(long long T, int sms) {
-  const long long nt = (T + KT - 1) / KT;
-  return static_cast<int>(nt < sms ? (nt < 1 ? 1 : nt) : sms);
+// Token chunks of one weight gradient over T tokens: one per SM, and at least C / 64 K tiles a chunk: a partial is C / 64 times a
+// tile's size or more, and is written and read again (C = 256, 16384 tokens: k_wgrad 18.8
+// us and its reduction 9.6 with 152 chunks, 16.9 and 5.9 with 64).
+int wgrad_chunks(long long T, int C, int sms) {
+  const long long nt = (T + KT - 1) / KT, most = (nt + C / 64 - 1) / (C / 64);
+  return static_cast<int>(most < sms ? (most < 1 ? 1 : most) : sms);
 }
 
 cudaError_t transpose2(const void* in0, void* out0, const void* in1, void* out1, int C, cudaStream_t stream) {
@@ -231,7 +230,7 @@ cudaError_t wgrad_c(const void* a_tok, const void* b_tok, float* part, float* ou
   const void* k = reinterpret_cast<const void*>(k_wgrad<C>);
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  int nchunk = wgrad_chunks(T, sms);
+  int nchunk = wgrad_chunks(T, C, sms);
   const uint16_t* a = static_cast<const uint16_t*>(a_tok);
   const uint16_t* b = static_cast<const uint16_t*>(b_tok);
   void* args[] = {&a, &b, &part, &T, &nchunk, &err};
@@ -246,7 +245,7 @@ cudaError_t wgrad_c(const void* a_tok, const void* b_tok, float* part, float* ou
 }
 
 // dW = A^T B over the T tokens of the [T, C] bf16 operands a_tok, b_tok; part holds
-// wgrad_chunks(T, sms) partial [C, C] fp32 planes; out is 16-byte aligned.
+// wgrad_chunks(T, C, sms) partial [C, C] fp32 planes; out is 16-byte aligned.
 cudaError_t wgrad(const void* a_tok, const void* b_tok, float* part, float* out, long long T, int C, int sms,
                   unsigned int* err, cudaStream_t stream) {
   switch (C) {

@@ -40,7 +40,7 @@ cudaError_t project(const void* x, const void* w, void* z, long long T, int C, b
 }  // namespace proj
 namespace bbwd {
 // whtmix_block_bwd.cu: the block backward's weight transposes and weight gradients on the tensor cores
-int wgrad_chunks(long long T, int sms);
+int wgrad_chunks(long long T, int C, int sms);
 cudaError_t transpose2(const void* in0, void* out0, const void* in1, void* out1, int C, cudaStream_t stream);
 cudaError_t wgrad(const void* a_tok, const void* b_tok, float* part, float* out, long long T, int C, int sms,
                   unsigned int* err, cudaStream_t stream);
@@ -997,7 +997,7 @@ int whtmix_block_backward(const void* x, const void* w_in, const void* gains, co
   if (rc != WHTMIX_OK) return rc;
   // slot-1 layout: Z, M, dM [T, C] bf16; the transposed weights [C, C] bf16; the per-chunk partials
   // [chunks, C, C] fp32 of a weight gradient
-  const int chunks = bbwd::wgrad_chunks(T, sms);
+  const int chunks = bbwd::wgrad_chunks(T, static_cast<int>(C), sms);
   size_t off[6], total = 0;
   const size_t sizes[6] = {pb, pb, pb, wb, wb, static_cast<size_t>(chunks) * wgb};
   for (int i = 0; i < 6; ++i) {

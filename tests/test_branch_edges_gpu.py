@@ -110,6 +110,24 @@ def test_wide_projection(T):
     assert (np.abs(got - want) <= tol).all(), float(np.max(np.abs(got - want) / tol))
 
 
+# token counts about a chunk's tiles: a last chunk of one tile, a ragged last tile, more tiles than chunks
+@pytest.mark.parametrize("B,N,C", [(1, 16, 256), (9, 32, 256), (1, 64, 64), (77, 128, 256), (153, 64, 64)])
+def test_weight_gradient_chunks(B, N, C):
+    x, dy = (bf16_dev(inputs.normal(s, B * N * C).reshape(B, N, C).astype(np.float32)) for s in (50, 51))
+    w_in, w_out = (bf16_dev((inputs.normal(s, C * C) / np.sqrt(C)).reshape(C, C).astype(np.float32)) for s in (52, 53))
+    g = torch.ones(N, C, dtype=torch.float32, device="cuda")
+    grads = whtmix.block_backward(x, w_in, g, w_out, dy)
+    whtmix.sync()
+    # under unit gains the mixer is the identity: M = Z = bf16(X W_in^T), dM = bf16(dY W_out), dZ = dM up to a bf16 rounding
+    x64, dy64 = (t.double().cpu().numpy().reshape(-1, C) for t in (x, dy))
+    wi, wo = (t.double().cpu().numpy() for t in (w_in, w_out))
+    for got, a, b, mag in ((grads[1], dy64 @ wo, x64, None), (grads[3], dy64, x64 @ wi.T, None)):
+        ref = a.T @ b
+        # each recomputed operand is within three bf16 roundings of the exact one
+        bound = 3 * 2.0 ** -8 * (np.abs(a).T @ np.abs(b)) + 1e-6 * np.abs(ref)
+        assert (np.abs(got.double().cpu().numpy() - ref) <= bound).all()
+
+
 def run_padded(B, n, N, C, dtype, backward):
     d = inputs.make_inputs(B, N, C, dtype, seed=n + N, n_valid=n, with_dy=backward)
     x, g = to_dev(d["x"], dtype)[:, :n].contiguous(), to_dev(d["g"], "f32")
