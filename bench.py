@@ -42,7 +42,7 @@ REASONS = {0x1: "gpu_idle", 0x2: "applications_clocks_setting", 0x4: "sw_power_c
 # The device-code files each kernel family is compiled from: a committed DRAM-traffic figure is
 # used only while the hash of its family's files is unchanged (and only for the kernel it names).
 KERNEL_FAMILY_SOURCES = {
-    "k_forward_fast": ("whtmix_kernels.cuh", "whtmix_fast.cuh", "whtmix_fast_launch.cuh", "whtmix_tri.cuh"),
+    "k_forward_fast": ("whtmix_kernels.cuh", "whtmix_fast.cuh", "whtmix_fast_launch.cuh", "whtmix_tri.cuh", "whtmix_x16.cuh"),
     "k_backward_fast": ("whtmix_kernels.cuh", "whtmix_fast.cuh", "whtmix_fast_launch.cuh", "whtmix_tri.cuh"),
     "k_block_fast": ("whtmix_kernels.cuh", "whtmix_fast.cuh", "whtmix_tri.cuh", "whtmix_block.cuh", "whtmix_block.cu"),
     "k_forward_plane": ("whtmix_kernels.cuh", "whtmix_fast.cuh", "whtmix_plane.cuh", "whtmix_plane.cu"),

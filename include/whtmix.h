@@ -216,8 +216,8 @@ WHTMIX_API int whtmix_block_forward(const void *x, const void *w_in, const void 
  * dM and dZ are rounded to bf16 (activation gradients); the weight gradients run on the tensor
  * cores in fp32 and are summed over token chunks in a fixed order, so every output is the same bit
  * for bit run to run.  dtype must be WHTMIX_BF16; C 64, 128 or 256.  B = 0 sets the three gain and
- * weight gradients to zero.  About fifteen launches on `stream`; the intermediates live in a second
- * library-managed workspace of the stream. */
+ * weight gradients to zero.  Ten launches on `stream`; the intermediates live in a second library-managed
+ * workspace of the stream. */
 WHTMIX_API int whtmix_block_backward(const void *x, const void *w_in, const void *gains, const void *w_out,
                                      const void *dy, void *dx, void *dw_in, void *dgains, void *dw_out, int64_t B,
                                      int64_t N, int64_t C, int dtype, void *stream);

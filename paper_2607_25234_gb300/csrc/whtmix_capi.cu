@@ -2,9 +2,10 @@
 //
 // Every check runs before anything is enqueued; a failing call enqueues and writes nothing.
 // The plain calls take their workspace from a per-(device, stream) cache; the _ex calls use the
-// caller's buffer.  Each call is one kernel launch for most shapes (five per plane group for planes
+// caller's buffer.  A forward is one kernel launch for most shapes (five per plane group for planes
 // of more than 2^26 elements), with programmatic stream serialisation, plus a stream-ordered
-// allocation the first time a cached workspace grows.
+// allocation the first time a cached workspace grows; log gains' gradients add two, and padding that
+// the kernels do not do themselves one per copy.
 #include <cuda_runtime.h>
 
 #include <cstring>

@@ -8,8 +8,8 @@
 #include <map>
 #include <mutex>
 
-#include "whtmix_fast.cuh"
 #include "whtmix_tri.cuh"
+#include "whtmix_x16.cuh"
 
 namespace whtmix {
 namespace fast {
@@ -42,8 +42,7 @@ inline cudaError_t occupancy_cached(const void* kernel, int threads, size_t smem
 // tcgen05.alloc while the first waits for it at the device-wide barrier.  The grid is one CTA per
 // SM, all resident at once; it is launched with programmatic stream serialisation (launch_pdl),
 // which lets its launch and tensor-memory allocation overlap the previous kernel's tail.
-inline cudaError_t launch_persistent(const void* k, const Params& P, int grid, cudaStream_t stream, int threads = THREADS,
-                                     size_t smem = SMEM_BYTES) {
+inline cudaError_t launch_persistent(const void* k, const Params& P, int grid, cudaStream_t stream, int threads, size_t smem) {
   int occ = 0;
   cudaError_t e = occupancy_cached(k, threads, smem, &occ);
   if (e != cudaSuccess) return e;
@@ -81,13 +80,13 @@ cudaError_t launch_backward(const Params& P, int sms, cudaStream_t stream) {
   return cudaErrorInvalidValue;
 }
 
-// The bf16-exchange forward (whtmix_forward_x16; whtmix_fast.cuh).  Rows of 2^13 elements at every size but 2^21;
+// The bf16-exchange forward (whtmix_forward_x16; whtmix_x16.cuh).  Rows of 2^13 elements at every size but 2^21;
 // 2^23-element planes take 1024-row columns (two lanes per column).  With 152 SMs, 1024 rows of 2^13 spread as 7 or 6
 // per CTA, where 512 rows of 2^14 give 56 CTAs four rows against three; 2^21-element planes take rows of 2^14 and
 // 128-row columns, one column per thread in registers, instead of 256-row columns in tensor memory.
 template <int D, int R, int Q>
 cudaError_t launch_x16_one(const Params& P, int sms, cudaStream_t stream) {
-  return launch_persistent(reinterpret_cast<const void*>(k_forward_fast<D, R, Q, false, WsB16>), P, sms, stream);
+  return launch_persistent(reinterpret_cast<const void*>(x16::k_forward_x16<D, R, Q>), P, sms, stream, x16::THREADS, x16::SMEM_BYTES);
 }
 template <int D>
 cudaError_t launch_forward_x16(const Params& P, int sms, cudaStream_t stream) {

@@ -299,13 +299,12 @@ __device__ __forceinline__ void row_out(float* slot, void* dst, long long e0, in
 
 // ---------------------------------------------------------------------------------------------
 // Columns.
-// Gains of one column: row(j), and rows2(j) = rows j and j + 1 (j even).
+// Gains of one column: rows2(j) = rows j and j + 1 (j even).
 template <int Q>
 struct LaneFull {
   const float* p;
   __device__ __forceinline__ LaneFull(const Params& P, const float*, int col) : p(static_cast<const float*>(P.g) + col) {}
   __device__ __forceinline__ float2 rows2(int j) const { return make_float2(__ldg(p + (j << R)), __ldg(p + ((j + 1) << R))); }
-  __device__ __forceinline__ float row(int j) const { return __ldg(p + (j << R)); }
 };
 // Separable log gains: G[n, c] = et[n] ec[c] from two tables that phase 1 builds (tab); the token table is
 // stored so that a column's rows are consecutive, et[(column >> cb) 2^Q + row].
@@ -316,8 +315,13 @@ struct LaneSep {
   __device__ __forceinline__ LaneSep(const Params& P, const float* tab, int col)
       : p(tab + (static_cast<long long>(col >> P.cbits) << Q)), e(tab[(1ll << (P.m - P.cbits)) + (col & ((1 << P.cbits) - 1))]) {}
   __device__ __forceinline__ float2 rows2(int j) const { return mul2(*reinterpret_cast<const float2*>(p + j), make_float2(e, e)); }
-  __device__ __forceinline__ float row(int j) const { return p[j] * e; }
 };
+
+// The token of entry i of that table.
+template <int Q>
+__device__ __forceinline__ long long sep_token_of(long long i, int cb) {
+  return ((i & ((1ll << Q) - 1)) << (R - cb)) | (i >> Q);
+}
 
 __device__ __forceinline__ void tmem_ld8(uint32_t ta, float (&r)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
@@ -1078,7 +1082,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_forward_fast(Params P) {
     const long long n_t = 1ll << (m - P.cbits), n_tab = n_t + (1ll << P.cbits);
     for (long long i = static_cast<long long>(blockIdx.x) * THREADS + threadIdx.x; i < n_tab;
          i += static_cast<long long>(gridDim.x) * THREADS)
-      tab[i] = expf(i < n_t ? P.gt[fast::sep_token_of<R, Q>(i, P.cbits)] : P.gc[i - n_t]);
+      tab[i] = expf(i < n_t ? P.gt[sep_token_of<Q>(i, P.cbits)] : P.gc[i - n_t]);
   }
   for (long long b0 = 0; b0 < P.B; b0 += P.gp) {
     const int nb = static_cast<int>(min(static_cast<long long>(P.gp), P.B - b0));
