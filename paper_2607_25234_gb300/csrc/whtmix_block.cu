@@ -17,7 +17,7 @@ cudaError_t launch(const Params& P, const void* w_in, const void* w_out, int sms
   const __nv_bfloat16* wi = static_cast<const __nv_bfloat16*>(w_in);
   const __nv_bfloat16* wo = static_cast<const __nv_bfloat16*>(w_out);
   void* args[] = {&p, &wi, &wo};
-  return launch_pdl(k, static_cast<unsigned>(fast::tri_grid(P, sms)), tri::THREADS, tri::BLK_SMEM, stream, args);
+  return launch_pdl(k, static_cast<unsigned>(fast::tri_grid(P.B << (P.m - tri::R), sms)), tri::THREADS, tri::BLK_SMEM, stream, args);
 }
 
 template <int C>

@@ -9,7 +9,8 @@
 // M-major and N-major operands (the channels are contiguous, the contraction runs down the panel's rows), so nothing is
 // transposed; one thread issues tcgen05.mma (kind::f16, M = 128, N = C, K = 16) into a TMEM accumulator per 128 input
 // channels i.  A lane of the accumulator is an i, a column an o, so that a warp stores 32 consecutive floats of the chunk's
-// fp32 partial [C, C] at a time (with the roles swapped, 32 rows at a stride: 16384 tokens of 256 channels 16.9 us, so 11.8); k_wgrad_reduce adds the partials in a fixed order, so dW is the same bit for bit on every run.
+// fp32 partial [C, C] at a time (with the roles swapped, 32 rows at a stride: 16384 tokens of 256 channels 16.9 us, so 11.8);
+// k_wgrad_reduce adds the partials in a fixed order, so dW is the same bit for bit on every run.
 // A chunk is a few tiles (3.4 at 32768 tokens), so its time is the latency of its chain: with 8 x 8 transposes in registers
 // and one tile ahead it took 13.2 us, now 9.0 (32768 tokens, C = 128; whole block_train step [8, 4096, 128] 140 -> 124).
 #include <cuda_bf16.h>

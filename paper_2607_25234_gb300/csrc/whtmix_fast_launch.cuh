@@ -53,9 +53,10 @@ inline cudaError_t launch_persistent(const void* k, const Params& P, int grid, c
 }
 // CTAs of a three-phase launch: one per SM, or one per row of a small batch (at least 64, for the columns): the
 // device-wide barriers wait for fewer arrivals ([1, 4096, 64] bf16, 32 rows: 152 CTAs 9.8 us, 64 8.9, 32 9.4;
-// [1, 2048, 64] 9.4, 8.4, 8.6; [1, 16384, 64], 128 rows: 14.4 with 152, 14.2 with 128).
-inline int tri_grid(const Params& P, int sms) {
-  const long long rows = P.B << (P.m - tri::R), want = rows < 64 ? 64 : rows;
+// [1, 2048, 64] 9.4, 8.4, 8.6; [1, 16384, 64], 128 rows: 14.4 with 152, 14.2 with 128).  The backward's rows are X's
+// and dY's.
+inline int tri_grid(long long rows, int sms) {
+  const long long want = rows < 64 ? 64 : rows;
   return want < sms ? static_cast<int>(want) : sms;
 }
 
@@ -65,7 +66,7 @@ template <int D, bool SEP, int M = 14>
 cudaError_t launch_forward_tri(const Params& P, int sms, cudaStream_t stream) {
   if constexpr (M <= 25) {
     if (P.m != M) return launch_forward_tri<D, SEP, M + 1>(P, sms, stream);
-    return launch_persistent(reinterpret_cast<const void*>(tri::k_forward_fast<D, M - tri::R, SEP>), P, tri_grid(P, sms), stream,
+    return launch_persistent(reinterpret_cast<const void*>(tri::k_forward_fast<D, M - tri::R, SEP>), P, tri_grid(P.B << (M - tri::R), sms), stream,
                              tri::THREADS, tri::smem_bytes<D>());
   }
   return cudaErrorInvalidValue;
@@ -74,7 +75,7 @@ template <int D, int M = 14>
 cudaError_t launch_backward(const Params& P, int sms, cudaStream_t stream) {
   if constexpr (M <= 23) {
     if (P.m != M) return launch_backward<D, M + 1>(P, sms, stream);
-    return launch_persistent(reinterpret_cast<const void*>(tri::k_backward_fast<D, M - tri::R>), P, tri_grid(P, sms), stream,
+    return launch_persistent(reinterpret_cast<const void*>(tri::k_backward_fast<D, M - tri::R>), P, tri_grid(2 * P.B << (M - tri::R), sms), stream,
                              tri::THREADS, tri::smem_bytes<D>());
   }
   return cudaErrorInvalidValue;

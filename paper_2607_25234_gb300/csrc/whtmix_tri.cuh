@@ -27,6 +27,8 @@
 // rows took phase 1 of the 2^23-element plane from 13.5 to 8.7 us.
 #pragma once
 
+#include <type_traits>
+
 #include "whtmix_fast.cuh"
 #include "whtmix_tc.cuh"
 
@@ -435,7 +437,7 @@ enum Mode { FWD, SPECTRUM, ADJOINT };
 // B the warps at the same place of their quarters trade values through shared memory, each then holding all NQ of 16 / NQ
 // row pairs, and trade them back after the gain.  Against units of 2^14 elements in shared memory (8 columns of 1024 or 2048
 // rows, 4 of 4096: 32- and 16-byte row segments, each a whole wavefront of the SM's data path): 2^23 elements 39.6 -> 38.0 us
-// (log gains 37.9 -> 35.5, backward included 148 -> 132), 2^24 116 -> 101, 2^25 526 -> 222 (generic engine: 967).
+// (log gains 37.9 -> 35.5, backward included 148 -> 132), 2^24 116 -> 101, 2^25 526 -> 222 (generic engine: 967), 189 with their groups strided over the CTAs.
 template <int Q>
 struct Lane {
   static constexpr bool TALL = Q >= 10;
@@ -669,24 +671,50 @@ __device__ __forceinline__ void col_lanes(float* ws, int begin, int end, int tot
 }
 
 // Backward columns of up to 256 rows, X and dY of a column in one pass: the spectrum of X waits on chip (in
-// registers up to 32 rows, else in tensor memory) while dY is transformed; the dG term (W X)(W dY)/L goes to X's
-// place in wsx, dY through gain and column bits to its own in wsd.  Against a pass over X that stores its spectrum
-// and a pass over dY that reads it back, the exchange is a third smaller.
+// registers up to 32 rows, else in tensor memory) while dY is transformed; dY goes through gain and column bits to its
+// place in wsd.  Against a pass over X that stores its spectrum and a pass over dY that reads it back, the exchange is a
+// third smaller.
+// The dG terms (W X)(W dY)/L never reach the workspace: a team of pl warps (groups of warps above 64 rows) takes the same
+// 32 columns of pl planes, its terms meet in shared memory, and each warp adds some rows up in ascending b.  What bounds
+// these phases is the exchange through L2: storing the terms and reading them back after a barrier was 8 of a group's 62 us
+// (four planes of 2^21), and the stores part of its 22 us of columns.  Forward and backward, back to back, with terms in
+// the workspace and now: [16, 8192, 256] bf16 375 -> 353 us, [32, 4000 of 4096, 64] f32 log gains 110 -> 104,
+// [256, 512, 64] bf16 94 -> 77, [512, 256, 64] 124 -> 92, [1, 256, 64] 15.3 -> 14.5, [8, 4096, 128] bf16 52.3 -> 52.0.
 template <int Q>
-__device__ __forceinline__ void col_regs_bwd(float* wsx, float* wsd, int cols, const Params& P, uint32_t tmem, float* slots) {
+__device__ __forceinline__ void col_regs_bwd(const float* wsx, float* wsd, int nb, bool first, const Params& P, uint32_t tmem,
+                                             float* slots) {
   constexpr int NR = 1 << Q, NP = NR / 2, m = R + Q;
-  constexpr int PER = 32 * (NR < 4 ? 4 : NR);
-  constexpr int RING = WARP_STAGE / PER > 3 ? 3 : WARP_STAGE / PER;  // blocks in flight: X, dY, X, ... in turn
+  constexpr int NG = NP < 16 ? NP : 16;  // pairs per batch of gains and of dG terms
+  constexpr int PER = 32 * (NR < 4 ? 4 : NR), TERMS = 64 * NG;
+  constexpr int RING = (WARP_STAGE - TERMS) / PER > 3 ? 3 : (WARP_STAGE - TERMS) / PER;  // blocks in flight: X, dY, X, ...
+  static_assert(RING >= 1, "a block and a batch of dG terms");
   const float2 sc = make_float2(P.scale, P.scale);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t ta = tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + 64 * (warp >> 2);
-  const int first = warp * gridDim.x + blockIdx.x, step = gridDim.x * (THREADS / 32), n = cols / 32;
-  float* stg = slots + warp * WARP_STAGE;
-  auto offset = [&](int w) { return (static_cast<long long>((32 * w) >> R) << m) + ((32 * w) & (TILE - 1)); };
-  int sw = first, sd = 0, sslot = 0;  // the next block to stage
+  float *stg = slots + warp * WARP_STAGE, *terms = stg + RING * PER;
+  int pl = 1;  // planes a team of warps holds at a time
+  constexpr int MAXPL = THREADS / 32;
+  while (pl < nb && pl < MAXPL) pl <<= 1;
+  // a team of pl >= NG warps owns at most two rows of a batch per warp and keeps their sums in registers over its sets of pl
+  // planes; among these, the pl with the fewest rounds of the CTA's warps
+  if constexpr (NG < MAXPL) {
+    const int blocks = (TILE / 32 + gridDim.x - 1) / gridDim.x;
+    auto rounds = [&](int p) { return (nb + p - 1) / p * ((blocks * p + MAXPL - 1) / MAXPL); };
+    for (int p = pl / 2; p >= NG; p /= 2)
+      if (rounds(p) < rounds(pl)) pl = p;
+  }
+  const int team = warp / pl, member = warp % pl, teams = MAXPL / pl;
+  auto team_sync = [&] {
+    if (pl > 1) asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(32 * pl) : "memory");
+    else __syncwarp();
+  };
+  const bool direct = first && nb == 1;  // the only terms: stored as they are
+  int gb, ge;  // blocks of 32 columns
+  share(TILE / 32, &gb, &ge);
+  int sg = gb + team, sb = member, sd = 0, sslot = 0;  // the next block to stage
   auto stage = [&] {
-    if (sw < n) {
-      const float* b = (sd ? wsd : wsx) + offset(sw);
+    if (sg < ge && sb < nb) {
+      const float* b = (sd ? wsd : wsx) + (sb << m) + 32 * sg;
       if constexpr (NR >= 4) {
         stage_block<NR>(b, stg + sslot * PER, lane);
       } else {
@@ -696,7 +724,10 @@ __device__ __forceinline__ void col_regs_bwd(float* wsx, float* wsd, int cols, c
     }
     fast::cp_async_commit();
     sslot = sslot + 1 == RING ? 0 : sslot + 1;
-    sw += sd ? step : 0;
+    if (sd) {
+      sb += pl;
+      if (sb >= nb) sb = member, sg += teams;
+    }
     sd ^= 1;
   };
 #pragma unroll
@@ -715,146 +746,284 @@ __device__ __forceinline__ void col_regs_bwd(float* wsx, float* wsd, int cols, c
     for (int j = 0; j < NP; ++j) bf_in(v[j]);
     fast::bfly_all<NP>(v);
   };
-  constexpr int NG = NP < 16 ? NP : 16;  // pairs per batch of gains
-  for (int w = first; w < n; w += step) {
-    const long long o = offset(w) + lane;
-    const LaneFull<Q> gain(P, nullptr, ((32 * w) & (TILE - 1)) + lane);
-    float2 xh[NG];
-    float2 v[NP];
-    take(v);
-    if constexpr (NP > 16) {
-#pragma unroll
-      for (int q = 0; q < NP / 8; ++q) st_pairs<8>(ta + 16 * q, v + 8 * q);
-      fast::tmem_wait_st();
-    } else {
-#pragma unroll
-      for (int j = 0; j < NP; ++j) xh[j] = v[j];
+  // dG at rows h + member, h + member + pl, ... of the batch: the team's terms in ascending b
+  auto add_terms = [&](float (&own)[2], int g, int b, int h) {
+    const int np = min(pl, nb - b);
+    if (NP <= 16 && pl >= NG) {
+      auto keep = [&](auto full) {  // (with the full team's constants 6% faster on large batches)
+        constexpr bool FULL = decltype(full)::value;
+        const int ps = FULL ? MAXPL : pl;
+        const float* t = slots + (FULL ? 0 : team * pl) * WARP_STAGE + RING * PER + lane + 32 * member;
+        for (int p = 0; p < np; ++p) {
+          if (member < 2 * NG) own[0] += t[p * WARP_STAGE];
+          if (member + ps < 2 * NG) own[1] += t[p * WARP_STAGE + 32 * ps];
+        }
+        if (b + ps >= nb) {
+          float* o = static_cast<float*>(P.dg) + 32 * g + lane + ((h + member) << R);
+          if (member < 2 * NG) __stcg(o, own[0]);
+          if (member + ps < 2 * NG) __stcg(o + (ps << R), own[1]);
+        }
+      };
+      if (NG == MAXPL || pl == MAXPL) keep(std::true_type{});
+      else keep(std::false_type{});
+      return;
     }
-    take(v);
+    float* o = static_cast<float*>(P.dg) + 32 * g + lane + (h << R);
+#pragma unroll 1
+    for (int r = member; r < 2 * NG; r += 4 * pl) {
+      float acc[4];
 #pragma unroll
-    for (int h = 0; h < NP; h += NG) {
+      for (int k = 0; k < 4; ++k) acc[k] = (first && b == 0) || r + k * pl >= 2 * NG ? 0.f : __ldcg(o + ((r + k * pl) << R));
+#pragma unroll 1
+      for (int p = 0; p < np; ++p) {
+        const float* t = slots + (team * pl + p) * WARP_STAGE + RING * PER + lane;
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (r + k * pl < 2 * NG) acc[k] += t[32 * (r + k * pl)];
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (r + k * pl < 2 * NG) __stcg(o + ((r + k * pl) << R), acc[k]);
+    }
+  };
+  for (int g = gb + team; g < ge; g += teams) {
+    float own[2];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int r = member + (NG == MAXPL ? MAXPL : pl) * k;
+      own[k] = first || NP > 16 || pl < NG || r >= 2 * NG ? 0.f : __ldcg(static_cast<float*>(P.dg) + 32 * g + lane + (r << R));
+    }
+    for (int b0 = 0; b0 < nb; b0 += pl) {
+      const int b = b0 + member;
+      if (b >= nb) {  // no plane for this warp: only its share of the sums
+#pragma unroll 1
+        for (int h = 0; h < NP; h += NG) {
+          team_sync();
+          team_sync();
+          add_terms(own, g, b0, 2 * h);
+        }
+        continue;
+      }
+      const LaneFull<Q> gain(P, nullptr, 32 * g + lane);
+      float2 xh[NG];
+      float2 v[NP];
+      take(v);
       if constexpr (NP > 16) {
 #pragma unroll
-        for (int q = 0; q < 2; ++q) ld_pairs<8>(ta + 2 * h + 16 * q, xh + 8 * q);
-        fast::tmem_wait_ld();
+        for (int q = 0; q < NP / 8; ++q) st_pairs<8>(ta + 16 * q, v + 8 * q);
+        fast::tmem_wait_st();
+      } else {
+#pragma unroll
+        for (int j = 0; j < NP; ++j) xh[j] = v[j];
       }
-      float2 gg[NG];
+      take(v);
 #pragma unroll
-      for (int j = 0; j < NG; ++j) gg[j] = gain.rows2(2 * (h + j));
+      for (int h = 0; h < NP; h += NG) {
+        if constexpr (NP > 16) {
 #pragma unroll
-      for (int j = 0; j < NG; ++j) {
-        const float2 pr = mul2(mul2(xh[j], v[h + j]), sc);
-        __stcg(wsx + o + ((2 * (h + j)) << R), pr.x);
-        __stcg(wsx + o + ((2 * (h + j) + 1) << R), pr.y);
+          for (int q = 0; q < 2; ++q) ld_pairs<8>(ta + 2 * h + 16 * q, xh + 8 * q);
+          fast::tmem_wait_ld();
+        }
+        float2 gg[NG];
+#pragma unroll
+        for (int j = 0; j < NG; ++j) gg[j] = gain.rows2(2 * (h + j));
+        if (direct) {
+          float* d = static_cast<float*>(P.dg) + 32 * g + lane;
+#pragma unroll
+          for (int j = 0; j < NG; ++j) {
+            const float2 pr = mul2(mul2(xh[j], v[h + j]), sc);
+            __stcg(d + ((2 * (h + j)) << R), pr.x);
+            __stcg(d + ((2 * (h + j) + 1) << R), pr.y);
+          }
+        } else {
+          team_sync();  // the batch before this one has been added up
+#pragma unroll
+          for (int j = 0; j < NG; ++j) {
+            const float2 pr = mul2(mul2(xh[j], v[h + j]), sc);
+            terms[64 * j + lane] = pr.x;
+            terms[64 * j + 32 + lane] = pr.y;
+          }
+        }
+#pragma unroll
+        for (int j = 0; j < NG; ++j) v[h + j] = mul2(v[h + j], mul2(gg[j], sc));
+        if (!direct) {
+          team_sync();
+          add_terms(own, g, b0, 2 * h);
+        }
       }
+      float* o = wsd + (b << m) + 32 * g + lane;
 #pragma unroll
-      for (int j = 0; j < NG; ++j) v[h + j] = mul2(v[h + j], mul2(gg[j], sc));
-    }
+      for (int j = 0; j < NP; ++j) bf_in(v[j]);
+      fast::bfly_all<NP>(v);
 #pragma unroll
-    for (int j = 0; j < NP; ++j) bf_in(v[j]);
-    fast::bfly_all<NP>(v);
-#pragma unroll
-    for (int j = 0; j < NP; ++j) {
-      __stcg(wsd + o + ((2 * j) << R), v[j].x);
-      __stcg(wsd + o + ((2 * j + 1) << R), v[j].y);
+      for (int j = 0; j < NP; ++j) {
+        __stcg(o + ((2 * j) << R), v[j].x);
+        __stcg(o + ((2 * j + 1) << R), v[j].y);
+      }
     }
   }
   asm volatile("cp.async.wait_group 0;" ::: "memory");
 }
 
-// 128 and 256 rows: NB = 2, 4 warps hold 32 columns, one block of 64 rows of X and of dY each.
+// 128 and 256 rows: NB = 2, 4 warps (a group) hold 32 columns of a plane, one block of 64 rows of X and of dY each.  The
+// groups of a team of pl take the same columns of consecutive planes and add their dG terms up as above, eight rows of dG
+// loaded before the team meets (after: their latency cost half the gain; before a pass: its registers spill).
 template <int Q>
-__device__ __forceinline__ void col_lanes_bwd(float* wsx, float* wsd, int begin, int end, const Params& P, uint32_t tmem,
-                                              float* slots) {
+__device__ __forceinline__ void col_lanes_bwd(const float* wsx, float* wsd, int nb, bool first, const Params& P,
+                                              uint32_t tmem, float* slots) {
   constexpr int m = R + Q, NB = 1 << (Q - 6), W = 32 / NB, WP = W / 2, GROUPS = THREADS / 32 / NB;
+  constexpr int STAGED = 64 * 32;  // floats: a block of dY, then the warp's 32 x 32 dG terms of a pass
+  static_assert(STAGED + 32 * 32 <= WARP_STAGE, "a block and its dG terms");
   const float2 sc = make_float2(P.scale, P.scale);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, quarter = warp & 3;
   const int half = (warp >> 2) / NB, i = (warp >> 2) % NB, group = quarter + 4 * half;
   // words of the lane: the spectrum of X, then dY
   const uint32_t tx = tmem + (static_cast<uint32_t>(32 * quarter) << 16) + half * (128 * NB), td = tx + 64 * NB;
-  float* stg = slots + warp * WARP_STAGE;
-  auto offset = [&](int g) { return (static_cast<long long>((32 * g) >> R) << m) + ((32 * g) & (TILE - 1)); };
-  const long long own = static_cast<long long>(64 * i) << R;
-  if (begin + group < end) stage_block<64>(wsd + offset(begin + group) + own, stg, lane);
-  for (int g = begin + group; g < end; g += GROUPS) {
-    const long long o = offset(g) + lane;
-    const LaneFull<Q> gain(P, nullptr, ((32 * g) & (TILE - 1)) + lane);
-    auto rows64 = [&](float2 (&v)[32]) {
+  float *stg = slots + warp * WARP_STAGE, *terms = stg + STAGED;
+  int pl = 1;  // planes a team holds at a time
+  while (pl < nb && pl < GROUPS) pl <<= 1;
+  const int team = group / pl, member = group % pl, teams = GROUPS / pl;
+  auto team_sync = [&] {
+    fast::tmem_wait_st();
+    fast::tmem_fence_before();
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(32 * NB * pl) : "memory");
+    fast::tmem_fence_after();
+  };
+  int gb, ge;  // blocks of 32 columns
+  share(TILE / 32, &gb, &ge);
+  const int own = (64 * i) << R;
+  auto stage = [&](int g, int b) {
+    if (g < ge && b < nb) stage_block<64>(wsd + (b << m) + 32 * g + own, stg, lane);
+  };
+  auto rows64 = [&](float2 (&v)[32]) {
 #pragma unroll
-      for (int j = 0; j < 32; ++j) bf_in(v[j]);
-      bfly32<0>(v);
-    };
-    {
-      float2 v[32];
-      const float* src = wsx + o + own;
+    for (int j = 0; j < 32; ++j) bf_in(v[j]);
+    bfly32<0>(v);
+  };
+  auto across = [&](float2 (&v)[16]) {
 #pragma unroll
-      for (int j = 0; j < 32; ++j) v[j] = make_float2(__ldcg(src + ((2 * j) << R)), __ldcg(src + ((2 * j + 1) << R)));
-      rows64(v);
+    for (int h = WP; h < 16; h <<= 1)
 #pragma unroll
-      for (int q = 0; q < 4; ++q) st_pairs<8>(tx + 64 * i + 16 * q, v + 8 * q);
-      fast::cp_async_wait_all();
-      __syncwarp();
+      for (int k = 0; k < 16; ++k)
+        if ((k & h) == 0) bf2(v[k], v[k + h]);
+  };
+  const int low0 = (64 / NB) * i;
+  // dG at this warp's share of the 32 rows of a pass, eight rows at a time (row r of the terms is row
+  // low + 64 (r / W) + r % W of the column); the first eight are loaded before the team meets
+  const int r0 = member * (32 / pl), r1 = r0 + 32 / pl;
+  const bool direct = first && nb == 1;  // the only terms: stored as they are
+  auto dg_row = [&](int g, int low, int r) { return static_cast<float*>(P.dg) + 32 * g + lane + ((low + 64 * (r / W) + r % W) << R); };
+  auto load_dg = [&](float (&acc)[8], int g, int b, int low, int r) {
 #pragma unroll
-      for (int j = 0; j < 32; ++j) v[j] = make_float2(stg[64 * j + lane], stg[64 * j + 32 + lane]);
-      __syncwarp();
-      if (g + GROUPS < end) stage_block<64>(wsd + offset(g + GROUPS) + own, stg, lane);
-      rows64(v);
-#pragma unroll
-      for (int q = 0; q < 4; ++q) st_pairs<8>(td + 64 * i + 16 * q, v + 8 * q);
-    }
-    const int low0 = (64 / NB) * i;
-    auto across = [&](float2 (&v)[16]) {
-#pragma unroll
-      for (int h = WP; h < 16; h <<= 1)
-#pragma unroll
-        for (int k = 0; k < 16; ++k)
-          if ((k & h) == 0) bf2(v[k], v[k + h]);
-    };
-    float2 gg[16];
-#pragma unroll
-    for (int k = 0; k < 16; ++k) gg[k] = gain.rows2(64 * (k / WP) + low0 + 2 * (k % WP));
-    lane_sync<NB>(group);
+    for (int k = 0; k < 8; ++k) acc[k] = (first && b == 0) || r + k >= r1 ? 0.f : __ldcg(dg_row(g, low, r + (k & 4)) + ((k & 3) << R));
+  };
+  auto add_terms = [&](float (&acc)[8], int g, int b, int low) {
+    const int np = min(pl, nb - b);
 #pragma unroll 1
-    for (int pass = 0; pass < 2; ++pass) {
-      const int low = low0 + W * pass;
-      float2 xh[16], v[16];
+    for (int r = r0;;) {
+      for (int p = 0; p < np; ++p) {
+        const int gr = team * pl + p;
+        const float* t = slots + ((gr & 3) + 4 * ((gr >> 2) * NB + i)) * WARP_STAGE + STAGED + 32 * r + lane;
 #pragma unroll
-      for (int s = 0; s < NB; ++s) ld_pairs<WP>(tx + 64 * s + low, xh + WP * s);
-#pragma unroll
-      for (int s = 0; s < NB; ++s) ld_pairs<WP>(td + 64 * s + low, v + WP * s);
-      fast::tmem_wait_ld();
-      across(xh);
-      across(v);
-      float* xo = wsx + o + (static_cast<long long>(low) << R);
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        const float2 pr = mul2(mul2(xh[k], v[k]), sc);
-        __stcg(xo + ((64 * (k / WP) + 2 * (k % WP)) << R), pr.x);
-        __stcg(xo + ((64 * (k / WP) + 2 * (k % WP) + 1) << R), pr.y);
+        for (int k = 0; k < 8; ++k)
+          if (r + k < r1) acc[k] += t[32 * k];
       }
 #pragma unroll
-      for (int k = 0; k < 16; ++k) v[k] = mul2(v[k], mul2(gg[k], sc));
-      if (pass == 0) {
-#pragma unroll
-        for (int k = 0; k < 16; ++k) gg[k] = gain.rows2(64 * (k / WP) + low0 + W + 2 * (k % WP));
-      }
-      across(v);
-#pragma unroll
-      for (int s = 0; s < NB; ++s) st_pairs<WP>(td + 64 * s + low, v + WP * s);
+      for (int k = 0; k < 8; ++k)
+        if (r + k < r1) __stcg(dg_row(g, low, r + (k & 4)) + ((k & 3) << R), acc[k]);
+      r += 8;
+      if (r >= r1) break;
+      load_dg(acc, g, b, low, r);
     }
-    lane_sync<NB>(group);
-    {
-      float2 v[32];
-      float* dst = wsd + o + own;
-      read_row(td + 64 * i, v);
-      rows64(v);
+  };
+  stage(gb + team, member);
+  for (int g = gb + team; g < ge; g += teams)
+    for (int b0 = 0; b0 < nb; b0 += pl) {
+      const int b = b0 + member;
+      const bool active = b < nb;  // of the whole warp
+      const int o = (b << m) + 32 * g + lane;  // (a group's workspace is below 2^31 elements)
+      const LaneFull<Q> gain(P, nullptr, 32 * g + lane);
+      float2 gg[16];
+      if (active) {
+        float2 v[32];
+        const float* src = wsx + o + own;
 #pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        __stcg(dst + ((2 * j) << R), v[j].x);
-        __stcg(dst + ((2 * j + 1) << R), v[j].y);
+        for (int j = 0; j < 32; ++j) v[j] = make_float2(__ldcg(src + ((2 * j) << R)), __ldcg(src + ((2 * j + 1) << R)));
+        rows64(v);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) st_pairs<8>(tx + 64 * i + 16 * q, v + 8 * q);
+        fast::cp_async_wait_all();
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 32; ++j) v[j] = make_float2(stg[64 * j + lane], stg[64 * j + 32 + lane]);
+        __syncwarp();
+        if (b + pl < nb) stage(g, b + pl);
+        else stage(g + teams, member);
+        rows64(v);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) st_pairs<8>(td + 64 * i + 16 * q, v + 8 * q);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) gg[k] = gain.rows2(64 * (k / WP) + low0 + 2 * (k % WP));
+      }
+      team_sync();
+#pragma unroll 1
+      for (int pass = 0; pass < 2; ++pass) {
+        const int low = low0 + W * pass;
+        if (active) {
+          float2 xh[16], v[16];
+#pragma unroll
+          for (int s = 0; s < NB; ++s) ld_pairs<WP>(tx + 64 * s + low, xh + WP * s);
+#pragma unroll
+          for (int s = 0; s < NB; ++s) ld_pairs<WP>(td + 64 * s + low, v + WP * s);
+          fast::tmem_wait_ld();
+          across(xh);
+          across(v);
+#pragma unroll
+          for (int k = 0; k < 16; ++k) xh[k] = mul2(mul2(xh[k], v[k]), sc);
+          if (direct) {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+              float* d = static_cast<float*>(P.dg) + 32 * g + lane + ((low + 64 * (k / WP) + 2 * (k % WP)) << R);
+              __stcg(d, xh[k].x);
+              __stcg(d + TILE, xh[k].y);
+            }
+          } else {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+              terms[64 * k + lane] = xh[k].x;
+              terms[64 * k + 32 + lane] = xh[k].y;
+            }
+          }
+#pragma unroll
+          for (int k = 0; k < 16; ++k) v[k] = mul2(v[k], mul2(gg[k], sc));
+          if (pass == 0) {
+#pragma unroll
+            for (int k = 0; k < 16; ++k) gg[k] = gain.rows2(64 * (k / WP) + low0 + W + 2 * (k % WP));
+          }
+          across(v);
+#pragma unroll
+          for (int s = 0; s < NB; ++s) st_pairs<WP>(td + 64 * s + low, v + WP * s);
+        }
+        if (direct) continue;
+        float acc[8];
+        load_dg(acc, g, b0, low, r0);
+        team_sync();
+        add_terms(acc, g, b0, low);
+        if (pass == 0) team_sync();  // (the next block's first team_sync is the other one)
+      }
+      if (direct) team_sync();
+      if (active) {
+        float2 v[32];
+        float* dst = wsd + o + own;
+        read_row(td + 64 * i, v);
+        rows64(v);
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+          __stcg(dst + ((2 * j) << R), v[j].x);
+          __stcg(dst + ((2 * j + 1) << R), v[j].y);
+        }
       }
     }
-  }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1023,16 +1192,17 @@ __device__ __forceinline__ void columns(Cta& c, float* ws, int nb, const Params&
   }
 }
 
-// Backward columns of nb planes: the dG terms over wsx, dY through gain and back over wsd.
+// Backward columns of nb planes: dY through gain and back over wsd; dG's terms over wsx or, where sums_dg(Q) (a plane group of
+// taller columns is one or two planes), added to P.dg
+// (which holds the earlier groups' sum unless `first`).
+__host__ __device__ constexpr bool sums_dg(int q) { return q <= 8; }
 template <int Q>
-__device__ __forceinline__ void columns_bwd(Cta& c, float* wsx, float* wsd, int nb, const Params& P) {
+__device__ __forceinline__ void columns_bwd(Cta& c, float* wsx, float* wsd, int nb, bool first, const Params& P) {
   if constexpr (Q <= 6) {
-    col_regs_bwd<Q>(wsx, wsd, nb << R, P, c.tmem, c.slots);
+    col_regs_bwd<Q>(wsx, wsd, nb, first, P, c.tmem, c.slots);
     fast::tmem_fence_before();
   } else if constexpr (Q <= 8) {
-    int gb, ge;
-    share(static_cast<unsigned>(nb) << (R - 5), &gb, &ge);
-    col_lanes_bwd<Q>(wsx, wsd, gb, ge, P, c.tmem, c.slots);
+    col_lanes_bwd<Q>(wsx, wsd, nb, first, P, c.tmem, c.slots);
     fast::tmem_fence_before();
   } else {
     columns<Q, false, SPECTRUM>(c, wsx, nb, P, nullptr);
@@ -1123,10 +1293,10 @@ __global__ void __launch_bounds__(THREADS, 1) k_forward_fast(Params P) {
 // Per group of planes the same three phases over X and dY
 // together,
 //   phase 1  rows of X and dY                                            X, dY -> wsx, wsd
-//   phase 2  columns: the spectrum of X in place, then dY through gain and back, the products
-//            (W X)(W dY)/L replacing the spectrum                        wsx, wsd -> wsx, wsd
-//   phase 3  rows of wsd -> dX; then dG at this CTA's positions: dG (0 for the first group) plus the
-//            group's products in ascending b, so that dG is summed over b = 0, 1, ..., B-1 in that order.
+//   phase 2  columns: the spectrum of X, then dY through gain and back, the terms (W X)(W dY)/L added to dG (0 for
+//            the first group) in ascending b, so that dG is summed over b = 0, 1, ..., B-1 in that order
+//                                                                        wsx, wsd -> wsd, dG
+//   phase 3  rows of wsd -> dX; for columns above 256 rows, whose terms replaced the spectrum in wsx, then dG.
 // dG at plane positions [lb, le) (multiples of 4), NPOS positions of NPL planes loaded at a time: loaded one plane
 // after another the sum was bound by the latency of its loads (14 us instead of 7 for four 8 MiB planes).
 template <int NPOS, int NPL>
@@ -1207,13 +1377,13 @@ __global__ void __launch_bounds__(THREADS, 1) k_backward_fast(Params P) {
           });
     }
     if (!gsync()) break;
-    columns_bwd<Q>(c, wsx, wsd, nb, P);
+    columns_bwd<Q>(c, wsx, wsd, nb, b0 == 0, P);
     if (!gsync()) break;
     int rb, re;
     share(static_cast<unsigned>(rows), &rb, &re);
     rows_out<D>(c, re - rb, wsd + (static_cast<long long>(rb) << R), P.dx,
                 [&](int k, long long* e0, int* lim) { fast::row_loc<R, Q>(b0, rb + k, P.lv, e0, lim); });
-    dg_reduce(static_cast<float*>(P.dg), wsx, m, nb, b0 == 0, lb, le);
+    if constexpr (!sums_dg(Q)) dg_reduce(static_cast<float*>(P.dg), wsx, m, nb, b0 == 0, lb, le);
     if (b0 + P.gp < P.B && !gsync()) break;
   }
   pdl_trigger();

@@ -150,6 +150,17 @@ def run_padded(B, n, N, C, dtype, backward):
     dg.assert_intact("dG")
 
 
+# the backward's dG sums: teams of one warp or group, teams with idle members, full teams over several sets of planes, and
+# a second plane group, for every column height they cover
+@pytest.mark.parametrize("B,n,N,C", [(1, 256, 256, 64), (6, 256, 256, 64), (40, 250, 256, 64), (515, 64, 256, 64), (17, 512, 512, 64),
+                                     (20, 1024, 1024, 64), (33, 2047, 2048, 64), (1, 4096, 4096, 64), (3, 4096, 4096, 64),
+                                     (35, 4000, 4096, 64), (2, 8192, 8192, 64), (17, 100, 8192, 64), (5, 16384, 16384, 64),
+                                     (9, 16384, 16384, 64), (1, 32768, 32768, 64), (7, 30000, 32768, 64)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_gain_gradient_sums(B, n, N, C, dtype):
+    run_padded(B, n, N, C, dtype, backward=True)
+
+
 # one plane a CTA (2^14, 2^15, and 2^16 from its smallest batch): whole, cut inside a 16-byte chunk's row, one token stored;
 # more planes than SMs
 @pytest.mark.parametrize("B,n,N,C", [(1, 256, 256, 64), (3, 249, 256, 64), (2, 1, 512, 64), (3, 1023, 1024, 32), (48, 512, 512, 128),
