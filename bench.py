@@ -56,7 +56,9 @@ def block_fused(w) -> bool:
 
 
 def kernel_name(w) -> str:
-    """The kernel one whtmix_forward call launches for this workload (mirrors the C ABI's dispatch)."""
+    """A stable label of the kernel one whtmix_forward call launches for this workload, kept as recorded with earlier results:
+    rows are 2^13 elements at every size now (the label's 2^14 at 2^21 stays only for the bf16 exchange), and planes of 2^16
+    go one per CTA from a batch of 48."""
     m = (w.N * w.C).bit_length() - 1
     if block_fused(w):
         return f"k_block_fast<bf16, R=13, Q={m - 13}>"
@@ -64,23 +66,27 @@ def kernel_name(w) -> str:
     if (w.dtype in ("f32", "bf16") and 14 <= m <= 16 and (m < 16 or w.B >= 80) and w.gains == "full"
             and not w.block and (not w.padded_io or padded_ok)):
         return f"k_forward_plane<{w.dtype}, column bits {m - 14}> (one plane per CTA, in tensor memory)"
-    if w.dtype in ("f32", "bf16") and 14 <= m <= 23:
+    if w.dtype in ("f32", "bf16") and 14 <= m <= 25:
         r = 14 if m == 21 else 13
         sep = ", separable gains" if w.gains == "separable" else ""
         pad = ", in-kernel token padding" if w.padded_io else ""
         x16 = ", bf16 exchange" if w.exchange == "bf16" else ""
         name = f"k_forward_fast<{w.dtype}, R={r}, Q={m - r}{sep}{pad}{x16}>"
         return f"k_proj<C={w.C}> + {name} + k_proj<C={w.C}>" if w.block else name
+    if w.dtype in ("f32", "bf16") and 10 <= m <= 13:
+        return f"k_forward_small<{w.dtype}, {m}>"
     return "k_forward_s" if m <= 13 else "k_forward_m"
 
 
 def backward_kernel_name(w) -> str:
-    """The kernel one whtmix_backward call launches for this workload (mirrors the C ABI's dispatch);
-    for the block, the mixer backward inside whtmix_block_backward."""
+    """A stable label of the kernel one whtmix_backward call launches for this workload (rows are 2^13 elements at every size
+    now); for the block, the mixer backward inside whtmix_block_backward."""
     m = (w.N * w.C).bit_length() - 1
     if w.dtype in ("f32", "bf16") and 14 <= m <= 23:
         r = 14 if m >= 21 else 13
         return f"k_backward_fast<{w.dtype}, R={r}, Q={m - r}>"
+    if w.dtype in ("f32", "bf16") and 10 <= m <= 13:
+        return f"k_backward_small<{w.dtype}, {m}> + k_small_dg"
     return "k_backward_s" if m <= 13 else "k_backward_m" if m <= 26 else "k_pass_* (five launches per group)"
 
 
@@ -433,10 +439,9 @@ def ours(args, w):
     fwd_block = lib.whtmix_block_forward
     fwd_x16 = lib.whtmix_forward_x16
     bwd_block = lib.whtmix_block_backward
-    # launches of our kernels per step; the block backward: projection, mixer forward, weight
-    # transpose, projection, weight gradient and its reduction, mixer backward, weight gradient
-    # and reduction, weight transpose, projection
-    block_bwd_launches = 11
+    # launches of our kernels per step; the block backward: both weight transposes, projection, mixer forward,
+    # projection, weight gradient and its reduction, mixer backward, weight gradient and reduction, projection
+    block_bwd_launches = 10
     launches_per_step = ((1 if block_fused(w) else 3) + block_bwd_launches if w.block and w.backward else
                          2 if w.backward else 3 if w.block and not block_fused(w) else 1)
     if w.block:

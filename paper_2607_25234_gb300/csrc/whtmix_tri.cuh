@@ -437,7 +437,8 @@ enum Mode { FWD, SPECTRUM, ADJOINT };
 // B the warps at the same place of their quarters trade values through shared memory, each then holding all NQ of 16 / NQ
 // row pairs, and trade them back after the gain.  Against units of 2^14 elements in shared memory (8 columns of 1024 or 2048
 // rows, 4 of 4096: 32- and 16-byte row segments, each a whole wavefront of the SM's data path): 2^23 elements 39.6 -> 38.0 us
-// (log gains 37.9 -> 35.5, backward included 148 -> 132), 2^24 116 -> 101, 2^25 526 -> 222 (generic engine: 967), 189 with their groups strided over the CTAs.
+// (log gains 37.9 -> 35.5, backward included 148 -> 132), 2^24 116 -> 101, 2^25 526 -> 222 (generic engine:
+// 967); with their groups strided over the CTAs 88 and 189.
 template <int Q>
 struct Lane {
   static constexpr bool TALL = Q >= 10;
