@@ -105,7 +105,8 @@ __device__ __forceinline__ void cp_async16(float* smem_dst, const void* gsrc) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gsrc) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+// every copy this thread has issued, committed to a group or not (wait_group 0 passes over those that were not)
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Where row r of the plane group that starts at plane b0 lives in X / Y (planes of lv stored
 // elements, back to back): its first element and how many of its 2^R elements are stored.

@@ -344,7 +344,8 @@ __device__ __forceinline__ void tmem_st4(uint32_t ta, const float (&r)[4]) {
                ::"r"(ta), "f"(r[0]), "f"(r[1]), "f"(r[2]), "f"(r[3]) : "memory");
 }
 
-// Staging of a warp's column blocks: NR rows of 32 columns (128 bytes a row), by the warp's own cp.async.
+// Staging of a warp's column blocks: NR rows of 32 columns (128 bytes a row), by the warp's own cp.async.  No group is
+// committed here: the caller commits and counts groups (col_regs), or waits for every copy (col_lanes: cp_async_wait_all).
 template <int NR>
 __device__ __forceinline__ void stage_block(const float* src32, float* stg, int lane) {  // src32: the block's first column
   const float* s = src32 + (static_cast<long long>(lane >> 3) << R) + 4 * (lane & 7);

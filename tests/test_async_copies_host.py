@@ -1,0 +1,83 @@
+"""Every asynchronous copy of the CUDA sources is waited for, checked on the source text (CPU).
+
+cp.async.wait_group covers committed groups only: a copy that was issued and never committed is not ordered before what follows
+the wait.  So each function or lambda that issues copies commits them, hands them to an mbarrier, or belongs to a function whose
+only wait is cp_async_wait_all, which has to be cp.async.wait_all."""
+import os
+import re
+
+import pytest
+
+from paper_2607_25234_gb300 import build
+
+# helpers that issue copies for a caller that commits them or waits for all
+ISSUERS = ("cp_async16", "cp_async16z", "cp_async16_zfill", "cp_async4", "copy16", "stage_block", "load_x_bf16")
+ISSUE = re.compile(r"\b(?:%s)\s*(?:<\w+>)?\(|cp\.async\.c[ag]\.shared" % "|".join(ISSUERS))
+WAIT_ALL = re.compile(r"cp_async_wait_all\(\)|cp\.async\.wait_all")
+TRACKED = re.compile(r"cp_async_commit\(|cp\.async\.commit_group|cp_async_arrive\(")
+
+
+def without_comments(text):
+    return re.sub(r"//[^\n]*", "", text)
+
+
+def body(text, brace):
+    """The text from the opening brace to its match."""
+    depth = 0
+    for i in range(brace, len(text)):
+        depth += (text[i] == "{") - (text[i] == "}")
+        if depth == 0:
+            return text[brace:i + 1]
+    raise AssertionError("unbalanced braces")
+
+
+def functions(text):
+    """(name, body) of the device functions at namespace level."""
+    text = re.sub(r"__launch_bounds__\((?:[^()]|\([^()]*\))*\)", "", text)
+    for m in re.finditer(r"^[^\n;={}#]*\b(?:__device__|__global__)[^;{}]*?\b(\w+)\([^;{}]*\)[^;{}]*\{", text, re.M):
+        yield m.group(1), body(text, m.end() - 1)
+
+
+def lambdas(text):
+    for m in re.finditer(r"\bauto (\w+) = \[[&=\w, ]*\](?:\([^()]*(?:\([^()]*\)[^()]*)*\))?\s*(?:mutable\s*)?\{", text):
+        yield m.group(1), body(text, m.end() - 1)
+
+
+def sources():
+    return sorted(f for f in os.listdir(build.CSRC) if f.endswith((".cu", ".cuh")))
+
+
+def read(name):
+    with open(os.path.join(build.CSRC, name)) as f:
+        return without_comments(f.read())
+
+
+def test_wait_all_waits_for_uncommitted_copies_too():
+    waits = dict(functions(read("whtmix_fast.cuh")))
+    assert "cp.async.wait_all" in waits["cp_async_wait_all"] and "wait_group" not in waits["cp_async_wait_all"]
+
+
+@pytest.mark.parametrize("name", sources())
+def test_every_copy_is_committed_or_waited_for_with_the_rest(name):
+    for fn, text in functions(read(name)):
+        if fn in ISSUERS or not ISSUE.search(text):
+            continue
+        groups = "cp.async.wait_group" in text
+        rest = text
+        for lam, part in lambdas(text):
+            rest = rest.replace(part, "")
+            if lam not in ISSUERS and ISSUE.search(part):
+                assert TRACKED.search(part) or (not groups and WAIT_ALL.search(text)), f"{name}: {fn}: {lam}"
+        if ISSUE.search(rest):
+            # (a lambda called afterwards may commit them with its own)
+            assert TRACKED.search(text) or (not groups and WAIT_ALL.search(text)), f"{name}: {fn}"
+
+
+def test_the_check_sees_a_missing_commit():
+    kernel = '__device__ void f() { auto stage = [&](int g) { stage_block<64>(g); COMMIT }; stage(0); WAIT }'
+    for commit, wait, ok in (("", 'asm("cp.async.wait_group 0;");', False), ("cp_async_commit();", 'asm("cp.async.wait_group 0;");', True),
+                             ("", "cp_async_wait_all();", True)):
+        (fn, text), = functions(kernel.replace("COMMIT", commit).replace("WAIT", wait))
+        (lam, part), = lambdas(text)
+        assert (fn, lam) == ("f", "stage") and ISSUE.search(part)
+        assert bool(TRACKED.search(part) or ("cp.async.wait_group" not in text and WAIT_ALL.search(text))) == ok

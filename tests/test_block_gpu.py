@@ -130,8 +130,10 @@ def rounds_z(N, C):
     return not (C == 128 and 21 <= m <= 23)
 
 
-# every kind of column pass of the fused kernel below 2^20 elements, both channel counts, and one shape of three launches
-@pytest.mark.parametrize("B,N,C", [(2, 64, 128), (1, 1024, 128), (3, 2048, 64), (1, 4096, 64), (2, 8192, 64), (8, 4096, 128)])
+# every kind of column pass of the fused kernel, both channel counts, with and without the rounding, and one shape of three launches
+@pytest.mark.parametrize("B,N,C", [(2, 64, 128), (1, 1024, 128), (3, 2048, 64), (1, 4096, 64), (2, 8192, 64), (8, 4096, 128),
+                                   (3, 8192, 128), (1, 16384, 64), (2, 16384, 128), (1, 65536, 64), (1, 1 << 17, 64),
+                                   (1, 65536, 128)])
 def test_block_forward_rounds_z_where_its_backward_does(B, N, C):
     """Z's rounding made visible.  Integers: Z = 384 + r with |r| < 64, so that an odd Z rounds to an even one; gains that
     make the mixer M[e] = Z[e] - Z[e ^ s] (G the transform of delta_0 - delta_s, 0 or 2), an integer of at most 128, which bf16
