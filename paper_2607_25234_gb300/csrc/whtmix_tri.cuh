@@ -513,6 +513,7 @@ __device__ __forceinline__ void col_lanes(float* ws, int begin, int end, int tot
   const int first = NQ > 1 ? static_cast<int>(blockIdx.x) * C::GROUPS + group : begin + group;
   const int step = NQ > 1 ? static_cast<int>(gridDim.x) * C::GROUPS : C::GROUPS;
   if constexpr (NQ > 1) end = total;
+  fast::tmem_fence_after();  // with the fence before the device-wide barrier: other warps read rows out of these words
   if (first < end) stage(first);
   for (int g = first; g < end; g += step) {
     const GainT gain(P, tab, first_col(g) + lcol);
@@ -734,6 +735,7 @@ __device__ __forceinline__ void col_regs_bwd(const float* wsx, float* wsd, int n
     }
     sd ^= 1;
   };
+  if constexpr (NP > 16) fast::tmem_fence_after();  // as in col_lanes
 #pragma unroll
   for (int k = 0; k < RING; ++k) stage();
   int slot = 0;
@@ -940,6 +942,7 @@ __device__ __forceinline__ void col_lanes_bwd(const float* wsx, float* wsd, int 
       load_dg(acc, g, b, low, r);
     }
   };
+  fast::tmem_fence_after();  // as in col_lanes
   stage(gb + team, member);
   for (int g = gb + team; g < ge; g += teams)
     for (int b0 = 0; b0 < nb; b0 += pl) {

@@ -1,8 +1,11 @@
-"""Every asynchronous copy of the CUDA sources is waited for, checked on the source text (CPU).
+"""Orderings that a run rarely shows to be missing, checked on the text of the CUDA sources (CPU).
 
-cp.async.wait_group covers committed groups only: a copy that was issued and never committed is not ordered before what follows
+Asynchronous copies: cp.async.wait_group covers committed groups only: a copy that was issued and never committed is not ordered before what follows
 the wait.  So each function or lambda that issues copies commits them, hands them to an mbarrier, or belongs to a function whose
-only wait is cp_async_wait_all, which has to be cp.async.wait_all."""
+only wait is cp_async_wait_all, which has to be cp.async.wait_all.
+
+Tensor memory: a column pass follows a device-wide barrier, before which other warps read and multiplied into the words it
+stores to.  tcgen05.fence::before_thread_sync stands before the barrier, so the pass opens with ::after_thread_sync."""
 import os
 import re
 
@@ -81,3 +84,24 @@ def test_the_check_sees_a_missing_commit():
         (lam, part), = lambdas(text)
         assert (fn, lam) == ("f", "stage") and ISSUE.search(part)
         assert bool(TRACKED.search(part) or ("cp.async.wait_group" not in text and WAIT_ALL.search(text))) == ok
+
+
+@pytest.mark.parametrize("name", ["col_lanes", "col_regs_bwd", "col_lanes_bwd"])
+def test_column_passes_open_with_the_tensor_memory_fence(name):
+    text = dict(functions(read("whtmix_tri.cuh")))[name]
+    stores = [m.start() for m in re.finditer(r"\bst_pairs<", text)]
+    assert stores, "a pass through tensor memory"
+    # the first statement loop over columns comes after the fence, whatever lambdas are defined before it
+    loop = re.search(r"\n  for \(int g = ", text).start()
+    assert loop < stores[0]
+    opening = text[:loop]
+    for _, part in lambdas(opening):
+        opening = opening.replace(part, "")
+    assert "tmem_fence_after()" in opening
+
+
+def test_every_phase_that_touches_tensor_memory_ends_with_the_fence():
+    fns = dict(functions(read("whtmix_tri.cuh")))
+    assert fns["rows_in"].count("tmem_fence_before()") == 2  # each product's, and the end of the bf16 rows
+    for name, calls in (("columns", 1), ("columns_bwd", 2)):
+        assert fns[name].count("tmem_fence_before()") == calls, name
