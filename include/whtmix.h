@@ -173,8 +173,8 @@ WHTMIX_API int whtmix_backward_padded(const void *x, const void *gains, const vo
  * G = fp32(expf(g_t[n]) * expf(g_c[c])), token padding included (N_valid as there; N_valid = N for
  * none).  dtype is WHTMIX_F32 or WHTMIX_BF16 (WHTMIX_I32 returns WHTMIX_ERR_BAD_DTYPE).  x, y, dy,
  * dx: 16-byte aligned; g_t, g_c, dg_t, dg_c: 4-byte aligned; device memory owned by the caller.
- * Forward: for the planes the three-phase kernel covers (2^14 <= N*C <= 2^25) with 2 <= C <= 2^13,
- * the gains are computed inside the kernel from two small tables of exp values
+ * Forward: for the planes the three-phase kernel covers (2^14 <= N*C <= 2^25) with 2 <= C <= 2^13
+ * (2^14 for N*C = 2^21), the gains are computed inside the kernel from two small tables of exp values
  * and G never exists in memory; other shapes build G in the library workspace first.
  * Backward: dx as whtmix_backward_padded with that G; dg_t[n] = sum_c dG[n, c] G[n, c] and
  * dg_c[c] = sum_n dG[n, c] G[n, c] with dG = sum_b (W X_b) o (W dY_b) (the chain rule through

@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(THREADS, 1) k_block_fast(Params P, const __nv_
     fast::tmem_fence_before();
     if (!gsync()) break;
     // phase 2
-    columns<Q, false, FWD>(c, ws, nb, P, nullptr);
+    columns<Q, FULL, FWD>(c, ws, nb, P, nullptr);
     fast::tmem_fence_before();
     if (!gsync()) break;
     // phase 3 (as rows_out up to the row in registers)

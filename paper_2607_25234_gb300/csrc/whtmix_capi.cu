@@ -484,8 +484,11 @@ SepPlan sep_plan(int m, int cbits) {
   return p;
 }
 
+// The log-gain forward computes its gains in the kernel where a row of 2^13 elements holds whole tokens, and at 2^21 elements for
+// C = 2^14 too, two rows a token: the kernel before this one had rows of 2^14 there (G built in the workspace instead, [1, 128,
+// 16384]: 22.4 us f32, 23.0 bf16, in the kernel 16.1 and 16.0).
 bool use_fast_separable(int dtype, int m, int cbits) {
-  return use_fast_forward(dtype, m) && cbits >= 1 && cbits <= 13;
+  return use_fast_forward(dtype, m) && cbits >= 1 && (cbits <= 13 || (m == fast::WIDE_M && cbits == fast::WIDE_CBITS));
 }
 
 // Zero padding / crop on the token axis for the shapes the fast kernels do not pad themselves:

@@ -60,14 +60,19 @@ inline int tri_grid(long long rows, int sms) {
   return want < sms ? static_cast<int>(want) : sms;
 }
 
-// The three-phase kernels (whtmix_tri.cuh) of a 2^m-element plane: 2^(m-13) rows of 2^13.  SEP: separable log gains
-// (P.gt, P.gc) instead of G; needs 1 <= P.cbits <= 13.
-template <int D, bool SEP, int M = 14>
+// The three-phase kernels (whtmix_tri.cuh) of a 2^m-element plane: 2^(m-13) rows of 2^13.  LOG: log gains (P.gt, P.gc) instead of G,
+// whose channels lie within a row, 1 <= P.cbits <= 13; at 2^21 elements also C = 2^14, whose tokens are two rows each
+// (WIDE_M, WIDE_CBITS; measured at use_fast_separable).
+constexpr int WIDE_M = 21, WIDE_CBITS = 14;
+template <int D, tri::Gains G, int M = 14>
 cudaError_t launch_forward_tri(const Params& P, int sms, cudaStream_t stream) {
   if constexpr (M <= 25) {
-    if (P.m != M) return launch_forward_tri<D, SEP, M + 1>(P, sms, stream);
-    return launch_persistent(reinterpret_cast<const void*>(tri::k_forward_fast<D, M - tri::R, SEP>), P, tri_grid(P.B << (M - tri::R), sms), stream,
-                             tri::THREADS, tri::smem_bytes<D>());
+    if (P.m != M) return launch_forward_tri<D, G, M + 1>(P, sms, stream);
+    const void* k = reinterpret_cast<const void*>(tri::k_forward_fast<D, M - tri::R, G>);
+    if constexpr (G == tri::LOG && M == WIDE_M) {
+      if (P.cbits == WIDE_CBITS) k = reinterpret_cast<const void*>(tri::k_forward_fast<D, M - tri::R, tri::LOG_WIDE>);
+    }
+    return launch_persistent(k, P, tri_grid(P.B << (M - tri::R), sms), stream, tri::THREADS, tri::smem_bytes<D>());
   }
   return cudaErrorInvalidValue;
 }

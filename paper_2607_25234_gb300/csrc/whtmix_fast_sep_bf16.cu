@@ -4,6 +4,6 @@
 
 namespace whtmix {
 namespace fast {
-cudaError_t forward_sep_bf16(const Params& P, int sms, cudaStream_t stream) { return launch_forward_tri<DT_BF16, true>(P, sms, stream); }
+cudaError_t forward_sep_bf16(const Params& P, int sms, cudaStream_t stream) { return launch_forward_tri<DT_BF16, tri::LOG>(P, sms, stream); }
 }  // namespace fast
 }  // namespace whtmix

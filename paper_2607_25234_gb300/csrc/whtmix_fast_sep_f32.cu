@@ -4,6 +4,6 @@
 
 namespace whtmix {
 namespace fast {
-cudaError_t forward_sep_f32(const Params& P, int sms, cudaStream_t stream) { return launch_forward_tri<DT_F32, true>(P, sms, stream); }
+cudaError_t forward_sep_f32(const Params& P, int sms, cudaStream_t stream) { return launch_forward_tri<DT_F32, tri::LOG>(P, sms, stream); }
 }  // namespace fast
 }  // namespace whtmix

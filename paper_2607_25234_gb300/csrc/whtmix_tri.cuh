@@ -319,10 +319,25 @@ struct LaneSep {
   __device__ __forceinline__ float2 rows2(int j) const { return mul2(*reinterpret_cast<const float2*>(p + j), make_float2(e, e)); }
 };
 
-// The token of entry i of that table.
+// C = 2^14, two rows a token: rows j and j + 1 are one token's two halves of the channels, et[j / 2] (ec[col], ec[2^13 + col]), and
+// the token table is in natural order.
 template <int Q>
+struct LaneSepWide {
+  const float* p;
+  float2 e;
+  __device__ __forceinline__ LaneSepWide(const Params& P, const float* tab, int col)
+      : p(tab), e(make_float2(tab[(1 << (Q - 1)) + col], tab[(1 << (Q - 1)) + TILE + col])) {}
+  __device__ __forceinline__ float2 rows2(int j) const { return mul2(make_float2(p[j >> 1], p[j >> 1]), e); }
+};
+enum Gains { FULL, LOG, LOG_WIDE };
+template <int Q, Gains G> struct LaneGain { using T = LaneFull<Q>; };
+template <int Q> struct LaneGain<Q, LOG> { using T = LaneSep<Q>; };
+template <int Q> struct LaneGain<Q, LOG_WIDE> { using T = LaneSepWide<Q>; };
+
+// The token of entry i of the table.
+template <int Q, Gains G>
 __device__ __forceinline__ long long sep_token_of(long long i, int cb) {
-  return ((i & ((1ll << Q) - 1)) << (R - cb)) | (i >> Q);
+  return G == LOG_WIDE ? i : ((i & ((1ll << Q) - 1)) << (R - cb)) | (i >> Q);
 }
 
 __device__ __forceinline__ void tmem_ld8(uint32_t ta, float (&r)[8]) {
@@ -1186,10 +1201,10 @@ __device__ __forceinline__ void rows_out(Cta& c, int n, const float* wsr, void* 
 }
 
 // Column bits of nb planes of a workspace, all CTAs together.
-template <int Q, bool SEP, Mode MODE>
+template <int Q, Gains G, Mode MODE>
 __device__ __forceinline__ void columns(Cta& c, float* ws, int nb, const Params& P, const float* tab, const float* xws = nullptr,
                                         float* terms = nullptr) {
-  using LaneT = typename std::conditional<SEP, LaneSep<Q>, LaneFull<Q>>::type;
+  using LaneT = typename LaneGain<Q, G>::T;
   if constexpr (Q <= 6) {
     col_regs<Q, LaneT>(ws, nb << R, P, tab, c.slots);
   } else {
@@ -1216,8 +1231,8 @@ __device__ __forceinline__ void columns_bwd(Cta& c, float* wsx, float* wsd, int 
     col_lanes_bwd<Q>(wsx, wsd, nb, first, P, c.tmem, c.slots);
     fast::tmem_fence_before();
   } else {
-    columns<Q, false, SPECTRUM>(c, wsx, nb, P, nullptr);
-    columns<Q, false, ADJOINT>(c, wsd, nb, P, nullptr, wsx, dg_is_terms(nb, first) ? static_cast<float*>(P.dg) : wsx);
+    columns<Q, FULL, SPECTRUM>(c, wsx, nb, P, nullptr);
+    columns<Q, FULL, ADJOINT>(c, wsd, nb, P, nullptr, wsx, dg_is_terms(nb, first) ? static_cast<float*>(P.dg) : wsx);
   }
 }
 
@@ -1241,7 +1256,7 @@ __host__ __device__ constexpr bool prefetches_gains(int q) { return q <= 10; }
 
 // ---------------------------------------------------------------------------------------------
 // Forward kernel: persistent grid (one CTA per SM, all resident), plane groups of P.gp planes.
-template <int D, int Q, bool SEP>
+template <int D, int Q, Gains G>
 __global__ void __launch_bounds__(THREADS, 1) k_forward_fast(Params P) {
   extern __shared__ __align__(1024) unsigned char tri_smem[];
   __shared__ CtaShared sh;
@@ -1259,11 +1274,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_forward_fast(Params P) {
   pdl_wait();
   GridSync gsync(P.bar, &sh.flag);
   const GainPrefetch prefetch(P.g, m);
-  if constexpr (SEP) {  // the gain tables, part of the first phase 1
+  if constexpr (G != FULL) {  // the gain tables, part of the first phase 1
     const long long n_t = 1ll << (m - P.cbits), n_tab = n_t + (1ll << P.cbits);
     for (long long i = static_cast<long long>(blockIdx.x) * THREADS + threadIdx.x; i < n_tab;
          i += static_cast<long long>(gridDim.x) * THREADS)
-      tab[i] = expf(i < n_t ? P.gt[sep_token_of<Q>(i, P.cbits)] : P.gc[i - n_t]);
+      tab[i] = expf(i < n_t ? P.gt[sep_token_of<Q, G>(i, P.cbits)] : P.gc[i - n_t]);
   }
   for (long long b0 = 0; b0 < P.B; b0 += P.gp) {
     const int nb = static_cast<int>(min(static_cast<long long>(P.gp), P.B - b0));
@@ -1280,11 +1295,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_forward_fast(Params P) {
         },
         [&](int k) { return ws + (static_cast<long long>(rb + k) << R); },
         [&](int k) {
-          if (!SEP && prefetches_gains(Q) && b0 == 0) prefetch(k, n);
+          if (G == FULL && prefetches_gains(Q) && b0 == 0) prefetch(k, n);
         });
     if (!gsync()) break;
     // phase 2: columns
-    columns<Q, SEP, FWD>(c, ws, nb, P, tab);
+    columns<Q, G, FWD>(c, ws, nb, P, tab);
     if (!gsync()) break;
     // phase 3: workspace -> Y, row bits
     rows_out<D>(c, n, ws + (static_cast<long long>(rb) << R), P.y,

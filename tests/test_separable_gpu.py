@@ -1,8 +1,8 @@
 """GPU parity of the separable log-gain entry points (Section III-B, Eq. 2-3) against the fp64
 oracle: G[n, c] = exp(g_t[n]) exp(g_c[c]).
 
-The forward runs the fast kernel with the gains computed inside it (planes of 2^14..2^23 elements,
-2 <= C <= the kernel's row length) or, for every other shape, builds G in the workspace and runs
+The forward runs the fast kernel with the gains computed inside it (planes of 2^14..2^25 elements,
+2 <= C <= 2^13, and 2^14 at 2^21) or, for every other shape, builds G in the workspace and runs
 the full-gain kernels; both are covered below.  Acceptance as in the other parity
 tests (_checks.py): fp32 relative L2 <= 1e-6 per plane with an element-wise 1e-5 bound, bf16
 relative L2 <= 1e-2 per plane with the element-wise bound of one rounding to nearest even.  The
@@ -11,6 +11,8 @@ exactly and dG, G and the sums are fp32 / float64), so they take the float32 bou
 term scaled by the reference's RMS (they are sums over C or N products, not of unit scale).  Every
 output sits between guard regions that must come back untouched.
 """
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -140,3 +142,38 @@ def test_separable_autograd_function():
     check(x.grad, dx_ref, "f32", "autograd dX")
     check(gt.grad, dgt_ref, "f32", "autograd dg_t", per_plane=False)
     check(gc.grad, dgc_ref, "f32", "autograd dg_c", per_plane=False)
+
+
+def kernel_nodes(call) -> int:
+    """How many kernels `call` launches on the current stream, counted in a capture of it."""
+    cu = ctypes.CDLL("libcuda.so.1")
+    s, graph, n = torch.cuda.Stream(), ctypes.c_void_p(), ctypes.c_size_t(0)
+    s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        call()  # the stream's workspace
+        torch.cuda.synchronize()
+        assert cu.cuStreamBeginCapture_v2(ctypes.c_void_p(s.cuda_stream), 2) == 0  # (relaxed mode)
+        call()
+        assert cu.cuStreamEndCapture(ctypes.c_void_p(s.cuda_stream), ctypes.byref(graph)) == 0
+    assert cu.cuGraphGetNodes(graph, None, ctypes.byref(n)) == 0
+    assert cu.cuGraphDestroy(graph) == 0
+    return n.value
+
+
+# C = 2^13, the last whose tokens share a row; C = 2^14 with two rows a token, whole, padded (inside the kernel) and in several
+# planes; the same width beside 2^21, where G is built first
+@pytest.mark.parametrize("B,n,N,C,kernels", [(1, 256, 256, 1 << 13, 1), (1, 128, 128, 1 << 14, 1), (3, 77, 128, 1 << 14, 1),
+                                             (9, 128, 128, 1 << 14, 1), (2, 64, 64, 1 << 14, 2)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_wide_log_gains_are_computed_in_the_kernel(B, n, N, C, kernels, dtype):
+    d = inputs.make_inputs(B, N, C, dtype, seed=N + C, n_valid=n)
+    g_t, g_c = inputs.make_log_gains(N, C, seed=9)
+    x = to_dev(d["x"], dtype)[:, :n].contiguous()
+    gt, gc = torch.from_numpy(g_t).cuda(), torch.from_numpy(g_c).cuda()
+    y = Guarded(x.shape, x.dtype)
+    whtmix.forward_separable(x, gt, gc, out=y.t)
+    whtmix.sync()
+    y.assert_intact("Y")
+    ref = oracle.forward_separable(inputs.as_float64(d["x"], dtype), g_t.astype(np.float64), g_c.astype(np.float64))
+    check(y.t, ref[:, :n], dtype, f"separable Y [{B},{n} of {N},{C}] {dtype}")
+    assert kernel_nodes(lambda: whtmix.forward_separable(x, gt, gc, out=y.t)) == kernels
