@@ -373,39 +373,44 @@ __global__ void k_sep_gains(float* G, const float* gt, const float* gc, int m, i
 // dg_c[c] = sum over n of dG[n, c] G[n, c].  These sums run over up to 2^30 products with cancellation, so they
 // accumulate in float64 (the products of two floats are exact there), in a fixed order, and round once.
 //
-// One pass over dG and G.  A warp holds 32 channels (block cb) and the tokens of one chunk, 32 x 32 values at a
-// time: lane = channel adds them down the tokens as they are loaded, lane = token adds them along the channels out
-// of shared memory, so each value costs two float64 multiply-adds and no shuffles (float64 runs at a sixty-fourth
-// of the float32 rate here).  part_t[cb][n] (dg_t itself where one block holds every channel) and part_c[chunk][c] are
-// added up by k_sep_final.  Against one pass per gradient and a serial sum over 1024 chunks per channel:
-// [32, 4000 of 4096, 64] f32, forward and backward: 188 -> 115 us with both kernels.
+// One pass over dG and G.  A CTA holds 32 channels (block cb) and the tokens of one chunk; its warps (one per SM sub-partition) take
+// U tokens at a time in turn, U x 32 values: lane = channel adds them down the tokens as they are loaded; then 32 / U lanes a token
+// add them along the channels out of shared memory.  part_t[cb][n] (dg_t itself where one block holds every channel) and
+// part_c[chunk][c] are added up by k_sep_final.
+// What bounds it: float64.  A sub-partition takes some 170 cycles for a warp's float64 operation, a lone warp twice that, so
+// that 32 x 32 values (64 of them in a chain) take 13 us however few there are.  With U = 8, 18 operations for 8 x 32 values,
+// small calls end sooner; U = 32 has the fewest operations for large ones (SepPlan).  Against one pass per gradient and a
+// serial sum over 1024 chunks per channel: [32, 4000 of 4096, 64] f32, forward and backward: 188 -> 105 us with both kernels.
 constexpr int SEP_RED_WARPS = 4;
+template <int U>
 __global__ void __launch_bounds__(32 * SEP_RED_WARPS) k_sep_reduce(double* part_t, float* dgt, double* part_c, const float* dG,
                                                                    const float* G, int m, int cbits, int nchunks, long long per_chunk) {
-  __shared__ float sd[SEP_RED_WARPS][32][33], sg[SEP_RED_WARPS][32][33];
+  __shared__ float sd[SEP_RED_WARPS][U][33], sg[SEP_RED_WARPS][U][33];
+  __shared__ double sum[SEP_RED_WARPS][32];
+  constexpr int H = U < 16 ? U : 16, PARTS = 32 / U;  // rows loaded at a time; lanes a token
   const long long N = 1ll << (m - cbits), C = 1ll << cbits;
   const int ncb = static_cast<int>((C + 31) / 32), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int token = lane / PARTS, first = lane % PARTS * U;  // for the sums along the channels
   float(*d)[33] = sd[warp];
   float(*g)[33] = sg[warp];
-  for (long long w = static_cast<long long>(blockIdx.x) * SEP_RED_WARPS + warp; w < static_cast<long long>(ncb) * nchunks;
-       w += static_cast<long long>(gridDim.x) * SEP_RED_WARPS) {
+  for (long long w = blockIdx.x; w < static_cast<long long>(ncb) * nchunks; w += gridDim.x) {
     const int cb = static_cast<int>(w % ncb);
     const long long k = w / ncb, c = 32ll * cb + lane, n_end = min(N, (k + 1) * per_chunk);
     double acc_c = 0.0;
-    for (long long n0 = k * per_chunk; n0 < n_end; n0 += 32) {
-      const int rows = static_cast<int>(min(32ll, n_end - n0));
+    for (long long n0 = k * per_chunk + U * warp; n0 < n_end; n0 += U * SEP_RED_WARPS) {
+      const int rows = static_cast<int>(min(static_cast<long long>(U), n_end - n0));
       const float *pd = dG + (n0 << cbits) + c, *pg = G + (n0 << cbits) + c;
 #pragma unroll
-      for (int h = 0; h < 32; h += 16) {
-        float a[16], b[16];
+      for (int h = 0; h < U; h += H) {
+        float a[H], b[H];
 #pragma unroll
-        for (int r = 0; r < 16; ++r) {
+        for (int r = 0; r < H; ++r) {
           const bool in = c < C && h + r < rows;
           a[r] = in ? __ldcg(pd + (static_cast<long long>(h + r) << cbits)) : 0.f;
           b[r] = in ? __ldcg(pg + (static_cast<long long>(h + r) << cbits)) : 0.f;
         }
 #pragma unroll
-        for (int r = 0; r < 16; ++r) {
+        for (int r = 0; r < H; ++r) {
           d[h + r][lane] = a[r];
           g[h + r][lane] = b[r];
           acc_c += static_cast<double>(a[r]) * static_cast<double>(b[r]);
@@ -414,14 +419,23 @@ __global__ void __launch_bounds__(32 * SEP_RED_WARPS) k_sep_reduce(double* part_
       __syncwarp();
       double acc_t = 0.0;
 #pragma unroll 8
-      for (int j = 0; j < 32; ++j) acc_t += static_cast<double>(d[lane][j]) * static_cast<double>(g[lane][j]);
-      if (lane < rows) {
-        if (ncb == 1) dgt[n0 + lane] = static_cast<float>(acc_t);
-        else part_t[static_cast<long long>(cb) * N + n0 + lane] = acc_t;
+      for (int j = 0; j < U; ++j) acc_t += static_cast<double>(d[token][first + j]) * static_cast<double>(g[token][first + j]);
+#pragma unroll
+      for (int o = 1; o < PARTS; o <<= 1) acc_t += __shfl_xor_sync(0xffffffffu, acc_t, o);
+      if (lane % PARTS == 0 && token < rows) {
+        if (ncb == 1) dgt[n0 + token] = static_cast<float>(acc_t);
+        else part_t[static_cast<long long>(cb) * N + n0 + token] = acc_t;
       }
       __syncwarp();
     }
-    if (c < C) part_c[k * C + c] = acc_c;
+    sum[warp][lane] = acc_c;
+    __syncthreads();
+    if (warp == 0 && c < C) {
+#pragma unroll
+      for (int r = 1; r < SEP_RED_WARPS; ++r) acc_c += sum[r][lane];
+      part_c[k * C + c] = acc_c;
+    }
+    __syncthreads();
   }
 }
 // Blocks [0, t_blocks): dg_t, a token a thread.  The others: dg_c, 32 channels a block, eight runs of consecutive chunks
@@ -464,20 +478,26 @@ unsigned grid_for(long long work, int sms) {
   return static_cast<unsigned>(blocks < 1 ? 1 : blocks > cap ? cap : blocks);
 }
 
-// The reduction's token chunks: about two thousand warps over (channel block, chunk) pairs, at most 128 chunks (the
-// final sum runs over them one after another), whole multiples of 32 tokens.
+// The reduction's token chunks: about two CTAs an SM over (channel block, chunk) pairs, at most one an SM for each channel block
+// (k_sep_final's threads add an eighth of the chunks one after another), whole multiples of what the warps of a CTA take at a
+// time.  Eight tokens a warp below 2^10 blocks of 32 x 32 ([1, 4096, 64] backward 21.7 us, with 32 tokens 26.4;
+// [1, 32768, 32] 44.6 and 42.1, [1, 262144, 32] 278 and 248).
 struct SepPlan {
+  int unit;  // U
   int nchunks;
   long long per_chunk;
   size_t t_bytes, c_bytes;  // part_t, part_c
 };
 SepPlan sep_plan(int m, int cbits) {
+  constexpr long long SMS = 152;
   const long long N = 1ll << (m - cbits), C = 1ll << cbits, ncb = (C + 31) / 32;
-  long long want = 2048 / ncb;
-  want = want < 1 ? 1 : want > 128 ? 128 : want;
-  const long long blocks = (N + 31) / 32, per = (blocks + want - 1) / want;
+  long long want = 2 * SMS / ncb;
+  want = want < 1 ? 1 : want > SMS ? SMS : want;
+  const int unit = N * ncb < (1ll << 15) ? 8 : 32;
+  const long long step = unit * SEP_RED_WARPS, blocks = (N + step - 1) / step, per = (blocks + want - 1) / want;
   SepPlan p;
-  p.per_chunk = 32 * per;
+  p.unit = unit;
+  p.per_chunk = step * per;
   p.nchunks = static_cast<int>((blocks + per - 1) / per);
   p.t_bytes = ncb == 1 ? 0 : align256(static_cast<size_t>(ncb * N) * 8);
   p.c_bytes = align256(static_cast<size_t>(p.nchunks * C) * 8);
@@ -776,10 +796,9 @@ int run(const Call& c, void* user_ws, size_t user_ws_bytes, bool use_user_ws, vo
     const SepPlan sp = sep_plan(m, cbits);
     double* part_t = reinterpret_cast<double*>(wsb + lay.part);
     double* part_c = reinterpret_cast<double*>(wsb + lay.part + sp.t_bytes);
-    const long long ncb = (c.C + 31) / 32, warps = ncb * sp.nchunks;
-    const long long blocks = (warps + SEP_RED_WARPS - 1) / SEP_RED_WARPS;
-    k_sep_reduce<<<static_cast<unsigned>(blocks < 6ll * sms ? blocks : 6ll * sms), 32 * SEP_RED_WARPS, 0, stream>>>(
-        part_t, c.dgt, part_c, dG, G, m, cbits, sp.nchunks, sp.per_chunk);
+    const long long ncb = (c.C + 31) / 32, blocks = ncb * sp.nchunks;
+    (sp.unit == 8 ? k_sep_reduce<8> : k_sep_reduce<32>)<<<static_cast<unsigned>(blocks < 6ll * sms ? blocks : 6ll * sms), 32 * SEP_RED_WARPS, 0,
+                                                         stream>>>(part_t, c.dgt, part_c, dG, G, m, cbits, sp.nchunks, sp.per_chunk);
     const unsigned t_blocks = ncb == 1 ? 0 : grid_for(c.N, sms);
     k_sep_final<<<t_blocks + static_cast<unsigned>(ncb), SEP_THREADS, 0, stream>>>(c.dgt, c.dgc, part_t, part_c, m, cbits,
                                                                                   sp.nchunks, t_blocks);

@@ -47,8 +47,11 @@ def test_tall_columns_log_gains(N, C, dtype):
     y.assert_intact("Y")
 
 
-# one and two channel blocks of 32 and a part of one; token counts below, at and past a block of 32 and of a chunk
-@pytest.mark.parametrize("B,n,N,C,dtype", [(3, 5, 8, 4, "f32"), (2, 17, 32, 64, "f32"), (2, 4000, 4096, 32, "f32"),
+# one and two channel blocks of 32 and a part of one; token counts below, at and past a warp's eight, a CTA's 32 and a chunk; the
+# fourth to sixth and the last take 32 tokens a warp
+@pytest.mark.parametrize("B,n,N,C,dtype", [(1, 2, 4, 32, "f32"), (2, 64, 64, 64, "bf16"), (1, 1 << 13, 1 << 13, 8, "f32"),
+                                           (1, (1 << 17) - 4, 1 << 17, 32, "f32"), (1, 1 << 17, 1 << 17, 4, "bf16"),
+                                           (1, 40000, 1 << 16, 64, "f32"), (3, 5, 8, 4, "f32"), (2, 17, 32, 64, "f32"), (2, 4000, 4096, 32, "f32"),
                                            (1, 1 << 14, 1 << 14, 2, "bf16"), (1, 2, 2, 1 << 13, "f32"), (2, 8192, 8192, 256, "bf16")])
 def test_log_gain_gradients_in_one_pass(B, n, N, C, dtype):
     d = inputs.make_inputs(B, N, C, dtype, seed=n + C, n_valid=n, with_dy=True)
