@@ -158,7 +158,8 @@ def run_padded(B, n, N, C, dtype, backward):
 # a second plane group, for every column height they cover
 @pytest.mark.parametrize("B,n,N,C", [(1, 256, 256, 64), (6, 256, 256, 64), (40, 250, 256, 64), (515, 64, 256, 64), (17, 512, 512, 64),
                                      (20, 1024, 1024, 64), (33, 2047, 2048, 64), (1, 4096, 4096, 64), (3, 4096, 4096, 64),
-                                     (35, 4000, 4096, 64), (2, 8192, 8192, 64), (17, 100, 8192, 64), (5, 16384, 16384, 64),
+                                     (35, 4000, 4096, 64), (2, 8192, 8192, 64), (9, 8192, 8192, 64), (12, 8191, 8192, 64), (17, 100, 8192, 64),
+                                     (33, 60, 8192, 64), (5, 16384, 16384, 64),
                                      (9, 16384, 16384, 64), (1, 32768, 32768, 64), (7, 30000, 32768, 64), (1, 65536, 65536, 64),
                                      (3, 60000, 65536, 64), (1, 65536, 65536, 128), (2, 64800, 65536, 128)])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
