@@ -244,8 +244,8 @@ WHTMIX_API int whtmix_last_cuda_error(void);
  * passes through the workspace in one launch (2^13 < N*C <= 2^26), 3 = five passes, one launch
  * each (seven for the backward), through the workspace (2^26 < N*C <= 2^30); 0 for an invalid
  * shape.  (The fp32 / bf16 forward of a 2^14- or 2^15-element plane with full gains, and of a
- * 2^16-element plane in batches of 48 or more, runs one plane per CTA instead, in the SM's tensor
- * memory, without the workspace.) */
+ * 2^16-element plane in batches of 48 or more (bf16; fp32 64), runs one plane per CTA instead, in
+ * the SM's tensor memory, without the workspace.) */
 WHTMIX_API int whtmix_plan(int64_t N, int64_t C);
 
 #ifdef __cplusplus

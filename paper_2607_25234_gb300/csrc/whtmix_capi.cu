@@ -56,12 +56,15 @@ thread_local int g_last_cuda_error = 0;
 
 constexpr size_t HEADER_BYTES = sizeof(GridBarrier);
 constexpr size_t WS_TARGET_BYTES = 64ull << 20;  // plane-group workspace, L2-resident (126 MiB L2)
-constexpr int64_t PLANE_MIN_BATCH_16 = 48;
 // Smallest batch for which the one-plane-per-CTA forward beats the three-phase kernel: a plane of 2^16 elements takes a CTA the
-// same 15 us whether one or all SMs have one, where the three-phase kernel spreads a small batch over every SM (measured on
-// [B, 512, 128] bf16, back to back: B = 40 three-phase 14.7 us against 15.2, B = 64 17.9 against 15.2).  2^14 and 2^15
-// planes take less than the three-phase kernel's phases and barriers.
-int64_t plane_kernel_min_batch(int m) { return m == 16 ? PLANE_MIN_BATCH_16 : 1; }
+// same time whether one or all SMs have one, where the three-phase kernel spreads a small batch over every SM.  Measured on
+// [B, 512, 128], back to back, three-phase against this: bf16 B = 44 14.9 us and 15.1, 48 15.4 and 15.1, 64 18.0 and 15.2; f32, whose
+// rows go through registers on both sides, B = 48 16.4 and 20.1, 60 19.7 and 20.3, 64 20.4 and 20.2, 72 22.0 and 20.7.  2^14 and
+// 2^15 planes take less than the three-phase kernel's phases and barriers.
+constexpr int64_t PLANE_MIN_BATCH_16_BF16 = 48, PLANE_MIN_BATCH_16_F32 = 64;
+int64_t plane_kernel_min_batch(int m, int dtype) {
+  return m < 16 ? 1 : dtype == WHTMIX_BF16 ? PLANE_MIN_BATCH_16_BF16 : PLANE_MIN_BATCH_16_F32;
+}
 
 int cuda_fail(cudaError_t e) {
   g_last_cuda_error = static_cast<int>(e);
@@ -700,7 +703,7 @@ int run(const Call& c, void* user_ws, size_t user_ws_bytes, bool use_user_ws, vo
   // Planes of 2^14 .. 2^16 elements: one plane per CTA, the fp32 intermediate in the SM's tensor
   // memory, no workspace and no device-wide barrier.
   if (!c.backward && !c.separable && !c.w_in && c.dtype != WHTMIX_I32 && m >= 14 && m <= 16 &&
-      c.B >= plane_kernel_min_batch(m) && (lv == L || (lv * es) % 16 == 0) &&
+      c.B >= plane_kernel_min_batch(m, c.dtype) && (lv == L || (lv * es) % 16 == 0) &&
       c.B <= 0x7fffffff) {  // one CTA per plane: B fits a grid
     int dev = 0, sms = 0;
     rc = device_check(&dev, &sms);

@@ -167,10 +167,11 @@ def test_gain_gradient_sums(B, n, N, C, dtype):
     run_padded(B, n, N, C, dtype, backward=True)
 
 
-# one plane a CTA (2^14, 2^15, and 2^16 from its smallest batch): whole, cut inside a 16-byte chunk's row, one token stored;
+# one plane a CTA (2^14, 2^15, and 2^16 from its smallest batch, 48 for bf16 and 64 for f32, and the three-phase kernel below): whole, cut inside a 16-byte chunk's row, one token stored;
 # more planes than SMs
 @pytest.mark.parametrize("B,n,N,C", [(1, 256, 256, 64), (3, 249, 256, 64), (2, 1, 512, 64), (3, 1023, 1024, 32), (48, 512, 512, 128),
-                                     (49, 333, 512, 128), (310, 128, 128, 128), (160, 500, 512, 64)])
+                                     (49, 333, 512, 128),
+                                     (63, 512, 512, 128), (64, 500, 512, 128), (310, 128, 128, 128), (160, 500, 512, 64)])
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 def test_plane_in_tensor_memory(B, n, N, C, dtype):
     run_padded(B, n, N, C, dtype, False)
