@@ -115,21 +115,23 @@ def test_wide_projection(T):
 
 
 # token counts about a chunk's tiles: a last chunk of one tile, a ragged last tile, more tiles than chunks
-@pytest.mark.parametrize("B,N,C", [(1, 16, 256), (9, 32, 256), (1, 64, 64), (77, 128, 256), (153, 64, 64)])
+@pytest.mark.parametrize("B,N,C", [(1, 16, 256), (9, 32, 256), (1, 64, 64), (3, 32, 128), (77, 128, 256), (153, 64, 64), (160, 128, 128)])
 def test_weight_gradient_chunks(B, N, C):
-    x, dy = (bf16_dev(inputs.normal(s, B * N * C).reshape(B, N, C).astype(np.float32)) for s in (50, 51))
-    w_in, w_out = (bf16_dev((inputs.normal(s, C * C) / np.sqrt(C)).reshape(C, C).astype(np.float32)) for s in (52, 53))
+    """Bit for bit, so that no tile of tokens can be lost, doubled or taken from a neighbour: integer X and dY, projections that permute
+    the channels and flip signs, unit gains.  Then Z, M = Z, dM and dZ = dM are small integers (the fp32 transforms are exact, their
+    values integers below 2^24 over a power of two), and the weight gradients are sums of integers below 2^24."""
+    x, dy = (inputs.small_ints(s + C, B * N * C, -2, 2).reshape(B, N, C).astype(np.float32) for s in (50, 51))
+    w_in, w_out = (np.zeros((C, C), dtype=np.float32) for _ in range(2))
+    for s, w in ((52, w_in), (53, w_out)):
+        w[np.arange(C), np.argsort(inputs.normal(s + C, C))] = 2.0 * inputs.small_ints(s + 2 * C, C, 0, 1) - 1.0
     g = torch.ones(N, C, dtype=torch.float32, device="cuda")
-    grads = whtmix.block_backward(x, w_in, g, w_out, dy)
+    dx, dw_in, _, dw_out = whtmix.block_backward(bf16_dev(x), bf16_dev(w_in), g, bf16_dev(w_out), bf16_dev(dy))
     whtmix.sync()
-    # under unit gains the mixer is the identity: M = Z = bf16(X W_in^T), dM = bf16(dY W_out), dZ = dM up to a bf16 rounding
-    x64, dy64 = (t.double().cpu().numpy().reshape(-1, C) for t in (x, dy))
-    wi, wo = (t.double().cpu().numpy() for t in (w_in, w_out))
-    for got, a, b, mag in ((grads[1], dy64 @ wo, x64, None), (grads[3], dy64, x64 @ wi.T, None)):
-        ref = a.T @ b
-        # each recomputed operand is within three bf16 roundings of the exact one
-        bound = 3 * 2.0 ** -8 * (np.abs(a).T @ np.abs(b)) + 1e-6 * np.abs(ref)
-        assert (np.abs(got.double().cpu().numpy() - ref) <= bound).all()
+    x64, dy64, wi, wo = (a.astype(np.float64).reshape(-1, C) for a in (x, dy, w_in, w_out))
+    dz = dy64 @ wo
+    for name, got, want in (("dX", dx, dz @ wi), ("dW_in", dw_in, dz.T @ x64), ("dW_out", dw_out, dy64.T @ (x64 @ wi.T))):
+        got = got.double().cpu().numpy().reshape(want.shape)
+        assert np.array_equal(got, want), f"{name}: {int((got != want).sum())} of {want.size} differ"
 
 
 def run_padded(B, n, N, C, dtype, backward):
