@@ -10,7 +10,7 @@
 // stores it.  Both operands are K-major (X rows are tokens with their channels contiguous, W rows
 // are output channels with their input channels contiguous), laid out in shared memory as the
 // tensor core's no-swizzle canonical form: 8-row x 16-byte core matrices, the K-adjacent core
-// matrix 128 bytes on, the next group of 8 rows (C / 8) x 128 bytes on.  bf16 output takes
+// matrix 128 bytes on, the next group of 8 rows (C / 8) x 128 bytes on.  This is the fp32 output; bf16 output takes
 // other kernels below: the pipelined, warp-specialised k_proj_pipe (TMA in and out) at C = 64 and 128, k_proj_wide at 256.
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -29,10 +29,10 @@ constexpr size_t SMEM_MIN = 120 * 1024;  // more than half an SM: one CTA per SM
 
 using namespace tc;
 
-// C in {64, 128, 256}; OUT_F32: fp32 output (else bf16, round to nearest even).
-template <int C, bool OUT_F32>
-__global__ void __launch_bounds__(THREADS, 1) k_proj(const __nv_bfloat16* x, const __nv_bfloat16* __restrict__ w,
-                                                     void* z, long long T, unsigned int* err) {  // z may be x
+// C in {64, 128, 256}, fp32 output.
+template <int C>
+__global__ void __launch_bounds__(THREADS, 1) k_proj(const __nv_bfloat16* __restrict__ x, const __nv_bfloat16* __restrict__ w,
+                                                     float* __restrict__ z, long long T, unsigned int* err) {
   static_assert(C == 64 || C == 128 || C == 256, "channels");
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ uint64_t mbar;
@@ -102,21 +102,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_proj(const __nv_bfloat16* x, con
       tmem_ld16(tmem + lane_base + c0, v);
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
       if (t < T) {
-        if constexpr (OUT_F32) {
-          float4* o = reinterpret_cast<float4*>(static_cast<float*>(z) + t * C + c0);
+        float4* o = reinterpret_cast<float4*>(z + t * C + c0);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-        } else {
-          uint32_t h[8];
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            __nv_bfloat162 b = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
-            h[q] = *reinterpret_cast<uint32_t*>(&b);
-          }
-          uint4* o = reinterpret_cast<uint4*>(static_cast<__nv_bfloat16*>(z) + t * C + c0);
-          o[0] = make_uint4(h[0], h[1], h[2], h[3]);
-          o[1] = make_uint4(h[4], h[5], h[6], h[7]);
-        }
+        for (int q = 0; q < 4; ++q) o[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
       }
     }
     // every thread's TMEM reads are done before the next tile's MMAs overwrite the accumulator,
@@ -440,16 +428,17 @@ cudaError_t launch_pipe(const void* x, const void* w, void* z, long long T, unsi
   return cudaGetLastError();
 }
 
-template <int C, bool OUT_F32>
+template <int C>
 cudaError_t launch_c(const void* x, const void* w, void* z, long long T, unsigned int* err, int sms, cudaStream_t s) {
   const size_t need = static_cast<size_t>(C) * C * 2 + static_cast<size_t>(TILE_T) * C * 2;
   const size_t smem = need > SMEM_MIN ? need : SMEM_MIN;
-  auto k = k_proj<C, OUT_F32>;
+  auto k = k_proj<C>;
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   if (e != cudaSuccess) return e;
   const long long ntiles = (T + TILE_T - 1) / TILE_T;
   const unsigned grid = static_cast<unsigned>(ntiles < sms ? ntiles : sms);
-  k<<<grid, THREADS, smem, s>>>(static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(w), z, T, err);
+  k<<<grid, THREADS, smem, s>>>(static_cast<const __nv_bfloat16*>(x), static_cast<const __nv_bfloat16*>(w),
+                                static_cast<float*>(z), T, err);
   return cudaGetLastError();
 }
 
@@ -463,18 +452,14 @@ cudaError_t launch_wide(const void* x, const void* w, void* z, long long T, unsi
   return launch_pdl(reinterpret_cast<const void*>(k_proj_wide), static_cast<unsigned>(ntiles < sms ? ntiles : sms), PW_THREADS, PW_SMEM, s, args);
 }
 
-// Z = X W^T for T tokens of C channels (C = 64, 128 or 256); err: device word set on a timeout.
+// Z = X W^T for T tokens of C channels (C = 64, 128 or 256), all three 16-byte aligned; err: device word set on a timeout.
 cudaError_t project(const void* x, const void* w, void* z, long long T, int C, bool out_f32, unsigned int* err, int sms,
                     cudaStream_t s) {
   if (T <= 0) return cudaSuccess;
-  // bf16 output at C = 64, 128: the pipelined kernel (its TMA tensor maps need 16-byte aligned bases)
-  const bool aligned = ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(w) | reinterpret_cast<uintptr_t>(z)) & 15u) == 0;
-  if (!out_f32 && aligned && C == 64) return launch_pipe<64>(x, w, z, T, err, sms, s);
-  if (!out_f32 && aligned && C == 128) return launch_pipe<128>(x, w, z, T, err, sms, s);
   switch (C) {
-    case 64: return out_f32 ? launch_c<64, true>(x, w, z, T, err, sms, s) : launch_c<64, false>(x, w, z, T, err, sms, s);
-    case 128: return out_f32 ? launch_c<128, true>(x, w, z, T, err, sms, s) : launch_c<128, false>(x, w, z, T, err, sms, s);
-    case 256: return out_f32 ? launch_c<256, true>(x, w, z, T, err, sms, s) : launch_wide(x, w, z, T, err, sms, s);
+    case 64: return out_f32 ? launch_c<64>(x, w, z, T, err, sms, s) : launch_pipe<64>(x, w, z, T, err, sms, s);
+    case 128: return out_f32 ? launch_c<128>(x, w, z, T, err, sms, s) : launch_pipe<128>(x, w, z, T, err, sms, s);
+    case 256: return out_f32 ? launch_c<256>(x, w, z, T, err, sms, s) : launch_wide(x, w, z, T, err, sms, s);
     default: return cudaErrorInvalidValue;
   }
 }
