@@ -1328,8 +1328,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_forward_fast(Params P) {
 //            the first group) in ascending b, so that dG is summed over b = 0, 1, ..., B-1 in that order
 //                                                                        wsx, wsd -> wsd, dG
 //   phase 3  rows of wsd -> dX; for columns above 256 rows whose terms replaced the spectrum in wsx, then dG.
-// dG at plane positions [lb, le) (multiples of 4), NPOS positions of NPL planes loaded at a time: loaded one plane
-// after another the sum was bound by the latency of its loads (14 us instead of 7 for four 8 MiB planes).
+// dG at plane positions [lb, le) (multiples of 4), NPOS positions of NPL planes loaded at a time (four loads in flight a thread:
+// eight made the phases around it spill registers).  A plane group of these columns is one or two planes ([4, 65536, 64] bf16
+// backward 162 -> 152 us against four planes' loads at a position, two of them always off).
 template <int NPOS, int NPL>
 __device__ __forceinline__ void dg_sum(float* dg, const float* wsx, int m, int nb, bool first, long long lb, long long le) {
   for (long long l0 = lb + 4 * threadIdx.x; l0 < le; l0 += 4 * THREADS * NPOS) {
@@ -1365,10 +1366,9 @@ __device__ __forceinline__ void dg_sum(float* dg, const float* wsx, int m, int n
     }
   }
 }
-// (four loads in flight a thread: eight made the phases around it spill registers)
 __device__ __forceinline__ void dg_reduce(float* dg, const float* wsx, int m, int nb, bool first, long long lb, long long le) {
   if (nb == 1) dg_sum<4, 1>(dg, wsx, m, nb, first, lb, le);
-  else dg_sum<1, 4>(dg, wsx, m, nb, first, lb, le);
+  else dg_sum<2, 2>(dg, wsx, m, nb, first, lb, le);
 }
 template <int D, int Q>
 __global__ void __launch_bounds__(THREADS, 1) k_backward_fast(Params P) {
