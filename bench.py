@@ -22,6 +22,7 @@ import argparse
 import hashlib
 import json
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -39,14 +40,33 @@ FALLBACK_HBM_GBS = 6800.0
 REASONS = {0x1: "gpu_idle", 0x2: "applications_clocks_setting", 0x4: "sw_power_cap", 0x8: "hw_slowdown",
            0x10: "sync_boost", 0x20: "sw_thermal_slowdown", 0x40: "hw_thermal_slowdown",
            0x80: "hw_power_brake_slowdown", 0x100: "display_clock_setting"}
-# The device-code files each kernel family is compiled from: a committed DRAM-traffic figure is
-# used only while the hash of its family's files is unchanged (and only for the kernel it names).
-KERNEL_FAMILY_SOURCES = {
-    "k_forward_fast": ("whtmix_kernels.cuh", "whtmix_fast.cuh", "whtmix_fast_launch.cuh", "whtmix_tri.cuh", "whtmix_x16.cuh"),
-    "k_backward_fast": ("whtmix_kernels.cuh", "whtmix_fast.cuh", "whtmix_fast_launch.cuh", "whtmix_tri.cuh"),
-    "k_block_fast": ("whtmix_kernels.cuh", "whtmix_fast.cuh", "whtmix_tri.cuh", "whtmix_block.cuh", "whtmix_block.cu"),
-    "k_forward_plane": ("whtmix_kernels.cuh", "whtmix_fast.cuh", "whtmix_plane.cuh", "whtmix_plane.cu"),
+# The translation units each kernel family is compiled in: a committed DRAM-traffic figure is used only
+# while the hash of its family's units and of everything they include is unchanged (and only for the
+# kernel it names).
+KERNEL_FAMILY_UNITS = {
+    "k_forward_fast": ("whtmix_fast_f32.cu", "whtmix_fast_bf16.cu", "whtmix_fast_sep_f32.cu", "whtmix_fast_sep_bf16.cu"),
+    "k_forward_x16": ("whtmix_fast_x16.cu",),
+    "k_backward_fast": ("whtmix_fast_f32.cu", "whtmix_fast_bf16.cu"),
+    "k_block_fast": ("whtmix_block.cu",),
+    "k_forward_plane": ("whtmix_plane.cu",),
+    "k_forward_small": ("whtmix_small.cu",),
+    "k_backward_small": ("whtmix_small.cu",),
 }
+CSRC = os.path.join(ROOT, "paper_2607_25234_gb300", "csrc")
+
+
+def kernel_family_sources(family: str) -> list[str]:
+    """The files of csrc/ the family's kernels are compiled from: its units and their includes, theirs included."""
+    todo, seen = list(KERNEL_FAMILY_UNITS[family]), set()
+    while todo:
+        f = todo.pop()
+        if f in seen:
+            continue
+        seen.add(f)
+        with open(os.path.join(CSRC, f)) as src:
+            included = re.findall(r'^#include "([^"]+)"', src.read(), re.M)
+        todo += [i for i in included if os.path.exists(os.path.join(CSRC, i))]
+    return sorted(seen)
 
 
 def block_fused(w) -> bool:
@@ -92,14 +112,13 @@ def backward_kernel_name(w) -> str:
 
 def kernel_source_hash(kernel: str) -> str:
     """Hash of the source files of the kernel family `kernel` belongs to ("" if unknown)."""
-    family = next((f for f in KERNEL_FAMILY_SOURCES if kernel.startswith(f)), None)
+    family = next((f for f in KERNEL_FAMILY_UNITS if kernel.startswith(f)), None)
     if family is None:
         return ""
     h = hashlib.sha256()
-    for f in sorted(KERNEL_FAMILY_SOURCES[family]):
-        path = os.path.join(ROOT, "paper_2607_25234_gb300", "csrc", f)
-        if os.path.exists(path):
-            h.update(open(path, "rb").read())
+    for f in kernel_family_sources(family):
+        with open(os.path.join(CSRC, f), "rb") as src:
+            h.update(src.read())
     return h.hexdigest()[:16]
 
 

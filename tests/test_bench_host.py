@@ -4,6 +4,7 @@ turning null when the kernel it was measured on changes), the whole-job value an
 Expected values are worked out by hand from the shapes, independently of the bench's own formulas."""
 import json
 import os
+import shutil
 
 import pytest
 
@@ -39,6 +40,23 @@ def test_kernel_each_workload_launches():
     # 2^16-element planes go one per CTA only from a batch of 80
     small = inputs.Workload("x", 79, 512, 128, "bf16")
     assert bench.kernel_name(small).startswith("k_forward_fast<bf16, R=13, Q=3>")
+
+
+def test_traffic_hash_covers_what_a_kernel_is_compiled_from(monkeypatch, tmp_path):
+    assert {"whtmix_plane.cu", "whtmix_plane.cuh", "whtmix_tri.cuh", "whtmix_tc.cuh", "whtmix_fast.cuh", "whtmix_kernels.cuh"} <= \
+        set(bench.kernel_family_sources("k_forward_plane"))
+    assert {"whtmix_block.cuh", "whtmix_tri.cuh", "whtmix_tc.cuh", "whtmix_fast_launch.cuh"} <= set(bench.kernel_family_sources("k_block_fast"))
+    for family in bench.KERNEL_FAMILY_UNITS:
+        # an edit to any of the files, the last of the includes among them, changes the hash
+        before = bench.kernel_source_hash(family)
+        for name in bench.kernel_family_sources(family):
+            copy = tmp_path / family / name
+            shutil.copytree(bench.CSRC, copy)
+            with open(copy / name, "a") as f:
+                f.write("// edited\n")
+            with monkeypatch.context() as m:
+                m.setattr(bench, "CSRC", str(copy))
+                assert bench.kernel_source_hash(family) != before, (family, name)
 
 
 def test_alu_floor_counts_the_butterfly_adds():
