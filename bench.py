@@ -76,38 +76,37 @@ def block_fused(w) -> bool:
 
 
 def kernel_name(w) -> str:
-    """A stable label of the kernel one whtmix_forward call launches for this workload, kept as recorded with earlier results:
-    rows are 2^13 elements at every size now (the label's 2^14 at 2^21 stays only for the bf16 exchange), and planes of 2^16
-    go one per CTA from a batch of 48."""
+    """The kernel one whtmix_forward call launches for this workload (mirrors the C ABI's dispatch).  Rows are 2^13
+    elements, 2^14 in the bf16 exchange's kernel at 2^21."""
     m = (w.N * w.C).bit_length() - 1
     if block_fused(w):
         return f"k_block_fast<bf16, R=13, Q={m - 13}>"
     padded_ok = w.n_valid is None or (w.n_valid * w.C * (2 if w.dtype == "bf16" else 4)) % 16 == 0
-    if (w.dtype in ("f32", "bf16") and 14 <= m <= 16 and (m < 16 or w.B >= 80) and w.gains == "full"
-            and not w.block and (not w.padded_io or padded_ok)):
+    if (w.dtype in ("f32", "bf16") and 14 <= m <= 16 and (m < 16 or w.B >= (48 if w.dtype == "bf16" else 64))
+            and w.gains == "full" and not w.block and (not w.padded_io or padded_ok)):
         return f"k_forward_plane<{w.dtype}, column bits {m - 14}> (one plane per CTA, in tensor memory)"
     if w.dtype in ("f32", "bf16") and 14 <= m <= 25:
-        r = 14 if m == 21 else 13
+        if w.exchange == "bf16" and m <= 23:
+            r = 14 if m == 21 else 13
+            return f"k_forward_x16<{w.dtype}, R={r}, Q={m - r}>"
         sep = ", separable gains" if w.gains == "separable" else ""
         pad = ", in-kernel token padding" if w.padded_io else ""
-        x16 = ", bf16 exchange" if w.exchange == "bf16" else ""
-        name = f"k_forward_fast<{w.dtype}, R={r}, Q={m - r}{sep}{pad}{x16}>"
+        name = f"k_forward_fast<{w.dtype}, R=13, Q={m - 13}{sep}{pad}>"
         return f"k_proj<C={w.C}> + {name} + k_proj<C={w.C}>" if w.block else name
     if w.dtype in ("f32", "bf16") and 10 <= m <= 13:
         return f"k_forward_small<{w.dtype}, {m}>"
-    return "k_forward_s" if m <= 13 else "k_forward_m"
+    return "k_forward_s" if m <= 13 else "k_forward_m" if m <= 26 else "k_pass_* (five launches per group)"
 
 
 def backward_kernel_name(w) -> str:
-    """A stable label of the kernel one whtmix_backward call launches for this workload (rows are 2^13 elements at every size
-    now); for the block, the mixer backward inside whtmix_block_backward."""
+    """The kernel one whtmix_backward call launches for this workload (mirrors the C ABI's dispatch);
+    for the block, the mixer backward inside whtmix_block_backward."""
     m = (w.N * w.C).bit_length() - 1
     if w.dtype in ("f32", "bf16") and 14 <= m <= 23:
-        r = 14 if m >= 21 else 13
-        return f"k_backward_fast<{w.dtype}, R={r}, Q={m - r}>"
+        return f"k_backward_fast<{w.dtype}, R=13, Q={m - 13}>"
     if w.dtype in ("f32", "bf16") and 10 <= m <= 13:
         return f"k_backward_small<{w.dtype}, {m}> + k_small_dg"
-    return "k_backward_s" if m <= 13 else "k_backward_m" if m <= 26 else "k_pass_* (five launches per group)"
+    return "k_backward_s" if m <= 13 else "k_backward_m" if m <= 26 else "k_pass_* (seven launches per group)"
 
 
 def kernel_source_hash(kernel: str) -> str:

@@ -4,6 +4,7 @@ turning null when the kernel it was measured on changes), the whole-job value an
 Expected values are worked out by hand from the shapes, independently of the bench's own formulas."""
 import json
 import os
+import re
 import shutil
 
 import pytest
@@ -34,12 +35,25 @@ def test_kernel_each_workload_launches():
     assert bench.kernel_name(W["longseq_32x4096x64_f32"]) == "k_forward_fast<f32, R=13, Q=5>"
     assert bench.kernel_name(W["epipolar_128x512x128_bf16"]).startswith("k_forward_plane<bf16, column bits 2>")
     assert bench.kernel_name(W["tiny_1x256x64_f32"]).startswith("k_forward_plane<f32, column bits 0>")
-    assert bench.kernel_name(W["train_16x8192x256_bf16"]) == "k_forward_fast<bf16, R=14, Q=7>"
-    assert bench.backward_kernel_name(W["train_16x8192x256_bf16"]) == "k_backward_fast<bf16, R=14, Q=7>"
-    assert bench.backward_kernel_name(W["fullimage_train_1x65536x128_bf16"]) == "k_backward_fast<bf16, R=14, Q=9>"
-    # 2^16-element planes go one per CTA only from a batch of 80
-    small = inputs.Workload("x", 79, 512, 128, "bf16")
-    assert bench.kernel_name(small).startswith("k_forward_fast<bf16, R=13, Q=3>")
+    assert bench.kernel_name(W["train_16x8192x256_bf16"]) == "k_forward_fast<bf16, R=13, Q=8>"
+    assert bench.backward_kernel_name(W["train_16x8192x256_bf16"]) == "k_backward_fast<bf16, R=13, Q=8>"
+    assert bench.backward_kernel_name(W["fullimage_train_1x65536x128_bf16"]) == "k_backward_fast<bf16, R=13, Q=10>"
+    assert bench.kernel_name(inputs.Workload("x", 1, 1 << 20, 128, "f32")) == "k_pass_* (five launches per group)"
+    assert bench.backward_kernel_name(inputs.Workload("x", 1, 1 << 20, 128, "f32")) == "k_pass_* (seven launches per group)"
+
+
+def test_kernel_names_follow_the_dispatch_of_the_library():
+    """The bounds kernel_name repeats, against the constants the library compiles: 2^16-element planes go one per CTA from a batch that
+    depends on the dtype; the block is fused at C = 64 and 128 from 2^17 to 2^23."""
+    with open(os.path.join(bench.CSRC, "whtmix_capi.cu")) as f:
+        capi = f.read()
+    for dtype, const in (("bf16", "PLANE_MIN_BATCH_16_BF16"), ("f32", "PLANE_MIN_BATCH_16_F32")):
+        first = int(re.search(const + r" = (\d+)", capi).group(1))
+        assert bench.kernel_name(inputs.Workload("x", first - 1, 512, 128, dtype)) == f"k_forward_fast<{dtype}, R=13, Q=3>"
+        assert bench.kernel_name(inputs.Workload("x", first, 512, 128, dtype)).startswith(f"k_forward_plane<{dtype}, column bits 2>")
+    assert "bool use_fused_block(int64_t C, int m) { return (C == 64 || C == 128) && m >= 17 && m <= 23; }" in capi
+    for N, C, fused in ((1 << 10, 128, True), (1 << 9, 128, False), (1 << 17, 64, True), (1 << 17, 128, False), (1 << 13, 256, False)):
+        assert bench.block_fused(inputs.Workload("x", 1, N, C, "bf16", block=True)) == fused
 
 
 def test_traffic_hash_covers_what_a_kernel_is_compiled_from(monkeypatch, tmp_path):
@@ -138,10 +152,11 @@ def test_reference_arm_line_matches_ours_in_config_and_metric(monkeypatch, capsy
 
 
 def test_bf16_exchange_workload():
-    # the same shape, bytes and kernel as the full-image workload, with the exchange marked
+    # the same shape and bytes as the full-image workload, another kernel, with the exchange marked
     w, ref = W["fullimage_x16_1x65536x128_bf16"], W["fullimage_1x65536x128_bf16"]
     assert w.ideal_bytes() == ref.ideal_bytes() == 67_108_864
-    assert bench.kernel_name(w) == "k_forward_fast<bf16, R=13, Q=10, bf16 exchange>"
+    assert bench.kernel_name(w) == "k_forward_x16<bf16, R=13, Q=10>"
+    assert bench.kernel_name(inputs.Workload("x", 1, 32768, 64, "bf16", exchange="bf16")) == "k_forward_x16<bf16, R=14, Q=7>"
     cfg, cfg_ref = bench.workload_config(w, 1, 126 << 20), bench.workload_config(ref, 1, 126 << 20)
     assert cfg["exchange"] == "bf16" and cfg_ref["exchange"] == "f32"
     assert {k: v for k, v in cfg.items() if k not in ("workload", "exchange")} == \
