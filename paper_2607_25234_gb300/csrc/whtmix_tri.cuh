@@ -22,9 +22,15 @@
 // measured without arithmetic: 4.4 us to write it, 5.9 to read and write it by columns, 1.8 to read it back,
 // 1.4 per barrier), and within an SM the shared-memory data path (one 128-byte wavefront a cycle) more than the
 // additions.  Measured against the previous kernel (8 warps, 128 elements a thread, columns read straight from
-// L2): [32, 4096, 64] f32 40.6 -> 32.9 us, [1, 4096, 64] bf16 11.6 -> 9.7, [1, 65536, 128] bf16 41.9 -> 38.0, with
-// log gains 39.2 -> 35.5, [1, 32768, 128] bf16 28.4 -> 27.1, [8, 4096, 256] f32 42.6 -> 36.3; of that the tensor-core
+// L2): [32, 4096, 64] f32 40.6 -> 32.9 us, [1, 4096, 64] bf16 11.6 -> 8.9, [1, 65536, 128] bf16 41.9 -> 38.1, with
+// log gains 39.2 -> 35.4, [1, 32768, 128] bf16 28.4 -> 26.6, [8, 4096, 256] f32 42.6 -> 36.7; of that the tensor-core
 // rows took phase 1 of the 2^23-element plane from 13.5 to 8.7 us.
+//
+// What the tensor cores' additions cost in precision: their fp32 accumulator truncates where an addition rounds.  bf16 outputs hide
+// it.  dG, the one fp32 result of bf16 inputs, against 64 bits, as a multiple of the error of the same values passed as fp32 (whose
+// rows are additions): 0.97 to 1.02 (8e-8 to 1.4e-7) for N(0, 1) activations and gradients, planes of 2^14 to 2^23; 1.5 to 2.0
+// (2.1e-7 to 3.1e-7) where a few values dominate their row, N(0, 1) e^(2 N(0, 1)).  Two accumulators of 64 k each make the latter
+// 1.2 to 1.4, the backward of single small planes 3 to 6% slower; rows by additions 1.0, the training step 349 -> 376 us.
 #pragma once
 
 #include <type_traits>
@@ -698,7 +704,7 @@ __device__ __forceinline__ void col_lanes(float* ws, int begin, int end, int tot
 // 32 columns of pl planes, its terms meet in shared memory, and each warp adds some rows up in ascending b.  What bounds
 // these phases is the exchange through L2: storing the terms and reading them back after a barrier was 8 of a group's 62 us
 // (four planes of 2^21), and the stores part of its 22 us of columns.  Forward and backward, back to back, with terms in
-// the workspace and now: [16, 8192, 256] bf16 375 -> 353 us, [32, 4000 of 4096, 64] f32 log gains 110 -> 104,
+// the workspace and in shared memory: [16, 8192, 256] bf16 375 -> 353 us, [32, 4000 of 4096, 64] f32 log gains 110 -> 104,
 // [256, 512, 64] bf16 94 -> 77, [512, 256, 64] 124 -> 92, [1, 256, 64] 15.3 -> 14.5, [8, 4096, 128] bf16 52.3 -> 52.0.
 template <int Q>
 __device__ __forceinline__ void col_regs_bwd(const float* wsx, float* wsd, int nb, bool first, const Params& P, uint32_t tmem,
@@ -1316,11 +1322,11 @@ __global__ void __launch_bounds__(THREADS, 1) k_forward_fast(Params P) {
 }
 
 // Backward kernel (planes of 2^14 .. 2^23 elements).  Against the previous one (8 warps, one column a thread or two passes
-// through tensor memory, dG summed plane after plane), forward and backward together: [16, 8192, 256] bf16 465 -> 379 us,
-// [8, 4096, 256] bf16 118 -> 91, [1, 65536, 128] bf16 186 -> 132, [4, 16384, 256] bf16 335 -> 243, [32, 1024, 64] bf16
-// 36.3 -> 32.5.  Per group of four 2^21-element planes now: phase 1 18 us, columns 22, rows out 9, dG 7, barriers 5; its
-// workspaces (64 MiB) and the streamed X, dY, dX do not fit L2 together (700 MB of HBM traffic a call against 218 MB),
-// and smaller groups lose more to phases than they save (48 MiB 437 us, 32 MiB 461).
+// through tensor memory, dG summed plane after plane), forward and backward together: [16, 8192, 256] bf16 465 -> 350 us,
+// [8, 4096, 256] bf16 118 -> 90, [1, 65536, 128] bf16 186 -> 124, [4, 16384, 256] bf16 335 -> 219, [32, 1024, 64] bf16
+// 36.3 -> 30.6.  A group's workspaces (64 MiB) and the streamed X, dY, dX do not fit L2 together (531 MB of HBM traffic a call at
+// [16, 8192, 256], 218 MB of them X, dY, dX and the gains); smaller groups lose more to phases and barriers than they save
+// (48 MiB 403 us, 32 MiB 400), and 128 MiB take as long (349).
 // Per group of planes the same three phases over X and dY
 // together,
 //   phase 1  rows of X and dY                                            X, dY -> wsx, wsd
