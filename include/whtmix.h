@@ -141,11 +141,12 @@ WHTMIX_API int whtmix_backward_ex(const void *x, const void *gains, const void *
  * N*C <= 2^22 (4 Mi fp32 elements), else the call returns WHTMIX_ERR_WORKSPACE and enqueues
  * nothing.  B = 0 is a no-op.  The first call on each device looks up the array's device address
  * with a CUDA runtime call; make that first call before any stream capture.  A call enqueues two
- * 8-byte memsets (the barrier's arrival counts; none where the plane stays in one SM's tensor memory) and one kernel.  All calls share the array, which
- * keeps the previous call's contents: calls whose kernels can overlap on the GPU (different
- * streams, or different host threads) race on it -- order them on one stream.  A bounded
- * device-wide wait that gives up sets the array's error word, which stays set (later calls keep
- * it) until whtmix_sync reports it as WHTMIX_ERR_TIMEOUT and clears it. */
+ * 8-byte memsets (the barrier's arrival counts; none where the plane stays in one SM's tensor
+ * memory) and one kernel.  All calls share the array, which keeps the previous call's contents:
+ * calls whose kernels can overlap on the GPU (different streams, or different host threads) race
+ * on it -- order them on one stream.  A bounded device-wide wait that gives up sets the array's
+ * error word, which stays set (later calls keep it) until whtmix_sync reports it as
+ * WHTMIX_ERR_TIMEOUT and clears it. */
 WHTMIX_API int whtmix_forward_noalloc(const void *x, const void *gains, void *y, int64_t B, int64_t N,
                                       int64_t C, int dtype, void *stream);
 
