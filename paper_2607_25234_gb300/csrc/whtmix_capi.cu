@@ -857,7 +857,8 @@ Call separable_call(bool backward, const void* x, const float* gt, const float* 
 }
 
 // The fused block kernel covers 64 and 128 channels and planes of 2^17 to 2^23 elements.  Against three launches (projection,
-// mixer, projection): [1, 1024, 128] 19.9 -> 11.9 us, [8, 4096, 128] 31.3 -> 23.3, [32, 4096, 64] 50.5 -> 34.3.  Smaller planes run one per CTA between the projections.
+// mixer, projection): [1, 1024, 128] 17.8 -> 12.0 us, [16, 4096, 128] 44.8 -> 35.5, [32, 4096, 64] 44.6 -> 33.8, [8, 8192, 128] 47.9 ->
+// 39.4, [1, 131072, 64] 57.7 -> 48.3.  Smaller planes run one per CTA between the projections.
 bool use_fused_block(int64_t C, int m) { return (C == 64 || C == 128) && m >= 17 && m <= 23; }
 
 }  // namespace

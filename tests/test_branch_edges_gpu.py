@@ -83,8 +83,10 @@ def test_fused_block(B, N, C):
     x, g = to_dev(d["x"], "bf16"), to_dev(d["g"], "f32")
     y = Guarded(x.shape, torch.bfloat16)
     whtmix.block_forward(x, bf16_dev(w_in), g, bf16_dev(w_out), out=y.t)
+    three = whtmix.project(whtmix.forward(whtmix.project(x, bf16_dev(w_in)), g), bf16_dev(w_out))
     whtmix.sync()
     y.assert_intact("block Y")
+    assert torch.equal(y.t, three)  # the same sums in the same order, rounded at the same places
     x64, g64 = inputs.as_float64(d["x"], "bf16"), d["g"].astype(np.float64)
     wi, wo = (inputs.as_float64(inputs.f32_to_bf16_bits(w), "bf16") for w in (w_in, w_out))
     m = oracle.forward(bf16_round(x64 @ wi.T), g64)  # Z is rounded at each of these shapes
